@@ -22,7 +22,7 @@ namespace {
 
 thread_local std::string g_create_error = "no error";
 
-constexpr int kGraphChunk = 64;  // steps per captured graph (even: buffers return)
+constexpr int kGraphChunk = 64;  // steps per captured graph (a multiple of 8: buffers return, also by fours)
 
 size_t storage_bytes(int st) {
   switch (st) {
@@ -111,6 +111,7 @@ struct mdf_s {
   long long key_base = 0;   // global index of local node 0 (slabs of a larger lattice)
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // chunk starting from buffer 0 / 1
   void *buf[2] = {nullptr, nullptr};
+  bool fuse = false;     // runs of updates go by fused launches (see mdf_create)
   bool inplace = false;  // one buffer, AA pattern (buf[1] unused)
   int parity = 0;        // AA layout of the current state: 0 even, 1 odd
   void *mac[2] = {nullptr, nullptr};  // node moments of equilibrium-shifted storage
@@ -158,7 +159,11 @@ DevArgs base_args(const mdf_t h) {
   a.block = h->block;
   a.s1 = h->s1; a.s2 = h->s2;
   a.s1f = (float)h->s1; a.s2f = (float)h->s2;
-  for (int b = 0; b < 3; ++b) a.lid_u[b] = h->bc.lid ? h->bc.lid_u[b] : 0.0;
+  for (int b = 0; b < 3; ++b) {
+    a.lid_u[b] = h->bc.lid ? h->bc.lid_u[b] : 0.0;
+    a.wall[b] = h->bc.wall[b];
+  }
+  a.lid = h->bc.lid ? 1 : 0;
   a.min = h->mac[h->cur_index()];
   a.mout = h->mac[1 - h->cur_index()];
   a.partials = h->partials;
@@ -211,6 +216,28 @@ mdf_status one_update(mdf_t h, int mode, const mdf_fields_t *out) {
   return MDF_OK;
 }
 
+// Updates the next launch of a run of n should make: 4 or 2 fused ones where
+// the lattice has such a kernel, else 1.
+int fused_updates(const mdf_t h, long long n) {
+  if (!h->fuse || n < 2) return 1;
+  const int K = n >= 4 && h->ny >= 4 ? 4 : 2;
+  return h->ny >= K ? K : 1;
+}
+
+// Enqueue the next launch of a run of n updates, `tk` updates into its
+// launch group, and move to its result; *k is the updates it makes.
+cudaError_t launch_next(mdf_t h, long long n, int tk, int *k) {
+  DevArgs a = base_args(h);
+  a.tk = tk;
+  *k = fused_updates(h, n);
+  const LatticeLaunch *l = lattice_launch(h->d, h->q);
+  const cudaError_t e = *k > 1 ? l->fused(*k, h->walls, a, h->stream)
+                               : l->update(h->storage, MODE_STEP, h->walls, a, h->stream);
+  if (h->inplace) h->parity ^= 1;
+  else std::swap(h->cur, h->nxt);
+  return e;
+}
+
 // Capture kGraphChunk updates starting from buffer `which` (the AA parity
 // for the in-place pattern) into a graph.
 mdf_status build_graph(mdf_t h, int which) {
@@ -225,13 +252,8 @@ mdf_status build_graph(mdf_t h, int which) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    for (int k = 0; k < kGraphChunk && e == cudaSuccess; ++k) {
-      DevArgs a = base_args(h);
-      a.tk = k;  // the step is *clock + k; the clock is set before each replay
-      e = launch_update(h, MODE_STEP, a);
-      if (h->inplace) h->parity ^= 1;
-      else std::swap(h->cur, h->nxt);
-    }
+    for (int k = 0, made = 0; k < kGraphChunk && e == cudaSuccess; k += made)
+      e = launch_next(h, kGraphChunk - k, k, &made);  // the step is *clock + k; the clock is set before each replay
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
     if (e == cudaSuccess) e = e2;
   }
@@ -264,12 +286,10 @@ mdf_status run_steps(mdf_t h, long long n) {
     h->step += kGraphChunk;
   }
   if (n > 0) CU(h, launch_set_clock(h->clock, (int)h->step, h->stream));
-  for (int k = 0; k < n; ++k) {
-    DevArgs a = base_args(h);
-    a.tk = k;
-    CU(h, launch_update(h, MODE_STEP, a));
-    if (h->inplace) h->parity ^= 1;
-    else std::swap(h->cur, h->nxt);
+  for (long long k = 0; k < n;) {
+    int made = 1;
+    CU(h, launch_next(h, n - k, (int)k, &made));
+    k += made;
   }
   h->step += n;
   return MDF_OK;
@@ -378,6 +398,9 @@ mdf_status mdf_create(mdf_t *out, const mdf_grid *g, int d, const mdf_rates *r,
   h->block = opts.block ? opts.block : (h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage));
   h->vx = opts.vx ? opts.vx : (h->inplace ? default_vx_aa(d, h->storage) : default_vx(d, h->storage));
   h->vx = std::min(h->vx, max_vx(d, h->storage, h->inplace));
+  // a caller's own launch shape is that of the one-update kernel
+  h->fuse = lattice_launch(d, q)->fused && h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
+            !opts.block && h->plane < (1LL << 31) - 64;
 
   const size_t pb = h->pop_bytes();
   cudaError_t e = cudaMalloc(&h->buf[0], pb);

@@ -130,33 +130,6 @@ template <> struct Lanes<1> {
   static constexpr int N = 1, W = 1;
 };
 
-__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-
-#define MDF_F32X2_BINARY(name, op)                                                              \
-  __device__ __forceinline__ float2 name(float2 a, float2 b) {                                  \
-    float2 r;                                                                                   \
-    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n " op           \
-        " d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"                                                 \
-        : "=f"(r.x), "=f"(r.y)                                                                  \
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                              \
-    return r;                                                                                   \
-  }
-MDF_F32X2_BINARY(vadd, "add.rn.f32x2")
-MDF_F32X2_BINARY(vsub, "sub.rn.f32x2")
-MDF_F32X2_BINARY(vmul, "mul.rn.f32x2")
-#undef MDF_F32X2_BINARY
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) {
-  float2 r;
-  asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
-      " mov.b64 c, {%6, %7};\n fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return r;
-}
-
 template <class T> __device__ __forceinline__ T splat(float c);
 template <> __device__ __forceinline__ float splat<float>(float c) { return c; }
 template <> __device__ __forceinline__ float2 splat<float2>(float c) { return make_float2(c, c); }

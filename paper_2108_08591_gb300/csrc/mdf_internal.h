@@ -25,6 +25,7 @@ struct DevArgs {
   double s1, s2;                 // relaxation rates (s0 never acts: m0 = m0eq)
   float s1f, s2f;                // the same rates rounded to FP32 on the host
   double lid_u[3];               // lid velocity
+  int wall[3], lid;              // walls per axis, lid on the + face of the last axis
   // derived-field outputs (dense [N] layout), each nullable
   double *P, *u, *rho, *G, *div, *S, *sigma, *omega;
   // init inputs (dense FP64 on the device); Gin [d][d][N] nullable
@@ -88,18 +89,25 @@ cudaError_t launch_reduce_d3q6(int storage, bool walls, int kind, const DevArgs 
 cudaError_t launch_mask_d3q6(const int wall[3], int lid, const DevArgs &a, uint8_t *mask,
                              cudaStream_t s);
 
-// The four launchers of one lattice.
+// K = 2 or 4 updates in one launch (FP32, two buffers, all d + 1 sets, ny >= K).
+cudaError_t launch_fused_d2q5(int K, bool walls, const DevArgs &a, cudaStream_t s);
+cudaError_t launch_fused_d2q4(int K, bool walls, const DevArgs &a, cudaStream_t s);
+
+// The launchers of one lattice (fused: null where it is not built).
 struct LatticeLaunch {
   cudaError_t (*update)(int storage, int mode, bool walls, const DevArgs &a, cudaStream_t s);
   cudaError_t (*init)(int storage, bool walls, const DevArgs &a, cudaStream_t s);
   cudaError_t (*reduce)(int storage, bool walls, int kind, const DevArgs &a, cudaStream_t s);
   cudaError_t (*mask)(const int wall[3], int lid, const DevArgs &a, uint8_t *mask, cudaStream_t s);
+  cudaError_t (*fused)(int K, bool walls, const DevArgs &a, cudaStream_t s);
 };
 inline const LatticeLaunch *lattice_launch(int d, int q) {
-  static const LatticeLaunch d2q5{launch_update_d2q5, launch_init_d2q5, launch_reduce_d2q5, launch_mask_d2q5};
-  static const LatticeLaunch d3q7{launch_update_d3q7, launch_init_d3q7, launch_reduce_d3q7, launch_mask_d3q7};
-  static const LatticeLaunch d2q4{launch_update_d2q4, launch_init_d2q4, launch_reduce_d2q4, launch_mask_d2q4};
-  static const LatticeLaunch d3q6{launch_update_d3q6, launch_init_d3q6, launch_reduce_d3q6, launch_mask_d3q6};
+  static const LatticeLaunch d2q5{launch_update_d2q5, launch_init_d2q5, launch_reduce_d2q5, launch_mask_d2q5,
+                                  launch_fused_d2q5};
+  static const LatticeLaunch d3q7{launch_update_d3q7, launch_init_d3q7, launch_reduce_d3q7, launch_mask_d3q7, nullptr};
+  static const LatticeLaunch d2q4{launch_update_d2q4, launch_init_d2q4, launch_reduce_d2q4, launch_mask_d2q4,
+                                  launch_fused_d2q4};
+  static const LatticeLaunch d3q6{launch_update_d3q6, launch_init_d3q6, launch_reduce_d3q6, launch_mask_d3q6, nullptr};
   if (d == 2) return q == 5 ? &d2q5 : q == 4 ? &d2q4 : nullptr;
   if (d == 3) return q == 7 ? &d3q7 : q == 6 ? &d3q6 : nullptr;
   return nullptr;

@@ -15,6 +15,7 @@
 //   f_i(x, t) = -f*_{opp(i)}(x, t - 1) + 2 w_i ubar_wall.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "mdf_internal.h"
@@ -199,64 +200,62 @@ __device__ __forceinline__ void write_fields(const DevArgs &A, long long n, long
 // DITHER (FP32 storage): the velocity sets' post-collision values are
 // rounded stochastically, with the offsets drawn from `key` (node_key of
 // the node's global index and the time step; see mdf_lattice.cuh).
-template <class L, class TC, bool S2 = false>
-__device__ __forceinline__ void node_moments(const TC (&g)[L::D][L::Q], const TC (&F)[L::D],
+template <class L, class TC, bool S2 = false, class TF>
+__device__ __forceinline__ void node_moments(const TC (&g)[L::D][L::Q], const TF (&F)[L::D],
                                              TC (&u)[L::D], TC &Pp) {
   constexpr int D = L::D, Q = L::Q;
   // Eq. 2-7: u_alpha = sum_i f_{i,alpha} (the rest shift has zero sum);
   // Eq. 3-15: P' = (1/d)(sum_alpha sum_i c_{i,alpha} g_{i,alpha} - |u|^2).
-  TC tr = TC(0), usq = TC(0);
+  TC tr{}, usq{};
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    TC s = TC(0), t = TC(0);
+    TC s = g[a][0], p{}, m{};  // p, m: the populations along +e_a and -e_a
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      s += g[a][i];
-      if (L::c(i, a) > 0) t += g[a][i];
-      if (L::c(i, a) < 0) t -= g[a][i];
+      if (i > 0) s += g[a][i];
+      if (L::c(i, a) > 0) p = g[a][i];
+      if (L::c(i, a) < 0) m = g[a][i];
     }
-    if constexpr (S2) u[a] = s + TC(0.5) * F[a];  // Eq. 2-7a
+    if constexpr (S2) u[a] = s + lit<TC, (LIT_1_2)>() * F[a];  // Eq. 2-7a
     else u[a] = s;
-    tr += t;
+    tr = a == 0 ? p - m : tr + (p - m);
   }
 #pragma unroll
-  for (int a = 0; a < D; ++a) usq += u[a] * u[a];
-  Pp = (tr - usq) * TC(1.0 / D);
+  for (int a = 0; a < D; ++a) usq = a == 0 ? u[a] * u[a] : usq + u[a] * u[a];
+  Pp = (tr - usq) * lit<TC, (D == 2 ? LIT_1_2 : LIT_1_3)>();
 }
 
 // Relaxation of velocity set a (alpha = a + 1) of one node from its moments.
-template <class L, class TC, bool DITHER = false>
+template <class L, class TC, bool DITHER = false, class TF>
 __device__ __forceinline__ void relax_velocity_set(TC (&ga)[L::Q], int a, const TC (&u)[L::D], TC Pp,
-                                                   TC s1, TC s2, TC Fa, uint32_t key) {
+                                                   const Rates<TC> &R, TF Fa,
+                                                   typename NodeKey<TC>::T key) {
   constexpr int D = L::D, Q = L::Q;
   TC jeq[D];  // Eq. 3-7a: sum_i c_i f^eq = u_alpha u + P E_alpha (shifted: P')
 #pragma unroll
-  for (int b = 0; b < D; ++b) jeq[b] = u[a] * u[b] + (a == b ? Pp : TC(0));
+  for (int b = 0; b < D; ++b) jeq[b] = a == b ? u[a] * u[b] + Pp : u[a] * u[b];
   if constexpr (DITHER) {  // population k = a Q + i draws byte k & 3 of word k >> 2
-    float rz[Q];
+    TC rz[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int k = a * Q + i;
-      rz[i] = rand_scale(rand_word(key, k >> 2), k & 3);
-    }
-    L::template relax<true>(ga, jeq, s1, s2, Fa, rz);
+    for (int i = 0; i < Q; ++i) rz[i] = draw<TC>(key, a * Q + i);
+    L::template relax<true>(ga, jeq, R, Fa, rz);
   } else {
-    L::relax(ga, jeq, s1, s2, Fa);
+    L::relax(ga, jeq, R, Fa);
   }
 }
 
 // Relaxation of the alpha = 0 set of one node (ubar_0 = rho0 + rho'); r
 // receives rho'.
 template <class L, class TC>
-__device__ __forceinline__ void relax_rho_set(TC (&h)[L::Q], const TC (&u)[L::D], TC s1, TC s2, TC &r) {
+__device__ __forceinline__ void relax_rho_set(TC (&h)[L::Q], const TC (&u)[L::D], const Rates<TC> &R, TC &r) {
   constexpr int D = L::D, Q = L::Q;
-  r = TC(0);
+  r = h[0];
 #pragma unroll
-  for (int i = 0; i < Q; ++i) r += h[i];
+  for (int i = 1; i < Q; ++i) r += h[i];
   TC jeq[D];  // ubar_0 u
 #pragma unroll
-  for (int b = 0; b < D; ++b) jeq[b] = (TC(1) + r) * u[b];
-  L::relax(h, jeq, s1, s2, TC(0));
+  for (int b = 0; b < D; ++b) jeq[b] = (lit<TC, (LIT_1)>() + r) * u[b];
+  L::relax(h, jeq, R, NoForce{});
 }
 
 template <class L, class TC, bool S2 = false, bool DITHER = false>
@@ -265,16 +264,17 @@ __device__ __forceinline__ void collide_node(TC (&g)[L::D][L::Q], TC (&h)[L::Q],
                                              TC (&M)[L::D + 2], uint32_t key = 0u) {
   constexpr int D = L::D;
   TC u[D], Pp;
+  const Rates<TC> R(s1, s2);
   node_moments<L, TC, S2>(g, F, u, Pp);
 #pragma unroll
   for (int a = 0; a < D; ++a) M[a] = u[a];
   M[D] = Pp;
   M[D + 1] = TC(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) relax_velocity_set<L, TC, DITHER>(g[a], a, u, Pp, s1, s2, F[a], key);
+  for (int a = 0; a < D; ++a) relax_velocity_set<L, TC, DITHER>(g[a], a, u, Pp, R, F[a], key);
   if (with_rho) {
     TC r;
-    relax_rho_set<L, TC>(h, u, s1, s2, r);
+    relax_rho_set<L, TC>(h, u, R, r);
     M[D + 1] = r;
   }
 }
@@ -676,6 +676,7 @@ __device__ __forceinline__ void update_vec_body(const DevArgs &A) {
   // relaxed for every node and stored, so that its registers are free for
   // the next set (the node-by-node order needs ~145 registers here).
   TC u[VX][D], Pp[VX];
+  const Rates<TC> R(s1, s2);
   uint32_t key[VX];
   const int tstep = DZ ? launch_step(A) : 0;
 #pragma unroll
@@ -697,7 +698,7 @@ __device__ __forceinline__ void update_vec_body(const DevArgs &A) {
       TC ga[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) ga[i] = g[a][i][j];
-      relax_velocity_set<L, TC, DZ>(ga, a, u[j], Pp[j], s1, s2, F[a][j], key[j]);
+      relax_velocity_set<L, TC, DZ>(ga, a, u[j], Pp[j], R, F[a][j], key[j]);
 #pragma unroll
       for (int i = 0; i < Q; ++i) g[a][i][j] = ga[i];
     }
@@ -712,7 +713,7 @@ __device__ __forceinline__ void update_vec_body(const DevArgs &A) {
       TC hn[Q], r;
 #pragma unroll
       for (int i = 0; i < Q; ++i) hn[i] = h[i][j];
-      relax_rho_set<L, TC>(hn, u[j], s1, s2, r);
+      relax_rho_set<L, TC>(hn, u[j], R, r);
 #pragma unroll
       for (int i = 0; i < Q; ++i) h[i][j] = hn[i];
     }

@@ -26,6 +26,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "mdf_f32x2.cuh"
+
 namespace mdf {
 
 // ---------------------------------------------------------------------------
@@ -98,13 +100,38 @@ __device__ __forceinline__ float dithered_change(float dl, float v, float r) {
   return __fmaf_rn(r, p2, __fmaf_rn(-1.498046875f * 0x1p-23f, p2, dl));
 }
 
+__device__ __forceinline__ F2 dithered_change(F2 dl, F2 v, F2 r) {  // lane by lane the same
+  const float2 p2 = make_float2(__int_as_float(__float_as_int(v.x) & 0x7f800000),
+                                __int_as_float(__float_as_int(v.y) & 0x7f800000));
+  return F2(vfma(r.f2(), p2, vfma(kLit2[LIT_DITHER], p2, dl.f2())));
+}
+
+// Random keys of one node (float) or of a pair of nodes (F2), and their
+// draw for population k: byte k & 3 of word k >> 2.
+template <class TC> struct NodeKey { using T = uint32_t; };
+template <> struct NodeKey<F2> { using T = uint2; };
+template <class TC> __device__ __forceinline__ TC draw(uint32_t key, int k) {
+  return rand_scale(rand_word(key, k >> 2), k & 3);
+}
+template <class TC> __device__ __forceinline__ F2 draw(uint2 key, int k) {
+  return F2(rand_scale(rand_word(key.x, k >> 2), k & 3), rand_scale(rand_word(key.y, k >> 2), k & 3));
+}
+
 // g <- g + dl: the change of a population added once, dithered for FP32
 // storage (DZ) with the random scale rz[i].
 template <bool DZ, class TC>
-__device__ __forceinline__ void add_change(TC &g, TC dl, const float *rz, int i) {
+__device__ __forceinline__ void add_change(TC &g, TC dl, const TC *rz, int i) {
   if constexpr (DZ) g = g + dithered_change(dl, g, rz[i]);
   else g = g + dl;
 }
+// Relaxation rates as relax() uses them.  The halves and quarters of M^-1's
+// columns are taken into the rates: scaling by a power of two is exact.
+template <class TC> struct Rates {
+  TC s1h, s2, s2h, s2q;  // s1 / 2, s2, s2 / 2, s2 / 4
+  __device__ __forceinline__ Rates(TC s1, TC s2_)
+      : s1h(lit<TC, (LIT_1_2)>() * s1), s2(s2_), s2h(lit<TC, (LIT_1_2)>() * s2_), s2q(lit<TC, (LIT_1_2)>() * s2h) {}
+};
+
 // Round-to-nearest storage (16-bit rest-shifted, FP64): the change of each
 // population is added term by term, g - h1 - ... + w F, in the order that
 // keeps fewest values live; the stored rounding dominates there.
@@ -136,24 +163,24 @@ struct D2Q5 {
   // jeq[b]: equilibrium first moment (shifted); F: source Fbar_alpha; rz:
   // random scales (rand_scale) dithering each change before it meets g (DZ,
   // FP32 only).
-  template <bool DZ = false, class TC>
-  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], TC s1, TC s2, TC F,
-                                               const float *rz = nullptr) {
+  template <bool DZ = false, class TC, class TF>
+  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
+                                               const TC *rz = nullptr) {
     const TC m0 = g[0] + g[1] + g[2] + g[3] + g[4];
-    const TC d1 = s1 * ((g[1] - g[3]) - jeq[0]);
-    const TC d2 = s1 * ((g[2] - g[4]) - jeq[1]);
-    const TC d3 = s2 * ((g[1] + g[3]) - (g[2] + g[4]));
-    const TC d4 = s2 * ((g[1] + g[2] + g[3] + g[4]) - TC(4) * g[0] + TC(2.0 / 3.0) * m0);
-    const TC h1 = TC(0.5) * d1, h2 = TC(0.5) * d2, q3 = TC(0.25) * d3, e4 = TC(0.05) * d4;
-    const TC Fw = F * TC(1.0 / 6.0);
+    const TC h1 = R.s1h * ((g[1] - g[3]) - jeq[0]);
+    const TC h2 = R.s1h * ((g[2] - g[4]) - jeq[1]);
+    const TC q3 = R.s2q * ((g[1] + g[3]) - (g[2] + g[4]));
+    const TC d4 = R.s2 * (add_scaled<LIT_M4>(g[1] + g[2] + g[3] + g[4], g[0]) + lit<TC, (LIT_2_3)>() * m0);
+    const TC e4 = lit<TC, (LIT_1_20)>() * d4;
+    const auto Fw = F * TC(1.0 / 6.0);
     if constexpr (DZ) {
-      add_change<DZ>(g[0], TC(0.2) * d4 + F * TC(1.0 / 3.0), rz, 0);
+      add_change<DZ>(g[0], lit<TC, (LIT_1_5)>() * d4 + F * TC(1.0 / 3.0), rz, 0);
       add_change<DZ>(g[1], ((Fw - h1) - q3) - e4, rz, 1);
       add_change<DZ>(g[2], ((Fw - h2) + q3) - e4, rz, 2);
       add_change<DZ>(g[3], ((Fw + h1) - q3) - e4, rz, 3);
       add_change<DZ>(g[4], ((Fw + h2) + q3) - e4, rz, 4);
     } else {
-      g[0] = g[0] + TC(0.2) * d4 + F * TC(1.0 / 3.0);
+      g[0] = g[0] + lit<TC, (LIT_1_5)>() * d4 + F * TC(1.0 / 3.0);
       g[1] = g[1] - h1 - q3 - e4 + Fw;
       g[2] = g[2] - h2 + q3 - e4 + Fw;
       g[3] = g[3] + h1 - q3 - e4 + Fw;
@@ -185,23 +212,21 @@ struct D3Q7 {
   __host__ __device__ static constexpr double w(int i) { return i == 0 ? 0.25 : 0.125; }
   static constexpr int UP = 5;
 
-  template <bool DZ = false, class TC>
-  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], TC s1, TC s2, TC F,
-                                               const float *rz = nullptr) {
+  template <bool DZ = false, class TC, class TF>
+  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
+                                               const TC *rz = nullptr) {
     const TC sx = g[1] + g[2], sy = g[3] + g[4], sz = g[5] + g[6];
     const TC m0 = g[0] + sx + sy + sz;
-    const TC d1 = s1 * ((g[1] - g[2]) - jeq[0]);
-    const TC d2 = s1 * ((g[3] - g[4]) - jeq[1]);
-    const TC d3 = s1 * ((g[5] - g[6]) - jeq[2]);
-    const TC d4 = s2 * ((sx + sy + sz) - TC(6) * g[0] + TC(0.75) * m0);
-    const TC d5 = s2 * (TC(2) * sx - sy - sz);
-    const TC d6 = s2 * (sy - sz);
-    const TC h1 = TC(0.5) * d1, h2 = TC(0.5) * d2, h3 = TC(0.5) * d3;
-    const TC e4 = d4 * TC(1.0 / 42.0);
-    const TC ex = d5 * TC(1.0 / 6.0), eo = d5 * TC(1.0 / 12.0), q6 = TC(0.25) * d6;
-    const TC Fw = F * TC(0.125);
+    const TC h1 = R.s1h * ((g[1] - g[2]) - jeq[0]);
+    const TC h2 = R.s1h * ((g[3] - g[4]) - jeq[1]);
+    const TC h3 = R.s1h * ((g[5] - g[6]) - jeq[2]);
+    const TC d4 = R.s2 * ((sx + sy + sz) + lit<TC, (LIT_M6)>() * g[0] + lit<TC, (LIT_3_4)>() * m0);
+    const TC d5h = R.s2h * ((sx + sx) - sy - sz);
+    const TC e4 = d4 * lit<TC, (LIT_1_42)>();
+    const TC eo = d5h * lit<TC, (LIT_1_6)>(), ex = eo + eo, q6 = R.s2q * (sy - sz);
+    const auto Fw = F * TC(0.125);
     if constexpr (DZ) {
-      add_change<DZ>(g[0], d4 * TC(1.0 / 7.0) + F * TC(0.25), rz, 0);
+      add_change<DZ>(g[0], d4 * lit<TC, (LIT_1_7)>() + F * TC(0.25), rz, 0);
       add_change<DZ>(g[1], ((Fw - h1) - e4) - ex, rz, 1);
       add_change<DZ>(g[2], ((Fw + h1) - e4) - ex, rz, 2);
       add_change<DZ>(g[3], (((Fw - h2) - e4) + eo) - q6, rz, 3);
@@ -209,7 +234,7 @@ struct D3Q7 {
       add_change<DZ>(g[5], (((Fw - h3) - e4) + eo) + q6, rz, 5);
       add_change<DZ>(g[6], (((Fw + h3) - e4) + eo) + q6, rz, 6);
     } else {
-      g[0] = g[0] + d4 * TC(1.0 / 7.0) + F * TC(0.25);
+      g[0] = g[0] + d4 * lit<TC, (LIT_1_7)>() + F * TC(0.25);
       g[1] = g[1] - h1 - e4 - ex + Fw;
       g[2] = g[2] + h1 - e4 - ex + Fw;
       g[3] = g[3] - h2 - e4 + eo - q6 + Fw;
@@ -240,14 +265,13 @@ struct D2Q4 {
   __host__ __device__ static constexpr double w(int) { return 0.25; }
   static constexpr int UP = 1;
 
-  template <bool DZ = false, class TC>
-  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], TC s1, TC s2, TC F,
-                                               const float *rz = nullptr) {
-    const TC d1 = s1 * ((g[0] - g[2]) - jeq[0]);
-    const TC d2 = s1 * ((g[1] - g[3]) - jeq[1]);
-    const TC d3 = s2 * ((g[0] + g[2]) - (g[1] + g[3]));
-    const TC h1 = TC(0.5) * d1, h2 = TC(0.5) * d2, q3 = TC(0.25) * d3;
-    const TC Fw = F * TC(0.25);
+  template <bool DZ = false, class TC, class TF>
+  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
+                                               const TC *rz = nullptr) {
+    const TC h1 = R.s1h * ((g[0] - g[2]) - jeq[0]);
+    const TC h2 = R.s1h * ((g[1] - g[3]) - jeq[1]);
+    const TC q3 = R.s2q * ((g[0] + g[2]) - (g[1] + g[3]));
+    const auto Fw = F * TC(0.25);
     if constexpr (DZ) {
       add_change<DZ>(g[0], (Fw - h1) - q3, rz, 0);
       add_change<DZ>(g[1], (Fw - h2) + q3, rz, 1);
@@ -279,18 +303,16 @@ struct D3Q6 {
   __host__ __device__ static constexpr double w(int) { return 1.0 / 6.0; }
   static constexpr int UP = 4;
 
-  template <bool DZ = false, class TC>
-  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], TC s1, TC s2, TC F,
-                                               const float *rz = nullptr) {
+  template <bool DZ = false, class TC, class TF>
+  static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
+                                               const TC *rz = nullptr) {
     const TC sx = g[0] + g[1], sy = g[2] + g[3], sz = g[4] + g[5];
-    const TC d1 = s1 * ((g[0] - g[1]) - jeq[0]);
-    const TC d2 = s1 * ((g[2] - g[3]) - jeq[1]);
-    const TC d3 = s1 * ((g[4] - g[5]) - jeq[2]);
-    const TC d4 = s2 * (TC(2) * sx - sy - sz);
-    const TC d5 = s2 * (sy - sz);
-    const TC h1 = TC(0.5) * d1, h2 = TC(0.5) * d2, h3 = TC(0.5) * d3;
-    const TC ex = d4 * TC(1.0 / 6.0), eo = d4 * TC(1.0 / 12.0), q5 = TC(0.25) * d5;
-    const TC Fw = F * TC(1.0 / 6.0);
+    const TC h1 = R.s1h * ((g[0] - g[1]) - jeq[0]);
+    const TC h2 = R.s1h * ((g[2] - g[3]) - jeq[1]);
+    const TC h3 = R.s1h * ((g[4] - g[5]) - jeq[2]);
+    const TC d4h = R.s2h * ((sx + sx) - sy - sz);
+    const TC eo = d4h * lit<TC, (LIT_1_6)>(), ex = eo + eo, q5 = R.s2q * (sy - sz);
+    const auto Fw = F * TC(1.0 / 6.0);
     if constexpr (DZ) {
       add_change<DZ>(g[0], (Fw - h1) - ex, rz, 0);
       add_change<DZ>(g[1], (Fw + h1) - ex, rz, 1);

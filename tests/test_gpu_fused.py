@@ -1,0 +1,60 @@
+"""Fused updates (several per launch, 2D FP32) against single updates: the
+same bits for every boundary, force scheme, width and number of steps."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+# strip edges (56 and 60 stored columns of 64), odd and even rows, rows too
+# short for the deeper kernels, one to several strips
+SHAPES = [(2, 4), (3, 5), (24, 7), (55, 9), (56, 2), (57, 4), (60, 33), (61, 12), (64, 64), (113, 17),
+          (128, 3), (129, 130), (300, 41)]
+BCS = [((0, 0), False), ((1, 0), False), ((0, 1), True), ((1, 1), True)]
+
+
+@pytest.mark.parametrize("q", [0, 4])
+@pytest.mark.parametrize("forcing", ["none", "eq3-21", "scheme2"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_fused_updates_equal_single_updates(shape, forcing, q):
+    import torch
+    from paper_2108_08591_gb300 import Lattice
+
+    N = shape[0] * shape[1]
+    rng = np.random.default_rng([*shape, q])
+    P = 1.0 + 1e-3 * rng.standard_normal(N)
+    u, F = 0.01 * rng.standard_normal((2, N)), 1e-5 * rng.standard_normal((2, N))
+    for wall, lid in BCS:
+        outs = []
+        for kw in ({}, {"vx": 1}):  # an own launch shape keeps to single updates
+            lat = Lattice(shape, s1=1.8, wall=wall, lid=lid, lid_u=(0.05, 0.01, 0.0), q=q, **kw)
+            if forcing != "none":
+                lat.set_forcing(forcing)
+                lat.set_force(F)
+            lat.init(P, u)
+            got = []
+            for n in (1, 2, 3, 4, 7):  # 1: single; 2, 3: one launch of two; 4, 7: of four
+                lat.step(n)
+                got += [v.clone() for v in lat.fields(("P", "u", "rho", "G")).values()]
+            lat.close()
+            outs.append(got)
+        for a, b in zip(*outs):
+            assert torch.equal(a, b), (wall, lid)
+
+
+def test_fused_updates_in_a_captured_chunk():
+    import torch
+    from paper_2108_08591_gb300 import Lattice
+
+    P = np.ones(97 * 50)
+    u = 0.01 * np.random.default_rng(1).standard_normal((2, 97 * 50))
+    outs = []
+    for kw in ({}, {"vx": 1}):
+        s = torch.cuda.Stream()
+        lat = Lattice((97, 50), s1=1.7, stream=s, **kw)
+        lat.init(P, u)
+        lat.step(64 * 2 + 3)
+        lat.step(64 + 1)
+        outs.append(lat.fields_host(("P", "u", "G")))
+        lat.close()
+    for k in outs[0]:
+        assert np.array_equal(outs[0][k], outs[1][k]), k
