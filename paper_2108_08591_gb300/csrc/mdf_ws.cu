@@ -21,6 +21,7 @@
 #include <string>
 #include <vector>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -40,6 +41,7 @@ struct Layer {
 };
 
 inline unsigned grid1(long long n, int b = 256) { return (unsigned)((n + b - 1) / b); }
+constexpr int kBiasBlocks = 152 * 4;  // row blocks of the bias gradients (four per SM)
 
 // SplitMix64 (Steele, Lea & Flood 2014) for the weight initialisation.
 inline uint64_t splitmix(uint64_t &s) {
@@ -68,9 +70,9 @@ struct mdf_ws_s {
   // gradients / scratch
   bf16 *dyh = nullptr, *wt = nullptr, *gA = nullptr, *gB = nullptr, *gC = nullptr;
   std::vector<bf16 *> dcat;
-  float *part = nullptr;
+  float *part = nullptr, *bpart = nullptr;  // weight / bias gradient partial sums
   double *lpart = nullptr;
-  long long part_n = 0, wt_n = 0, gbuf_n = 0;
+  long long part_n = 0, gbuf_n = 0;
   std::string err = "no error";
 
   int Hl(int l) const { return H >> l; }
@@ -212,46 +214,6 @@ void halo_tile(const ConvArgs &a, int &bn, int &kc, int &mt) {
   if (g_halo_mt) mt = g_halo_mt;
 }
 
-cudaError_t conv_fwd(cudaStream_t s, const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
-                     float *yf, int B, int H, int W, int Cin, int Cout, int ldy, int yoff,
-                     int relu) {
-  ConvArgs a{x, w, bias, y, yf, B, H, W, Cin, Cout, ldy, yoff, relu};
-  const long long M = (long long)B * H * W;
-  if (g_conv_kernel == 2 && Cin % 16 == 0) {
-    int *err = tc_error_flag();
-    if (!err) return cudaErrorMemoryAllocation;
-    int bn, kc, mt;
-    halo_tile(a, bn, kc, mt);
-    switch (bn) {
-      case 16: return launch_halo_bn<16>(s, a, err, kc, mt);
-      case 32: return launch_halo_bn<32>(s, a, err, kc, mt);
-      case 64: return launch_halo_bn<64>(s, a, err, kc, mt);
-      case 128: return launch_halo_bn<128>(s, a, err, kc, mt);
-      case 256: return launch_halo_bn<256>(s, a, err, kc, mt);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  if (g_conv_kernel >= 1) {
-    int *err = tc_error_flag();
-    if (!err) return cudaErrorMemoryAllocation;
-    int bn, st;
-    tc_tile(M, Cout, bn, st);
-    switch (bn) {
-      case 16: return launch_tc_s<16>(s, a, M, err, st);
-      case 32: return launch_tc_s<32>(s, a, M, err, st);
-      case 64: return launch_tc_s<64>(s, a, M, err, st);
-      case 128: return launch_tc_s<128>(s, a, M, err, st);
-      case 256: return launch_tc_s<256>(s, a, M, err, st);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  dim3 grid((unsigned)((M + CBM - 1) / CBM), (unsigned)((Cout + CBN - 1) / CBN));
-  k_conv_fwd<<<grid, 128, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-int pix_per_split(long long M) { return M >= 8192 ? 2048 : 256; }
-
 // Streaming multiprocessors of the current device (152 when the query fails).
 int sm_count() {
   int dev = 0, n = 0;
@@ -300,6 +262,47 @@ bool nhwc_map(CUtensorMap *m, const bf16 *p, int B, int H, int W, int C, int bc,
             CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+
+cudaError_t conv_fwd(cudaStream_t s, const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
+                     float *yf, int B, int H, int W, int Cin, int Cout, int ldy, int yoff,
+                     int relu) {
+  ConvArgs a{x, w, bias, y, yf, B, H, W, Cin, Cout, ldy, yoff, relu};
+  const long long M = (long long)B * H * W;
+  if (g_conv_kernel == 2 && Cin % 16 == 0) {
+    int *err = tc_error_flag();
+    if (!err) return cudaErrorMemoryAllocation;
+    int bn, kc, mt;
+    halo_tile(a, bn, kc, mt);
+    switch (bn) {
+      case 16: return launch_halo_bn<16>(s, a, err, kc, mt);
+      case 32: return launch_halo_bn<32>(s, a, err, kc, mt);
+      case 64: return launch_halo_bn<64>(s, a, err, kc, mt);
+      case 128: return launch_halo_bn<128>(s, a, err, kc, mt);
+      case 256: return launch_halo_bn<256>(s, a, err, kc, mt);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  if (g_conv_kernel >= 1) {
+    int *err = tc_error_flag();
+    if (!err) return cudaErrorMemoryAllocation;
+    int bn, st;
+    tc_tile(M, Cout, bn, st);
+    switch (bn) {
+      case 16: return launch_tc_s<16>(s, a, M, err, st);
+      case 32: return launch_tc_s<32>(s, a, M, err, st);
+      case 64: return launch_tc_s<64>(s, a, M, err, st);
+      case 128: return launch_tc_s<128>(s, a, M, err, st);
+      case 256: return launch_tc_s<256>(s, a, M, err, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  dim3 grid((unsigned)((M + CBM - 1) / CBM), (unsigned)((Cout + CBN - 1) / CBN));
+  k_conv_fwd<<<grid, 128, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+int pix_per_split(long long M) { return M >= 8192 ? 2048 : 256; }
 
 template <bool SWAP, int KC, int BN, int S>
 cudaError_t launch_wgrad_tma(cudaStream_t s, const CUtensorMap &xm, const CUtensorMap &dm, const WgradTmaArgs &a,
@@ -375,6 +378,40 @@ int wgrad_tile(int C) {
   return C % 64 == 0 ? 64 : C % 32 == 0 ? 32 : 16;
 }
 
+cudaError_t sum_splits(cudaStream_t s, const float *part, int splits, long long n, float *dst) {
+  const bool vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(part) & 15u) == 0;
+  if (splits >= 64 && n <= 4096) k_sum_splits<1, 8, 64><<<grid1(n, 8), 512, 0, s>>>(part, splits, n, dst);
+  else if (!vec) k_sum_splits<1, 32, 8><<<grid1(n, 32), 256, 0, s>>>(part, splits, n, dst);
+  else if (splits >= 64) k_sum_splits<4, 8, 32><<<grid1(n, 32), 256, 0, s>>>(part, splits, n, dst);
+  else if (splits >= 8) k_sum_splits<4, 32, 8><<<grid1(n, 128), 256, 0, s>>>(part, splits, n, dst);
+  else k_sum_splits<4, 128, 1><<<grid1(n, 512), 128, 0, s>>>(part, splits, n, dst);
+  return cudaGetLastError();
+}
+
+cudaError_t f32_to_bf16(cudaStream_t s, const float *x, bf16 *y, long long n) {
+  if (n % 8 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0)
+    k_f32_to_bf16<true><<<grid1(n / 8), 256, 0, s>>>(x, y, n);
+  else
+    k_f32_to_bf16<false><<<grid1(n), 256, 0, s>>>(x, y, n);
+  return cudaGetLastError();
+}
+
+// Adds a layer to a flip list.
+void flip_add(FlipList &f, int cin, int cout, long long off) {
+  const int k = f.n++;
+  f.cin[k] = cin;
+  f.cout[k] = cout;
+  f.off[k] = off;
+  f.tile0[k + 1] = f.tile0[k] + 9 * ((cin + 31) / 32) * ((cout + 31) / 32);
+}
+cudaError_t flip_weights(cudaStream_t s, const bf16 *w, bf16 *wt, const FlipList &f) {
+  k_flip_weights<<<(unsigned)f.tile0[f.n], 256, 0, s>>>(w, wt, f);
+  return cudaGetLastError();
+}
+
+// Grid of the row-wise element kernels: rows x runs of 256 vectors.
+dim3 row_grid(long long rows, int width, int C) { return dim3((unsigned)rows, grid1((long long)width * (C / 8))); }
+
 cudaError_t conv_wgrad(cudaStream_t s, const bf16 *x, const bf16 *dz, float *part, float *dw,
                        int B, int H, int W, int Cin, int Cout) {
   const long long M = (long long)B * H * W;
@@ -410,17 +447,13 @@ cudaError_t conv_wgrad(cudaStream_t s, const bf16 *x, const bf16 *dz, float *par
     cudaError_t e = swap ? launch_wgrad_tma_k<true>(s, kc, bn, S, xm, dm, a, err)
                          : launch_wgrad_tma_k<false>(s, kc, bn, S, xm, dm, a, err);
     if (e != cudaSuccess) return e;
-    const long long n = (long long)Cout * 9 * Cin;
-    k_sum_splits<<<grid1(n), 256, 0, s>>>(part, a.splits, n, dw, 0);
-    return cudaGetLastError();
+    return sum_splits(s, part, a.splits, (long long)Cout * 9 * Cin, dw);
   }
   const int K = 9 * Cin;
   WgradArgs a{x, dz, part, B, H, W, Cin, Cout, pps};
   dim3 grid((unsigned)((K + 63) / 64), (unsigned)((Cout + 63) / 64), (unsigned)splits);
   k_conv_wgrad<<<grid, 128, 0, s>>>(a);
-  const long long n = (long long)Cout * K;
-  k_sum_splits<<<grid1(n), 256, 0, s>>>(part, splits, n, dw, 0);
-  return cudaGetLastError();
+  return sum_splits(s, part, splits, (long long)Cout * K, dw);
 }
 
 long long wgrad_part_size(long long M, int Cin, int Cout) {
@@ -430,8 +463,10 @@ long long wgrad_part_size(long long M, int Cin, int Cout) {
 
 cudaError_t conv_dgrad(cudaStream_t s, const bf16 *dz, const bf16 *w, bf16 *wt, bf16 *dx, int B,
                        int H, int W, int Cin, int Cout) {
-  const long long n = (long long)Cout * 9 * Cin;
-  k_flip_weights<<<grid1(n), 256, 0, s>>>(w, Cout, Cin, wt);
+  FlipList f{};
+  flip_add(f, Cin, Cout, 0);
+  cudaError_t e = flip_weights(s, w, wt, f);
+  if (e != cudaSuccess) return e;
   return conv_fwd(s, dz, wt, nullptr, dx, nullptr, B, H, W, Cout, Cin, Cin, 0, 0);
 }
 
@@ -489,14 +524,13 @@ mdf_status mdf_ws_create(mdf_ws_t *out, int H, int W, int levels, const int *cha
     }
   }
   const int B = max_batch;
-  long long part_n = 0, wt_n = 0, gbuf = 0;
+  long long part_n = 0, gbuf = 0, maxc = 0;
   for (const Layer &ly : w->layers) {
     part_n = std::max(part_n, wgrad_part_size(w->Ml(ly.level, B), ly.cin, ly.cout));
-    wt_n = std::max(wt_n, (long long)ly.cout * 9 * ly.cin);
+    maxc = std::max(maxc, (long long)ly.cout);
     gbuf = std::max(gbuf, w->Ml(ly.level, B) * std::max(ly.cin, ly.cout));
   }
   w->part_n = part_n;
-  w->wt_n = wt_n;
   w->gbuf_n = gbuf;
   cudaError_t e = cudaSuccess;
   auto alloc = [&](void **ptr, size_t bytes) {
@@ -528,16 +562,16 @@ mdf_status mdf_ws_create(mdf_ws_t *out, int H, int W, int levels, const int *cha
   }
   alloc((void **)&w->yf, (size_t)w->Ml(0, B) * cout * 4);
   alloc((void **)&w->dyh, (size_t)w->Ml(0, B) * cout * 2);
-  alloc((void **)&w->wt, (size_t)wt_n * 2);
+  alloc((void **)&w->wt, np * 2);
+  alloc((void **)&w->bpart, (size_t)kBiasBlocks * maxc * 4);
   alloc((void **)&w->gA, (size_t)gbuf * 2);
   alloc((void **)&w->gB, (size_t)gbuf * 2);
   alloc((void **)&w->gC, (size_t)gbuf * 2);
   alloc((void **)&w->part, (size_t)part_n * 4);
-  alloc((void **)&w->lpart, (size_t)grid1(w->Ml(0, B) * cout) * 8);
+  alloc((void **)&w->lpart, (size_t)grid1(w->Ml(0, B)) * 8);
   if (e == cudaSuccess) e = cudaMemcpyAsync(w->p32, p.data(), np * 4, cudaMemcpyHostToDevice, w->stream);
   if (e == cudaSuccess) {
-    k_f32_to_bf16<<<grid1(w->nparam), 256, 0, w->stream>>>(w->p32, w->pbf, w->nparam);
-    e = cudaGetLastError();
+    e = f32_to_bf16(w->stream, w->p32, w->pbf, w->nparam);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
   if (e != cudaSuccess) {
@@ -556,7 +590,7 @@ void mdf_ws_destroy(mdf_ws_t w) {
   cudaStreamSynchronize(w->stream);
   for (void *p : {(void *)w->p32, (void *)w->g32, (void *)w->m, (void *)w->v, (void *)w->pbf,
                   (void *)w->xin, (void *)w->yf, (void *)w->dyh, (void *)w->wt, (void *)w->gA,
-                  (void *)w->gB, (void *)w->gC, (void *)w->part, (void *)w->lpart})
+                  (void *)w->gB, (void *)w->gC, (void *)w->part, (void *)w->bpart, (void *)w->lpart})
     cudaFree(p);
   for (auto *vec : {&w->a, &w->pool, &w->cat, &w->sdeep, &w->da, &w->db, &w->dcat})
     for (bf16 *p : *vec) cudaFree(p);
@@ -578,8 +612,7 @@ mdf_status mdf_ws_get_params(mdf_ws_t w, float *host, float *grad_host) {
 mdf_status mdf_ws_set_params(mdf_ws_t w, const float *host) {
   if (!w || !host) return MDF_EINVAL;
   WCU(w, cudaMemcpyAsync(w->p32, host, w->nparam * 4, cudaMemcpyHostToDevice, w->stream));
-  k_f32_to_bf16<<<grid1(w->nparam), 256, 0, w->stream>>>(w->p32, w->pbf, w->nparam);
-  WCU(w, cudaGetLastError());
+  WCU(w, f32_to_bf16(w->stream, w->p32, w->pbf, w->nparam));
   WCU(w, cudaMemsetAsync(w->m, 0, w->nparam * 4, w->stream));
   WCU(w, cudaMemsetAsync(w->v, 0, w->nparam * 4, w->stream));
   w->adam_step = 0;
@@ -591,8 +624,8 @@ mdf_status mdf_ws_set_params(mdf_ws_t w, const float *host) {
 
 namespace {
 
-// Forward pass of B samples already in w->xin; output in w->yf (FP32).
-mdf_status forward(mdf_ws_t w, int B) {
+// Forward pass of B samples already in w->xin; output in yf (FP32).
+mdf_status forward(mdf_ws_t w, int B, float *yf) {
   const int L = w->L;
   cudaStream_t s = w->stream;
   const bf16 *in = w->xin;
@@ -602,8 +635,8 @@ mdf_status forward(mdf_ws_t w, int B) {
     const int H = w->Hl(l), W = w->Wl(l);
     if (l > 0) {  // pool s_{l-1} (a slice of cat_{l-1})
       const int ld = w->C[l] + w->C[l - 1];
-      k_avgpool2<<<grid1(w->Ml(l, B) * w->C[l - 1]), 256, 0, s>>>(w->cat[l - 1], ld, w->C[l], B,
-                                                                   2 * H, 2 * W, w->C[l - 1], w->pool[l]);
+      k_avgpool2<<<row_grid((long long)B * H, W, w->C[l - 1]), 256, 0, s>>>(w->cat[l - 1], ld, w->C[l], 2 * H, 2 * W,
+                                                                            w->C[l - 1], w->pool[l]);
       in = w->pool[l];
       cin = w->C[l - 1];
     }
@@ -621,15 +654,15 @@ mdf_status forward(mdf_ws_t w, int B) {
     const int H = w->Hl(l), W = w->Wl(l);
     const int ld = w->C[l + 1] + w->C[l];
     const bf16 *below = (l + 1 == L - 1) ? w->sdeep[l + 1] : w->db[l + 1];
-    k_upsample2<<<grid1(w->Ml(l, B) * w->C[l + 1]), 256, 0, s>>>(below, B, H / 2, W / 2, w->C[l + 1],
-                                                                  w->cat[l], ld);
+    k_upsample2<<<row_grid((long long)B * (H / 2), W / 2, w->C[l + 1]), 256, 0, s>>>(below, H / 2, W / 2, w->C[l + 1],
+                                                                                     w->cat[l], ld);
     WCU(w, conv_fwd(s, w->cat[l], w->pbf + la.woff, w->p32 + la.boff, w->da[l], nullptr, B, H, W, ld,
                     la.cout, la.cout, 0, 1));
     WCU(w, conv_fwd(s, w->da[l], w->pbf + lb.woff, w->p32 + lb.boff, w->db[l], nullptr, B, H, W,
                     lb.cin, lb.cout, lb.cout, 0, 1));
   }
   const Layer &hd = w->head();
-  WCU(w, conv_fwd(s, w->db[0], w->pbf + hd.woff, w->p32 + hd.boff, nullptr, w->yf, B, w->H, w->W,
+  WCU(w, conv_fwd(s, w->db[0], w->pbf + hd.woff, w->p32 + hd.boff, nullptr, yf, B, w->H, w->W,
                   hd.cin, hd.cout, hd.cout, 0, 0));
   return MDF_OK;
 }
@@ -641,14 +674,19 @@ mdf_status conv_back(mdf_ws_t w, const Layer &ly, int B, const bf16 *x, const bf
   cudaStream_t s = w->stream;
   const int H = w->Hl(ly.level), W = w->Wl(ly.level);
   const long long M = w->Ml(ly.level, B);
-  const bf16 *dzp = dout;
-  if (ly.relu) {
-    k_relu_bwd<<<grid1(M * ly.cout), 256, 0, s>>>(dout, lddo, dooff, out, ldo, ooff, dz, M, ly.cout);
-    dzp = dz;
-  }
+  const bf16 *dzp = ly.relu ? dz : dout;
+  const long long rows = (M + kBiasBlocks - 1) / kBiasBlocks;
+  const int nb = (int)((M + rows - 1) / rows);
+  if (ly.relu)
+    k_relu_bias<true><<<nb, kBiasThreads, 0, s>>>(dout, lddo, dooff, out, ldo, ooff, dz, M, ly.cout, rows, w->bpart);
+  else
+    k_relu_bias<false><<<nb, kBiasThreads, 0, s>>>(dout, lddo, dooff, nullptr, 0, 0, nullptr, M, ly.cout, rows,
+                                                   w->bpart);
+  WCU(w, cudaGetLastError());
+  WCU(w, sum_splits(s, w->bpart, nb, ly.cout, w->g32 + ly.boff));
   WCU(w, conv_wgrad(s, x, dzp, w->part, w->g32 + ly.woff, B, H, W, ly.cin, ly.cout));
-  k_bias_grad<<<ly.cout, 256, 0, s>>>(dzp, (int)M, ly.cout, w->g32 + ly.boff);
-  if (dx) WCU(w, conv_dgrad(s, dzp, w->pbf + ly.woff, w->wt, dx, B, H, W, ly.cin, ly.cout));
+  if (dx)  // with the weights flipped at the start of the pass
+    WCU(w, conv_fwd(s, dzp, w->wt + ly.woff, nullptr, dx, nullptr, B, H, W, ly.cout, ly.cin, ly.cin, 0, 0));
   return MDF_OK;
 }
 
@@ -656,6 +694,10 @@ mdf_status backward(mdf_ws_t w, int B) {
   const int L = w->L;
   cudaStream_t s = w->stream;
   mdf_status st;
+  FlipList flips{};
+  for (size_t k = 1; k < w->layers.size(); ++k)  // the first layer's input takes no gradient
+    flip_add(flips, w->layers[k].cin, w->layers[k].cout, w->layers[k].woff);
+  WCU(w, flip_weights(s, w->pbf, w->wt, flips));
   // head (linear): dz = dyh; d(db_0) -> gA
   const Layer &hd = w->head();
   if ((st = conv_back(w, hd, B, w->db[0], nullptr, 0, 0, w->dyh, hd.cout, 0, nullptr, w->gA))) return st;
@@ -667,8 +709,8 @@ mdf_status backward(mdf_ws_t w, int B) {
     if ((st = conv_back(w, la, B, w->cat[l], w->da[l], la.cout, 0, w->gC, la.cout, 0, w->gB, w->dcat[l]))) return st;
     // gradient of the tensor upsampled into cat_l: level l+1's output
     const int Hn = w->Hl(l + 1), Wn = w->Wl(l + 1);
-    k_upsample2_bwd<<<grid1(w->Ml(l + 1, B) * w->C[l + 1]), 256, 0, s>>>(w->dcat[l], ld, B, Hn, Wn,
-                                                                       w->C[l + 1], w->gA);
+    k_upsample2_bwd<<<row_grid((long long)B * Hn, Wn, w->C[l + 1]), 256, 0, s>>>(w->dcat[l], ld, Hn, Wn, w->C[l + 1],
+                                                                                 w->gA);
     dout = w->gA;
   }
   // encoder, deepest first; `dout` holds the gradient of s_{L-1}
@@ -679,9 +721,9 @@ mdf_status backward(mdf_ws_t w, int B) {
     int lds, soff;
     if (l < L - 1) {
       // gradient of s_l = pooled path (in gA, level l+1 sized) + skip slice of dcat_l
-      k_avgpool2_bwd_add<<<grid1(w->Ml(l, B) * w->C[l]), 256, 0, s>>>(
-          w->gA, w->dcat[l], w->C[l + 1] + w->C[l], w->C[l + 1], B, H, W, w->C[l], w->gB);
-      WCU(w, cudaMemcpyAsync(w->gA, w->gB, w->Ml(l, B) * w->C[l] * 2, cudaMemcpyDeviceToDevice, s));
+      k_avgpool2_bwd_add<<<row_grid((long long)B * H, W, w->C[l]), 256, 0, s>>>(
+          w->gA, w->dcat[l], w->C[l + 1] + w->C[l], w->C[l + 1], H, W, w->C[l], w->gB);
+      std::swap(w->gA, w->gB);
       sl = w->cat[l];
       lds = w->C[l + 1] + w->C[l];
       soff = w->C[l + 1];
@@ -701,8 +743,7 @@ mdf_status backward(mdf_ws_t w, int B) {
 
 mdf_status load_input(mdf_ws_t w, const float *x, int B) {
   const long long n = w->Ml(0, B) * w->cin;
-  k_f32_to_bf16<<<grid1(n), 256, 0, w->stream>>>(x, w->xin, n);
-  WCU(w, cudaGetLastError());
+  WCU(w, f32_to_bf16(w->stream, x, w->xin, n));
   return MDF_OK;
 }
 
@@ -714,10 +755,7 @@ mdf_status mdf_ws_forward(mdf_ws_t w, const float *x, int B, float *y) {
   if (!w || !x || !y) return MDF_EINVAL;
   if (B < 1 || B > w->maxb) return wfail(w, MDF_EINVAL, "batch %d outside [1, %d]", B, w->maxb);
   mdf_status st = load_input(w, x, B);
-  if (st == MDF_OK) st = forward(w, B);
-  if (st != MDF_OK) return st;
-  WCU(w, cudaMemcpyAsync(y, w->yf, w->Ml(0, B) * w->cout * 4, cudaMemcpyDeviceToDevice, w->stream));
-  return MDF_OK;
+  return st == MDF_OK ? forward(w, B, y) : st;
 }
 
 mdf_status mdf_ws_train_step(mdf_ws_t w, const float *x, const float *t, int B, float lr,
@@ -725,10 +763,9 @@ mdf_status mdf_ws_train_step(mdf_ws_t w, const float *x, const float *t, int B, 
   if (!w || !x || !t) return MDF_EINVAL;
   if (B < 1 || B > w->maxb) return wfail(w, MDF_EINVAL, "batch %d outside [1, %d]", B, w->maxb);
   mdf_status st = load_input(w, x, B);
-  if (st == MDF_OK) st = forward(w, B);
+  if (st == MDF_OK) st = forward(w, B, w->yf);
   if (st != MDF_OK) return st;
-  const long long n = w->Ml(0, B) * w->cout;
-  const unsigned nb = grid1(n);
+  const unsigned nb = grid1(w->Ml(0, B));
   k_mse<<<nb, 256, 0, w->stream>>>(w->yf, w->cout, t, w->cout_used, w->Ml(0, B), w->dyh, w->lpart);
   WCU(w, cudaGetLastError());
   if ((st = backward(w, B))) return st;

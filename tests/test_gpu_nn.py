@@ -214,3 +214,34 @@ def test_every_tcgen05_tile_matches_oracle():
         lib.mdf_nn_set_tc_tile(0, 0)
         lib.mdf_nn_set_halo_tile(0, 0)
         set_conv_kernel("tcgen05-halo")
+
+
+@pytest.mark.parametrize("channels,B,H,W", [((16, 48), 3, 10, 36), ((48, 80, 16), 1, 24, 12)])
+def test_unet_gradients_odd_widths_match_oracle(channels, B, H, W):
+    """Channel counts that are no power of two, rows that do not fill a block
+    of the element-wise kernels: every gradient against the oracle.  The bounds
+    are those of test_unet_gradients_match_oracle, a third wider for the few
+    pixels summed here."""
+    import torch
+    from paper_2108_08591_gb300 import WarmStartNet
+    cin = cout = 16
+    net = WarmStartNet(H, W, channels, cin=cin, cout=cout, cout_used=3, max_batch=B, seed=5)
+    xb, xn = _bf16((B, H, W, cin), 12)
+    t = np.sin(np.arange(B * H * W * 3) * 0.37).reshape(B, H, W, 3).astype(np.float32)
+    loss = net.train_step(xb.float().contiguous(), torch.from_numpy(t).cuda(), lr=0.0)
+    y = net.forward(xb.float().contiguous()).cpu().numpy()
+    assert loss == pytest.approx(float(np.mean((y[..., :3] - t).astype(np.float64) ** 2)), rel=1e-12)
+    p, g = net.get_params(grads=True)
+    params = _oracle_params(p, cin, channels, cout)
+    # the oracle averages over all `cout` channels: pad the targets with its own output there
+    yref, _ = onn.unet_forward(params, xn, channels)
+    tp = yref.copy()
+    tp[..., :3] = t
+    _, gref, _ = onn.unet_grads(params, xn, tp, channels)
+    got = _oracle_params(g, cin, channels, cout)
+    for name in params:
+        for k in (0, 1):
+            a, b = gref[name][k].ravel() * (cout / 3.0), got[name][k].ravel()
+            assert np.dot(a, b) / (np.linalg.norm(a) * np.linalg.norm(b)) > 0.98, (name, k)
+            assert _rel(a, b) < (4e-2 if name == "head" else 0.2), (name, k)
+    net.close()
