@@ -22,12 +22,14 @@
 #include <vector>
 
 #include <algorithm>
+#include <array>
 #include <map>
 #include <mutex>
 
 #include "mdf.h"
 #include "mdf_nn.cuh"
 #include "mdf_nn_wgrad_tc.cuh"
+#include "mdf_nn_pers.cuh"
 
 using namespace mdfnn;
 
@@ -197,6 +199,9 @@ cudaError_t launch_halo_bn(cudaStream_t s, const ConvArgs &a, int *err, int kc, 
   return mt == 2 ? launch_halo<BN, 16, 2>(s, a, err) : launch_halo<BN, 16, 1>(s, a, err);
 }
 
+// Channel chunk of the halo kernel, and so the order of every forward sum.
+int halo_kc(const ConvArgs &a) { return (a.Cin % 32 == 0 && a.Cin >= 128 && a.W <= 64) ? 32 : 16; }
+
 // Tile of the halo kernel, from a sweep over the network's layer shapes
 // (B = 8, 32^2 .. 256^2, Cin 16 .. 384, Cout 16 .. 256; every shape then runs
 // its fastest measured tile): N tile = Cout rounded up to a power of two, at
@@ -205,7 +210,7 @@ cudaError_t launch_halo_bn(cudaStream_t s, const ConvArgs &a, int *err, int kc, 
 // when that still gives at least 1.5 CTAs per SM.
 void halo_tile(const ConvArgs &a, int &bn, int &kc, int &mt) {
   bn = a.Cout <= 16 ? 16 : a.Cout <= 32 ? 32 : 64;
-  kc = (a.Cin % 32 == 0 && a.Cin >= 128 && a.W <= 64) ? 32 : 16;
+  kc = halo_kc(a);
   const HaloGeom g2 = halo_geom(a.H, a.W, 2);
   const long long ctas = (long long)a.B * g2.strips * g2.tiles * ((a.Cout + bn - 1) / bn);
   mt = 2 * ctas >= 3 * 152 ? 2 : 1;
@@ -264,6 +269,122 @@ bool nhwc_map(CUtensorMap *m, const bf16 *p, int B, int H, int W, int C, int bc,
 }
 
 
+// Tensor map of weights [Cout][9][Cin] (BF16, Cin % 8 == 0, 16-byte aligned)
+// with boxes of kc input channels of one tap of bn output channels, swizzled
+// at the box's row width.
+bool weight_map(CUtensorMap *m, const bf16 *p, int Cout, int Cin, int kc, int bn) {
+  EncodeTiledFn fn = encode_tiled();
+  if (!fn || Cin % 8 != 0 || (reinterpret_cast<uintptr_t>(p) & 15u) != 0) return false;
+  const CUtensorMapSwizzle swz = kc == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                 : kc == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                            : CU_TENSOR_MAP_SWIZZLE_32B;
+  const cuuint64_t dims[3] = {(cuuint64_t)Cin, 9, (cuuint64_t)Cout};
+  const cuuint64_t strides[2] = {(cuuint64_t)Cin * 2, (cuuint64_t)Cin * 18};
+  const cuuint32_t box[3] = {(cuuint32_t)kc, 1, (cuuint32_t)bn};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16 *>(p), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Shape of a persistent convolution launch.
+struct PersPlan {
+  PersArgs g;
+  int kc = 0, mt = 0, nb = 0, grid = 0;  // kc = 0: nothing fits
+  size_t smem = 0;
+};
+
+// The plan of least estimated cycles, over the channel chunk, M tiles per
+// CTA, split of the output channels and CTAs per SM that fit.  The constants
+// are read off 90 measured launches (15 layer shapes, 6 plans each; the plan
+// it picks is the fastest measured or within 20 % of it): an M = 128, K = 16
+// step takes max(N / 2, 53 + N / 4) cycles of the tensor pipe (its
+// arithmetic, or reading A and B from shared memory), and a CTA alone on its
+// SM leaves the pipe idle for another 800 per unit (tile, chunk); a halo box
+// takes 3.4, 2 or 7.2 cycles per 32-, 64- or 128-byte pixel row; an epilogue
+// 5100 + 1090 per 128 x 32 outputs, two of them at a time.  With one box per
+// tile two M tiles per CTA lose (16 -> 32 channels, 8 x 256^2: 29.5 us
+// against 21.2).
+PersPlan pers_search(const ConvArgs &a, int sms) {
+  PersPlan best;
+  double best_cost = 0.0;
+  const int group = halo_kc(a);
+  for (int kc = 64; kc >= group; kc /= 2) {
+    if (a.Cin % kc) continue;
+    const int nc = a.Cin / kc;
+    for (int mt = 2; mt >= 1; --mt) {
+      const HaloGeom h = halo_geom(a.H, a.W, mt);
+      const int rb = pers_rows(mt, h.P);
+      const long long ntiles = (long long)a.B * h.strips * h.tiles;
+      if (rb > 256 || ntiles > 0x3fffffff || (mt == 2 && nc == 1 && ntiles > sms)) continue;
+      const double box = (double)h.P * rb * (kc == 16 ? 3.4 : kc == 64 ? 7.2 : 2.0);
+      for (int nb = (a.Cout + 127) / 128; nb <= (a.Cout + 15) / 16 && nb <= 65535; ++nb) {
+        const int bn = ((a.Cout + nb - 1) / nb + 15) / 16 * 16;
+        if ((long long)bn * (nb - 1) >= a.Cout) continue;  // the same tiles with fewer blocks
+        const double mma = (double)nc * 9 * (kc / 16) * mt * std::max(0.5 * bn, 53.0 + 0.25 * bn);
+        for (int occ = 1; occ <= 2; ++occ) {
+          int accs = 4, tcols = 32;
+          if (accs * mt * bn * occ > 512) accs = 2;
+          while (tcols < accs * mt * bn) tcols *= 2;
+          if (occ * tcols > 512) continue;
+          const size_t budget = (size_t)kSmemPerSm / occ - 1024;
+          for (int res = 1; res >= 0; --res) {
+            int st = 0;
+            for (int k = PC_MAX_STAGES; k >= 2 && !st; --k)
+              if (pers_smem_bytes(a.Cin, kc, h.P, rb, bn, k, res) <= std::min(budget, (size_t)kMaxSmemOptin)) st = k;
+            if (!st) continue;
+            const int grid = (int)std::max<long long>(1, std::min<long long>(ntiles, (long long)sms * occ / nb));
+            const double per_cta = (double)((ntiles + grid - 1) / grid);
+            const double rounds = std::ceil((double)grid * nb / ((double)sms * occ));
+            const double epi = 5100.0 + 1090.0 * mt * bn / 32.0;
+            const double share = std::min<double>(occ, std::ceil((double)grid * nb / sms));
+            const double work = std::max(share * std::max(mma, nc * box), mma + 800.0 * nc);
+            const double cost =
+                rounds * (2400.0 + box + epi + (per_cta > 1.0 ? per_cta * std::max(work, 0.5 * epi) : work));
+            if (best.kc == 0 || cost < best_cost) {
+              best_cost = cost;
+              best.g = PersArgs{h.P, h.TW, h.strips, h.tiles, rb, (int)ntiles, (int)ntiles / grid, (int)ntiles % grid, bn, st, res, accs, tcols, group};
+              best.kc = kc;
+              best.mt = mt;
+              best.nb = nb;
+              best.grid = grid;
+              best.smem = pers_smem_bytes(a.Cin, kc, h.P, rb, bn, st, res);
+            }
+          }
+        }
+      }
+    }
+  }
+  return best;
+}
+
+// The search above costs ~10 us of host time, so the last shapes' plans are
+// kept (a plan depends on the shape alone), at most 256 of them.
+PersPlan pers_plan(const ConvArgs &a, int sms) {
+  static std::mutex mu;
+  static std::map<std::array<int, 6>, PersPlan> plans;
+  const std::array<int, 6> key{a.B, a.H, a.W, a.Cin, a.Cout, sms};
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = plans.find(key);
+  if (it != plans.end()) return it->second;
+  if (plans.size() >= 256) plans.clear();
+  return plans[key] = pers_search(a, sms);
+}
+
+template <int KC, int MT>
+cudaError_t launch_pers(cudaStream_t s, const ConvArgs &a, const PersPlan &p, const CUtensorMap &xm,
+                        const CUtensorMap &wm, int *err) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_conv_fwd_pers<KC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemOptin);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  k_conv_fwd_pers<KC, MT><<<dim3((unsigned)p.grid, (unsigned)p.nb), PC_THREADS, p.smem, s>>>(xm, wm, a, p.g, err);
+  return cudaGetLastError();
+}
+
 cudaError_t conv_fwd(cudaStream_t s, const bf16 *x, const bf16 *w, const float *bias, bf16 *y,
                      float *yf, int B, int H, int W, int Cin, int Cout, int ldy, int yoff,
                      int relu) {
@@ -272,6 +393,16 @@ cudaError_t conv_fwd(cudaStream_t s, const bf16 *x, const bf16 *w, const float *
   if (g_conv_kernel == 2 && Cin % 16 == 0) {
     int *err = tc_error_flag();
     if (!err) return cudaErrorMemoryAllocation;
+    if (!g_tc_bn && !g_halo_kc && !g_halo_mt) {  // no tile of the caller's own
+      const PersPlan p = pers_plan(a, sm_count());
+      CUtensorMap xm, wm;
+      if (p.kc && nhwc_map(&xm, x, B, H, W, Cin, p.kc, p.g.P, p.g.RB) && weight_map(&wm, w, Cout, Cin, p.kc, p.g.BN)) {
+        const bool two = p.mt == 2;
+        if (p.kc == 64) return two ? launch_pers<64, 2>(s, a, p, xm, wm, err) : launch_pers<64, 1>(s, a, p, xm, wm, err);
+        if (p.kc == 32) return two ? launch_pers<32, 2>(s, a, p, xm, wm, err) : launch_pers<32, 1>(s, a, p, xm, wm, err);
+        return two ? launch_pers<16, 2>(s, a, p, xm, wm, err) : launch_pers<16, 1>(s, a, p, xm, wm, err);
+      }
+    }
     int bn, kc, mt;
     halo_tile(a, bn, kc, mt);
     switch (bn) {

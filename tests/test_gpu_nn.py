@@ -245,3 +245,32 @@ def test_unet_gradients_odd_widths_match_oracle(channels, B, H, W):
             assert np.dot(a, b) / (np.linalg.norm(a) * np.linalg.norm(b)) > 0.98, (name, k)
             assert _rel(a, b) < (4e-2 if name == "head" else 0.2), (name, k)
     net.close()
+
+
+@pytest.mark.parametrize("B,H,W,Cin,Cout", [
+    (1, 1, 1, 16, 16), (1, 3, 2, 32, 16),      # fewer positions than one tile
+    (2, 33, 64, 48, 80), (1, 20, 65, 80, 24),  # one strip, one strip and a column; Cout no multiple of 16
+    (2, 130, 130, 16, 32), (1, 9, 200, 64, 96),
+    (2, 64, 64, 128, 128), (1, 64, 64, 384, 128),  # 32-channel groups, weights streamed
+    (1, 8, 9, 16, 200), (1, 16, 16, 32, 1024)])    # several blocks of output channels
+def test_persistent_convolution_equals_halo_kernel(B, H, W, Cin, Cout):
+    """The persistent forward kernel (the default) sums in the halo kernel's
+    order: the same bits, with every output form."""
+    import torch
+    from paper_2108_08591_gb300 import _lib, conv3x3_bf16, conv_timeout_flag
+    lib = _lib.load()
+    g = torch.Generator(device="cuda").manual_seed(B + H + W + Cin + Cout)
+    x = torch.randn(B, H, W, Cin, device="cuda", generator=g).bfloat16()
+    w = (torch.randn(Cout, 3, 3, Cin, device="cuda", generator=g) / (3 * Cin ** 0.5)).bfloat16()
+    b = torch.randn(Cout, device="cuda", generator=g)
+    kc = 32 if Cin % 32 == 0 and Cin >= 128 and W <= 64 else 16
+    try:
+        for bias, relu, f32 in ((None, False, True), (b, True, False), (b, False, True)):
+            got = conv3x3_bf16(x, w, bias, relu=relu, out_fp32=f32)
+            assert lib.mdf_nn_set_halo_tile(1, kc) == 0  # a tile of the caller's own: the halo kernel
+            ref = conv3x3_bf16(x, w, bias, relu=relu, out_fp32=f32)
+            assert lib.mdf_nn_set_halo_tile(0, 0) == 0
+            assert torch.equal(got, ref), (bias is None, relu, f32)
+    finally:
+        lib.mdf_nn_set_halo_tile(0, 0)
+    assert conv_timeout_flag() == 0
