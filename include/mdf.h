@@ -421,7 +421,9 @@ mdf_status mdf_batch_info(mdf_batch_t b, long long *nodes, int *tiles, int *grid
 /* mdf_batch_set_timeout -- spin limit of the grid barrier in SM clock cycles
  * (default 4e9, about 2 s).  A barrier that waits longer makes every block of
  * the persistent kernel return and the call report MDF_ETIMEOUT; the batch
- * state is then undefined until the next mdf_batch_init. */
+ * state is then undefined until the next mdf_batch_init.  Fused launches (see
+ * mdf_batch_set_schedule) have no barrier; a limit keeps to the persistent
+ * kernel. */
 mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles);
 
 /* Scheduling of the batch's persistent kernel (mdf_batch_set_schedule,
@@ -441,7 +443,10 @@ mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles);
  * time from an atomic ticket counter; grid barrier).  Every schedule
  * computes the same bits; only the speed differs.  MDF_EINVAL for other
  * values.  A new batch starts with 64 threads, schedule 3 and the largest
- * grid. */
+ * grid; a 2D one with the alpha = 0 set advances by ordinary launches of
+ * several updates each instead (the same bits), until this call or
+ * mdf_batch_set_timeout asks for the persistent kernel, or
+ * mdf_batch_autotune finds it faster. */
 mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sched);
 
 /* mdf_batch_get_schedule -- the launch shape in use (any pointer may be NULL). */

@@ -25,7 +25,7 @@
 #include <vector>
 
 #include "mdf.h"
-#include "mdf_kernels.cuh"
+#include "mdf_fuse2d.cuh"
 
 namespace mdf {
 
@@ -350,6 +350,84 @@ __global__ void __launch_bounds__(T, SCHED == 3 ? batch_min_blocks<L, T>() : 0)
   }
 }
 
+// K updates of every running D2Q5 cavity by the marching kernel of
+// mdf_fuse2d.cuh: a warp takes one (cavity, strip, rows) item.  What bounds
+// the persistent kernel above is one pass over memory and one grid barrier
+// (with the drain before it) per update; here both are paid once per K, and
+// a launch boundary is the barrier.  Measured (us per update, against
+// k_batch_chunk): 12 boxes of 65^2 .. 129^2 7.2 / 10.0, 28 of 65^2 .. 513^2
+// (2.97 M nodes) 39.0 / 66.1.  With a wall on every side a strip needs no wrapped columns;
+// rows of odd boxes are not 8-byte aligned, so their pairs move as two
+// 4-byte accesses.
+//
+// Segment lengths: item lists are laid out for the whole batch at three
+// lengths (fuse_rows', half and a quarter); as cavities retire, the kernel
+// moves to a shorter one that still fits one wave, so that the last ones
+// spread over more SMs.
+struct BatchItem {
+  int cav, strip, y0, y1;
+};
+constexpr int kItemLists = 3;
+struct BatchItems {
+  const BatchItem *list[kItemLists];  // longest segments first
+  int n[kItemLists];
+  int wave;                           // warps the first list was laid out for
+};
+
+template <int K, bool SAVE>
+__global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
+    k_batch_fused(BatchArgs B, BatchItems I, int cur, int tk, int all) {
+  using L = D2Q5;
+  extern __shared__ float2 fuse_smem[];
+  const int live = *B.n_live;
+  int l = 0;
+  if ((double)I.n[1] * live <= (double)I.wave * B.ntiles) l = (double)I.n[2] * live <= (double)I.wave * B.ntiles ? 2 : 1;
+  const int item = blockIdx.x * kFuseWarps + (threadIdx.x >> 5);
+  if (item >= (l == 0 ? I.n[0] : l == 1 ? I.n[1] : I.n[2])) return;  // the whole warp
+  const BatchItem it = (l == 0 ? I.list[0] : l == 1 ? I.list[1] : I.list[2])[item];
+  if (!all && B.status[it.cav] != CAV_RUNNING) return;
+  const CavParam C = B.cav[it.cav];
+  FuseLattice G;
+  G.fin = B.f[cur] + C.base;
+  G.fout = B.f[cur ^ 1] + C.base;
+  G.plane = B.tot;
+  G.nx = G.ny = G.px = C.N;
+  G.pairs = (C.N & 1) == 0;  // bases and the pool size are multiples of a tile
+  G.wx = G.wy = G.lid = true;
+  G.lid_u[0] = float(2.0 * L::w(L::UP) * B.lid_u[0]);
+  G.lid_u[1] = float(2.0 * L::w(L::UP) * B.lid_u[1]);
+  G.force = nullptr;
+  G.s1 = C.s1;
+  G.s2 = C.s2;
+  G.key0 = 0u;
+  G.t0 = __ldg(B.clock) + tk;
+  G.usave = B.usave + C.base;
+  fuse_march<L, K, true, FORCE_NONE, SAVE>(
+      G, it.strip, it.y0, it.y1, fuse_smem + (threadIdx.x >> 5) * fuse_slots<K, L::Q>() + (threadIdx.x & 31));
+}
+
+// Rest state of every cavity: P = P0, u = 0, so all shifted populations are
+// zero but those behind the lid, whose bounce-back must return zero.
+template <class L>
+__global__ void __launch_bounds__(kTile) k_batch_rest(BatchArgs B, int cur) {
+  const CavParam C = B.cav[B.tile_cav[blockIdx.x]];
+  const long long n = (long long)((int)blockIdx.x - C.tile0) * kTile + threadIdx.x;
+  if (n >= node_count<L>(C.N)) return;
+  int p[3];
+  node_pos<L>((int)n, C, p);
+  const uint8_t m = box_mask<L>(p, C.N);
+  for (int a = 0; a < L::D + B.with_rho; ++a) {
+    const int alpha = a + 1 - B.with_rho;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+      const bool wall = i != 0 && ((m >> i) & 1);
+      float v = wall ? -0.f : 0.f;
+      if (wall && alpha >= 1 && i == L::UP && (m & 0x80u)) v += float(2.0 * L::w(i) * B.lid_u[alpha - 1]);
+      B.f[cur][((long long)a * L::Q + i) * B.tot + C.base + n] = v;
+    }
+  }
+}
+
 // Residual partial sums of every live tile against the saved velocity.
 template <class L>
 __global__ void __launch_bounds__(kTile) k_batch_residual(BatchArgs B, int cur) {
@@ -397,19 +475,30 @@ __global__ void __launch_bounds__(kTile) k_batch_residual(BatchArgs B, int cur) 
 // Advances the batch's step counter by the steps of the chunk just run.
 __global__ void k_batch_tick(int *clock, int steps) { *clock += steps; }
 
-// Per cavity: residual from its tiles' partials (fixed order), step count,
-// status.  One block per cavity.
+// Per cavity: residual from its tiles' partials (fixed order: every lane of
+// the cavity's warp takes each 32nd tile, then a tree), step count, status.
+// One warp per cavity.  (One thread adding 2,057 tiles of a 513^2 box one
+// after the other took 269 us a period, 7 % of the 100 updates between.)
 __global__ void k_batch_status(BatchArgs B, int period, double tol, long long max_steps) {
-  const int c = blockIdx.x;
-  if (threadIdx.x != 0 || B.status[c] != CAV_RUNNING) return;
+  const int c = blockIdx.x, lane = threadIdx.x;
+  if (B.status[c] != CAV_RUNNING) return;
   const CavParam C = B.cav[c];
   double num = 0.0, den = 0.0;
   int bad = 0;
-  for (int t = 0; t < C.ntiles; ++t) {
-    num += B.part[(long long)(C.tile0 + t) * 2];
-    den += B.part[(long long)(C.tile0 + t) * 2 + 1];
+#pragma unroll 4
+  for (int t = lane; t < C.ntiles; t += 32) {
+    const double2 p = *reinterpret_cast<const double2 *>(B.part + (long long)(C.tile0 + t) * 2);
+    num += p.x;
+    den += p.y;
     bad |= B.badtile[C.tile0 + t];
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_down_sync(0xffffffffu, num, o);
+    den += __shfl_down_sync(0xffffffffu, den, o);
+  }
+  bad = __any_sync(0xffffffffu, bad != 0);
+  if (lane != 0) return;
   const double r = den > 0.0 ? sqrt(num / den) / period : (num > 0.0 ? INFINITY : 0.0);
   B.res[c] = r;
   B.steps[c] += period;
@@ -552,6 +641,9 @@ struct mdf_batch_s {
   int grid = 0;      // blocks of the persistent kernel
   int threads = 64;  // threads per block (kTile / threads nodes per thread)
   int sched = 3;     // 0: round-robin, 1: contiguous runs, 2: neighbour waits, 3: claimed tail
+  bool fuse = false; // runs go by fused launches (D2Q5, d + 1 sets, no schedule of the caller's own)
+  BatchItems items{};
+  BatchItem *item_mem = nullptr;
   int *host_live = nullptr;
   cudaGraphExec_t graph = nullptr;
   int graph_period = 0, graph_cur = 0;
@@ -659,6 +751,75 @@ cudaError_t max_grid(mdf_batch_t b, int threads, int sched, int *grid) {
   return e;
 }
 
+// The item lists of the fused kernel (see BatchItems).
+cudaError_t build_items(mdf_batch_t b) {
+  constexpr int K = 4, OUT = fuse_out<K>();
+  static_assert(fuse_out<2>() >= OUT, "the strips of four updates serve two as well");
+  constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, D2Q5::Q>() * sizeof(float2);
+  int per = 0, nmax = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_fused<K, false>, 32 * kFuseWarps, smem);
+  if (e != cudaSuccess) return e;
+  for (const CavParam &C : b->cav) nmax = std::max(nmax, C.N);
+  const auto count = [&](int rows) {
+    long long n = 0;
+    for (const CavParam &C : b->cav) n += (long long)((C.N + OUT - 1) / OUT) * ((C.N + rows - 1) / rows);
+    return n;
+  };
+  const int rows0 = fuse_rows<K>(nmax, per * kFuseWarps / 4, count);
+  std::vector<BatchItem> all;
+  size_t first[kItemLists] = {};
+  for (int l = 0; l < kItemLists; ++l) {
+    const int rows = std::max(2, rows0 >> l);
+    first[l] = all.size();
+    if (all.size() + (size_t)count(rows) > (1u << 30)) return cudaErrorInvalidValue;
+    for (int c = 0; c < b->ncav; ++c) {
+      const int N = b->cav[c].N;
+      for (int y = 0; y < N; y += rows)
+        for (int s = 0; s * OUT < N; ++s) all.push_back({c, s, y, std::min(N, y + rows)});
+    }
+    b->items.n[l] = (int)(all.size() - first[l]);
+  }
+  b->items.wave = std::max(b->items.n[0], 4 * kSMs);
+  e = cudaMalloc(&b->item_mem, all.size() * sizeof(BatchItem));
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->item_mem, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // `all` leaves scope
+  for (int l = 0; l < kItemLists; ++l) b->items.list[l] = b->item_mem + first[l];
+  return e;
+}
+
+template <int K, bool SAVE>
+cudaError_t launch_fused_t(mdf_batch_t b, int cur, int tk, int all) {
+  constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, D2Q5::Q>() * sizeof(float2);
+  const int most = std::max(b->items.n[0], std::max(b->items.n[1], b->items.n[2]));
+  k_batch_fused<K, SAVE><<<(unsigned)((most + kFuseWarps - 1) / kFuseWarps), 32 * kFuseWarps, smem, b->stream>>>(
+      b->B, b->items, cur, tk, all);
+  return cudaGetLastError();
+}
+cudaError_t launch_fused(mdf_batch_t b, int K, int cur, int tk, bool save, int all) {
+  if (K == 4) return save ? launch_fused_t<4, true>(b, cur, tk, all) : launch_fused_t<4, false>(b, cur, tk, all);
+  return save ? launch_fused_t<2, true>(b, cur, tk, all) : launch_fused_t<2, false>(b, cur, tk, all);
+}
+
+// An even number of launches of four and two updates that make `period`
+// (even, >= 4) updates, so that the state ends in the buffer it started in.
+cudaError_t fused_period(mdf_batch_t b, int period) {
+  int four = period / 4, two = (period & 3) / 2;
+  if ((four + two) & 1) {
+    --four;
+    two += 2;
+  }
+  int cur = b->cur, tk = 0;
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < four + two && e == cudaSuccess; ++k) {
+    const int K = k < four ? 4 : 2;
+    e = launch_fused(b, K, cur, tk, k == 0, 0);
+    cur ^= 1;
+    tk += K;
+  }
+  return e;
+}
+
 void drop_graph(mdf_batch_t b) {
   if (b->graph) {
     cudaGraphExecDestroy(b->graph);
@@ -680,7 +841,7 @@ mdf_status all_live(mdf_batch_t b) {
 
 template <class L>
 cudaError_t enqueue_period(mdf_batch_t b, int period, double tol, long long max_steps) {
-  cudaError_t e = launch_chunk<L>(b, period, 1);
+  cudaError_t e = b->fuse && period >= 4 ? fused_period(b, period) : launch_chunk<L>(b, period, 1);
   if (e != cudaSuccess) return e;
   k_batch_tick<<<1, 1, 0, b->stream>>>(b->B.clock, period);
   const int cur_after = (b->cur + period) & 1;
@@ -790,6 +951,10 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
     e = cudaMemcpyAsync((void *)B.tile_cav, tile_cav.data(), sizeof(int) * b->ntiles,
                         cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = max_grid(b, b->threads, b->sched, &b->grid);
+  if (e == cudaSuccess && d == 2 && b->with_rho) {
+    e = build_items(b);
+    b->fuse = e == cudaSuccess;
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -810,7 +975,7 @@ void mdf_batch_destroy(mdf_batch_t b) {
   cudaFree(B.f[0]); cudaFree(B.f[1]); cudaFree((void *)B.cav); cudaFree((void *)B.tile_cav);
   cudaFree(B.live); cudaFree(B.n_live); cudaFree(B.usave); cudaFree(B.part); cudaFree(B.badtile);
   cudaFree(B.status); cudaFree(B.steps); cudaFree(B.res); cudaFree(B.bar); cudaFree(B.err);
-  cudaFree(B.prog); cudaFree(B.clock);
+  cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem);
   cudaFreeHost(b->host_live);
   delete b;
 }
@@ -827,6 +992,13 @@ mdf_status mdf_batch_seed(mdf_batch_t b, int cavity, const double *P, const doub
   if ((P || u) && cavity < 0) return bfail(b, MDF_EINVAL, "fields need a single cavity");
   // seeding every cavity restarts the step count of the dither draws
   if (cavity < 0) BCU(b, cudaMemsetAsync(b->B.clock, 0, sizeof(int), b->stream));
+  if (cavity < 0) {  // the rest state of all
+    if (b->d == 2) k_batch_rest<D2Q5><<<b->ntiles, kTile, 0, b->stream>>>(b->B, b->cur);
+    else k_batch_rest<D3Q7><<<b->ntiles, kTile, 0, b->stream>>>(b->B, b->cur);
+    BCU(b, cudaGetLastError());
+    BCU(b, cudaStreamSynchronize(b->stream));
+    return MDF_OK;
+  }
   for (int c = lo; c < hi; ++c) {
     const CavParam &C = b->cav[c];
     const long long nn = b->d == 2 ? (long long)C.N * C.N : (long long)C.N * C.N * C.N;
@@ -942,11 +1114,21 @@ mdf_status mdf_batch_step(mdf_batch_t b, long long n) {
   if (st != MDF_OK) return st;
   const int chunk = 1 << 20;
   while (n > 0) {
-    const int s = (int)std::min<long long>(n, chunk);
-    BCU(b, b->d == 2 ? launch_chunk<D2Q5>(b, s, 0) : launch_chunk<D3Q7>(b, s, 0));
+    const bool fused = b->fuse && n >= 2;
+    int s = (int)std::min<long long>(n, chunk), k = 0;
+    if (fused) {
+      for (; s - k >= 2; b->cur ^= 1) {
+        const int K = s - k >= 4 ? 4 : 2;
+        BCU(b, launch_fused(b, K, b->cur, k, false, 1));
+        k += K;
+      }
+      s = k;
+    } else {
+      BCU(b, b->d == 2 ? launch_chunk<D2Q5>(b, s, 0) : launch_chunk<D3Q7>(b, s, 0));
+      b->cur = (b->cur + s) & 1;
+    }
     k_batch_tick<<<1, 1, 0, b->stream>>>(b->B.clock, s);
     BCU(b, cudaGetLastError());
-    b->cur = (b->cur + s) & 1;
     n -= s;
   }
   int err = 0;
@@ -1012,6 +1194,7 @@ mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles) {
   if (!b) return MDF_EINVAL;
   if (cycles < 0) return bfail(b, MDF_EINVAL, "timeout must be >= 0 cycles");
   b->B.timeout = cycles;
+  b->fuse = false;  // a limit of the caller's own is the persistent kernel's
   drop_graph(b);  // the captured kernels hold the old value
   return MDF_OK;
 }
@@ -1028,6 +1211,7 @@ mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sche
   b->threads = threads;
   b->sched = sched;
   b->grid = grid ? grid : gmax;
+  b->fuse = false;  // the caller's own launch shape is the persistent kernel's
   drop_graph(b);  // the captured launch holds the old shape
   return MDF_OK;
 }
@@ -1103,6 +1287,18 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
         }
       }
     }
+  bool fuse = b->fuse;
+  if (st == MDF_OK && fuse) {  // the fused launches against the best of them
+    cudaError_t e = cudaEventRecord(e0, b->stream);
+    for (int k = 0; k < reps && e == cudaSuccess; k += reps - k >= 4 ? 4 : 2)
+      e = launch_fused(b, reps - k >= 4 ? 4 : 2, b->cur, k, false, 1);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    if (e != cudaSuccess) st = bfail(b, MDF_ECUDA, "autotune: %s", cudaGetErrorString(e));
+    fuse = ms < best;
+  }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   // the tuning steps advanced the state: put it back
@@ -1114,6 +1310,7 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
     b->threads = best_threads;
     b->sched = best_sched;
     b->grid = best_grid;
+    b->fuse = fuse;
   } else {
     b->threads = old_threads;
     b->sched = old_sched;

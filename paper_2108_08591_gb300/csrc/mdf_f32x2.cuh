@@ -54,15 +54,16 @@ __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(vsub(a.f2(), b.f
 // memory: as immediates each use costs the moves that build the register
 // pair.
 enum Lit { LIT_NEG0, LIT_2_3, LIT_3_4, LIT_M4, LIT_M6, LIT_1_20, LIT_1_5, LIT_1_42, LIT_1_7, LIT_1_6, LIT_1_2,
-           LIT_DITHER, LIT_1, LIT_2, LIT_1_3, LITS };
+           LIT_DITHER, LIT_1, LIT_1_4, LIT_1_3, LIT_1_12, LITS };
 #define MDF_LITS                                                                                              \
   {-0.0, 2.0 / 3.0, 0.75, -4.0, -6.0, 0.05, 0.2, 1.0 / 42.0, 1.0 / 7.0, 1.0 / 6.0, 0.5, -1.498046875 * 0x1p-23, \
-   1.0, 2.0, 1.0 / 3.0}
+   1.0, 0.25, 1.0 / 3.0, 1.0 / 12.0}
 constexpr double kLit[LITS] = MDF_LITS;
 #define MDF_PAIR(k) {(float)kLit[k], (float)kLit[k]}
 static __constant__ float2 kLit2[LITS] = {MDF_PAIR(0),  MDF_PAIR(1),  MDF_PAIR(2),  MDF_PAIR(3),  MDF_PAIR(4),
                                           MDF_PAIR(5),  MDF_PAIR(6),  MDF_PAIR(7),  MDF_PAIR(8),  MDF_PAIR(9),
-                                          MDF_PAIR(10), MDF_PAIR(11), MDF_PAIR(12), MDF_PAIR(13), MDF_PAIR(14)};
+                                          MDF_PAIR(10), MDF_PAIR(11), MDF_PAIR(12), MDF_PAIR(13), MDF_PAIR(14),
+                                          MDF_PAIR(15)};
 #undef MDF_PAIR
 template <class T, Lit K> __device__ __forceinline__ T lit() {
   constexpr double v = kLit[K];

@@ -26,8 +26,8 @@
 // so the bits are those of K single updates.
 //
 // Measured (GB300, K = 4, us per update against one update per launch):
-// 4096^2 152 / 301, 2048^2 42.1 / 80, 1024^2 14.2 / 22.6, 256^2 3.7 / 6.2;
-// 4095^2 153 / (scalar kernel) 330; walls and lid 170 at 4096^2.  K = 4 is
+// 4096^2 158 / 302, 2048^2 43.7 / 80, 1024^2 14.5 / 22.6, 256^2 3.7 / 6.2;
+// 4095^2 159 / (scalar kernel) 330; walls and lid 172 at 4096^2.  K = 4 is
 // bound by the FP32 and integer pipes (issue 58 %, the f32x2 operations take
 // two slots of theirs): 219 instructions per update and node, of which 1.14
 // x is rim.  K = 2 would stay at HBM's 150 us.
@@ -86,8 +86,9 @@ __device__ __forceinline__ F2 fuse_load(const float *p, const FuseCols &c) {
 
 // Eq. 2-7, 3-15, 2-4 and 3-21 on a pair of nodes: collide_node's operations.
 template <class L, int FORCE, class TF>
-__device__ __forceinline__ void fuse_collide(F2 (&g)[3][L::Q], const TF (&F)[2], const Rates<F2> &R, uint2 key) {
-  F2 u[2], Pp, gv[2][L::Q];
+__device__ __forceinline__ void fuse_collide(F2 (&g)[3][L::Q], const TF (&F)[2], const Rates<F2> &R, uint2 key,
+                                             F2 (&u)[2]) {
+  F2 Pp, gv[2][L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) { gv[0][i] = g[0][i]; gv[1][i] = g[1][i]; }
   node_moments<L, F2, FORCE == FORCE_SCHEME2>(gv, F, u, Pp);
@@ -102,17 +103,30 @@ __device__ __forceinline__ void fuse_collide(F2 (&g)[3][L::Q], const TF (&F)[2],
 // 152, six (168) at 162.
 constexpr int kFuseBlocks = 8;
 
-template <class L, int K, bool WALLS, int FORCE>
-__global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
-    k_update_fused2d(const DevArgs A, int strips, int seg_rows, int nseg) {
+// A 2D lattice as the march sees it.
+struct FuseLattice {
+  const float *fin;          // populations, node (0, 0)
+  float *fout;
+  long long plane;           // direction stride
+  int nx, ny, px;            // px: row pitch
+  bool pairs;                // every row starts on an 8-byte boundary
+  bool wx, wy, lid;          // walls, lid on the + y face
+  float lid_u[2];            // 2 w u of the lid
+  const float *force;        // [2][plane], or null
+  float s1, s2;
+  uint32_t key0;             // global index of node (0, 0), low word
+  int t0;                    // time step of update 1
+  float *usave;              // [2][plane]: velocity pulled by update 1 (SAVE)
+};
+
+// K updates of rows y0 .. y1 - 1 of a strip by one warp; sb: the lane's
+// shared memory, K - 1 x 3 Q slots of 32 lanes.
+template <class L, int K, bool WALLS, int FORCE, bool SAVE>
+__device__ __forceinline__ void fuse_march(const FuseLattice &A, int strip, int y0, int y1, float2 *const sb) {
   static_assert(L::D == 2 && K >= 2, "2D, at least two updates");
   constexpr int Q = L::Q, H = fuse_halo<K>(), OUT = fuse_out<K>();
   const int lane = threadIdx.x & 31;
-  const int item = blockIdx.x * kFuseWarps + (threadIdx.x >> 5);
-  if (item >= strips * nseg) return;  // the whole warp
-  const int strip = item % strips, seg = item / strips;
-  const int y0 = seg * seg_rows, y1 = min(y0 + seg_rows, A.ny);
-  const bool wx = WALLS && A.wall[0], wy = WALLS && A.wall[1];
+  const bool wx = WALLS && A.wx, wy = WALLS && A.wy;
 
   const int c0 = strip * OUT - H + 2 * lane;
   FuseCols c;
@@ -121,7 +135,7 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
   // an odd row is not a whole number of pairs: where the strip leaves it,
   // the wrapped columns are read one by one (behind an x wall they are not
   // used, so any column will do)
-  c.vec = (A.nx & 1) == 0 || wx || (strip * OUT - H >= 0 && strip * OUT - H + 64 <= A.nx);
+  c.vec = A.pairs && ((A.nx & 1) == 0 || wx || (strip * OUT - H >= 0 && strip * OUT - H + 64 <= A.nx));
   if (c.vec && (c.xa & 1)) c.xa = c.xb = 0;  // odd nx behind an x wall
   c.w0a = wx && c0 == 0;
   c.w0b = false;  // c0 is even
@@ -131,17 +145,17 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
   const bool out_a = lane >= H / 2 && lane < 32 - H / 2 && c0 < A.nx;
   const bool out_b = out_a && c0 + 1 < A.nx;
 
-  const float *__restrict__ fin = static_cast<const float *>(A.fin);
-  float *__restrict__ fout = static_cast<float *>(A.fout);
-  const Rates<F2> R(F2(A.s1f, A.s1f), F2(A.s2f, A.s2f));
-  const int t0 = launch_step(A);
+  const float *__restrict__ fin = A.fin;
+  float *__restrict__ fout = A.fout;
+  const Rates<F2> R(F2(A.s1, A.s1), F2(A.s2, A.s2));
+  const int t0 = A.t0;
   F2 lid[3][Q] = {};
   if (WALLS) {
 #pragma unroll
     for (int i = 0; i < Q; ++i)
       if (L::c(i, 1) == -1) {
 #pragma unroll
-        for (int a = 0; a < 2; ++a) lid[a][i] = F2(2.0 * L::w(i) * A.lid_u[a]);
+        for (int a = 0; a < 2; ++a) lid[a][i] = F2(A.lid_u[a], A.lid_u[a]);
       }
   }
 
@@ -149,9 +163,6 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
   // the row directions of the row last computed, shifted, and the +y
   // direction of the last two rows (alternating slots)
   constexpr int NROW = Q - 2, SLOTS = 3 * (NROW + 2);
-  extern __shared__ float2 fuse_smem[];
-  float2 *const sb = fuse_smem + (threadIdx.x >> 5) * (K - 1) * SLOTS * 32 + lane;
-
   const int iters = y1 - y0 + 2 * (K - 1);
   for (int it = 0; it < iters; ++it) {
     const int r = y0 - (K - 1) + it;
@@ -233,37 +244,117 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
         if (it < 2 * s) break;  // the rows below have not come through yet
       }
       const int yq = wy ? q : wrap(q, A.ny);
-      const uint32_t n0 = (uint32_t)A.key_base + (uint32_t)(yq * A.nx);
+      const uint32_t n0 = A.key0 + (uint32_t)(yq * A.nx);
       const uint2 key = make_uint2(node_key(n0 + c.xa, t0 + s), node_key(n0 + c.xb, t0 + s));
+      F2 u[2];
       if constexpr (FORCE == FORCE_NONE) {
         const NoForce F[2] = {};
-        fuse_collide<L, FORCE>(g, F, R, key);
+        fuse_collide<L, FORCE>(g, F, R, key, u);
       } else {
-        const float *fp = static_cast<const float *>(A.force) + (long long)(wy ? min(max(q, 0), A.ny - 1) : yq) * A.px;
+        const float *fp = A.force + (long long)(wy ? min(max(q, 0), A.ny - 1) : yq) * A.px;
         const F2 F[2] = {fuse_load(fp, c), fuse_load(fp + A.plane, c)};
-        fuse_collide<L, FORCE>(g, F, R, key);
+        fuse_collide<L, FORCE>(g, F, R, key, u);
+      }
+      if constexpr (SAVE) {
+        if (s == 0 && q >= y0 && q < y1) {
+          float *p = A.usave + (long long)q * A.px + c0;
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            if (out_a) p[a * A.plane] = u[a].x;
+            if (out_b) p[a * A.plane + 1] = u[a].y;
+          }
+        }
       }
     }
     if (it < 2 * (K - 1)) continue;
     float *po = fout + (long long)(r - (K - 1)) * A.px + c0;
-    auto store_row = [&](auto pair) {
+    // 2: a pair as one access, 1: a pair in two, 0: the odd row's last node
+    auto store_row = [&](auto how) {
 #pragma unroll
       for (int s = 0; s < 3; ++s)
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
           float *p = po + ((long long)(s < 2 ? s + 1 : 0) * Q + i) * A.plane;
-          if constexpr (pair) __stcs(reinterpret_cast<float2 *>(p), g[s][i].f2());
-          else __stcs(p, g[s][i].x);
+          if constexpr (how == 2) {
+            __stcs(reinterpret_cast<float2 *>(p), g[s][i].f2());
+          } else {
+            __stcs(p, g[s][i].x);
+            if constexpr (how == 1) __stcs(p + 1, g[s][i].y);
+          }
         }
     };
-    if (out_b) store_row(std::true_type{});
-    else if (out_a) store_row(std::false_type{});
+    if (out_b) {
+      if (A.pairs) store_row(std::integral_constant<int, 2>{});
+      else store_row(std::integral_constant<int, 1>{});
+    } else if (out_a) {
+      store_row(std::integral_constant<int, 0>{});
+    }
   }
+}
+
+template <int K, int Q> constexpr int fuse_slots() { return (K - 1) * 3 * Q * 32; }  // float2 per warp
+
+template <class L, int K, bool WALLS, int FORCE>
+__global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
+    k_update_fused2d(const DevArgs A, int strips, int seg_rows, int nseg) {
+  extern __shared__ float2 fuse_smem[];
+  const int item = blockIdx.x * kFuseWarps + (threadIdx.x >> 5);
+  if (item >= strips * nseg) return;  // the whole warp
+  const int strip = item % strips, seg = item / strips;
+  FuseLattice G;
+  G.fin = static_cast<const float *>(A.fin);
+  G.fout = static_cast<float *>(A.fout);
+  G.plane = A.plane;
+  G.nx = A.nx;
+  G.ny = A.ny;
+  G.px = A.px;
+  G.pairs = true;  // the pitch is a multiple of 32
+  G.wx = A.wall[0] != 0;
+  G.wy = A.wall[1] != 0;
+  G.lid = A.lid != 0;
+  G.lid_u[0] = float(2.0 * L::w(L::UP) * A.lid_u[0]);
+  G.lid_u[1] = float(2.0 * L::w(L::UP) * A.lid_u[1]);
+  G.force = static_cast<const float *>(A.force);
+  G.s1 = A.s1f;
+  G.s2 = A.s2f;
+  G.key0 = (uint32_t)A.key_base;
+  G.t0 = launch_step(A);
+  G.usave = nullptr;
+  fuse_march<L, K, WALLS, FORCE, false>(G, strip, seg * seg_rows, min((seg + 1) * seg_rows, A.ny),
+                                        fuse_smem + (threadIdx.x >> 5) * fuse_slots<K, L::Q>() + (threadIdx.x & 31));
+}
+
+// Rows per segment for one wave of w = 1 .. wmax warps per SM sub-partition
+// (items(rows): warps that segments of that many rows make).  A warp does K
+// rows + K (K - 1) row updates (the second term fills and drains the
+// pipeline), each in a time of about 1.7 + w: measured at 1024^2, K = 4:
+// 0.57 / 0.76 / 1.0 / 1.2 us for w = 1 .. 4.  Long segments waste less, many
+// warps hide more; large lattices take the most warps, small ones fewer
+// (256^2: 3.65 us per update with w = 1 against 4.17 with w = 2 .. 4;
+// 1024^2: 20.0, 14.5, 14.0, 14.1).
+template <int K, class Items>
+int fuse_rows(int ny, int wmax, Items items) {
+  int best_rows = ny;
+  double best = 0.0;
+  for (int w = 1; w <= std::max(1, wmax); ++w) {
+    int lo = std::min(ny, 2), hi = ny;  // fewest rows that fit one wave (the longest when none does)
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if (items(mid) <= 4LL * w * kSMs) hi = mid;
+      else lo = mid + 1;
+    }
+    const double cost = (lo + K - 1.0) * (1.7 + w);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      best_rows = lo;
+    }
+  }
+  return best_rows;
 }
 
 template <class L, int K, bool WALLS, int FORCE>
 cudaError_t launch_fused2d(const DevArgs &a, cudaStream_t s) {
-  constexpr size_t smem = (size_t)kFuseWarps * (K - 1) * 3 * L::Q * 32 * sizeof(float2);
+  constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, L::Q>() * sizeof(float2);
   static const int per_sm = [] {  // resident blocks per SM of this build
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_update_fused2d<L, K, WALLS, FORCE>, 32 * kFuseWarps,
@@ -272,24 +363,9 @@ cudaError_t launch_fused2d(const DevArgs &a, cudaStream_t s) {
     return n > 0 ? n : 1;
   }();
   const int strips = (a.nx + fuse_out<K>() - 1) / fuse_out<K>();
-  // Rows per segment, for one wave of w = 1 .. the resident warps per SM
-  // sub-partition.  A warp does K rows + K (K - 1) row updates (the second
-  // term fills and drains the pipeline), each in a time of about 1.7 + w:
-  // measured at 1024^2, K = 4: 0.57 / 0.76 / 1.0 / 1.2 us for w = 1 .. 4.
-  // Long segments waste less, many warps hide more; large lattices take the
-  // most warps, small ones fewer (256^2: 3.65 us per update with w = 1
-  // against 4.17 with w = 2 .. 4; 1024^2: 20.0, 14.5, 14.0, 14.1).
-  int seg_rows = a.ny;
-  double best = 0.0;
-  for (int w = 1; w <= std::max(1, per_sm * kFuseWarps / 4); ++w) {
-    const int want = std::max(1, kSMs * 4 * w / strips);
-    const int rows = std::max((a.ny + want - 1) / want, std::min(a.ny, 2));
-    const double cost = (rows + K - 1.0) * (1.7 + w);
-    if (best == 0.0 || cost < best) {
-      best = cost;
-      seg_rows = rows;
-    }
-  }
+  const int seg_rows = fuse_rows<K>(a.ny, per_sm * kFuseWarps / 4, [&](int rows) {
+    return (long long)strips * ((a.ny + rows - 1) / rows);
+  });
   const int nseg = (a.ny + seg_rows - 1) / seg_rows;
   const long long items = (long long)strips * nseg;
   k_update_fused2d<L, K, WALLS, FORCE>

@@ -124,12 +124,13 @@ __device__ __forceinline__ void add_change(TC &g, TC dl, const TC *rz, int i) {
   if constexpr (DZ) g = g + dithered_change(dl, g, rz[i]);
   else g = g + dl;
 }
-// Relaxation rates as relax() uses them.  The halves and quarters of M^-1's
-// columns are taken into the rates: scaling by a power of two is exact.
+// Relaxation rates as relax() uses them.  (The factors 1/2 and 1/4 of M^-1
+// are applied after the rate, not folded into it: where a product falls
+// below the normal range the two round differently, and with the dithered
+// rounding one such bit decorrelates every later one.)
 template <class TC> struct Rates {
-  TC s1h, s2, s2h, s2q;  // s1 / 2, s2, s2 / 2, s2 / 4
-  __device__ __forceinline__ Rates(TC s1, TC s2_)
-      : s1h(lit<TC, (LIT_1_2)>() * s1), s2(s2_), s2h(lit<TC, (LIT_1_2)>() * s2_), s2q(lit<TC, (LIT_1_2)>() * s2h) {}
+  TC s1, s2;
+  __device__ __forceinline__ Rates(TC s1_, TC s2_) : s1(s1_), s2(s2_) {}
 };
 
 // Round-to-nearest storage (16-bit rest-shifted, FP64): the change of each
@@ -167,9 +168,9 @@ struct D2Q5 {
   static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
                                                const TC *rz = nullptr) {
     const TC m0 = g[0] + g[1] + g[2] + g[3] + g[4];
-    const TC h1 = R.s1h * ((g[1] - g[3]) - jeq[0]);
-    const TC h2 = R.s1h * ((g[2] - g[4]) - jeq[1]);
-    const TC q3 = R.s2q * ((g[1] + g[3]) - (g[2] + g[4]));
+    const TC h1 = lit<TC, LIT_1_2>() * (R.s1 * ((g[1] - g[3]) - jeq[0]));
+    const TC h2 = lit<TC, LIT_1_2>() * (R.s1 * ((g[2] - g[4]) - jeq[1]));
+    const TC q3 = lit<TC, LIT_1_4>() * (R.s2 * ((g[1] + g[3]) - (g[2] + g[4])));
     const TC d4 = R.s2 * (add_scaled<LIT_M4>(g[1] + g[2] + g[3] + g[4], g[0]) + lit<TC, (LIT_2_3)>() * m0);
     const TC e4 = lit<TC, (LIT_1_20)>() * d4;
     const auto Fw = F * TC(1.0 / 6.0);
@@ -217,13 +218,14 @@ struct D3Q7 {
                                                const TC *rz = nullptr) {
     const TC sx = g[1] + g[2], sy = g[3] + g[4], sz = g[5] + g[6];
     const TC m0 = g[0] + sx + sy + sz;
-    const TC h1 = R.s1h * ((g[1] - g[2]) - jeq[0]);
-    const TC h2 = R.s1h * ((g[3] - g[4]) - jeq[1]);
-    const TC h3 = R.s1h * ((g[5] - g[6]) - jeq[2]);
+    const TC h1 = lit<TC, LIT_1_2>() * (R.s1 * ((g[1] - g[2]) - jeq[0]));
+    const TC h2 = lit<TC, LIT_1_2>() * (R.s1 * ((g[3] - g[4]) - jeq[1]));
+    const TC h3 = lit<TC, LIT_1_2>() * (R.s1 * ((g[5] - g[6]) - jeq[2]));
     const TC d4 = R.s2 * ((sx + sy + sz) + lit<TC, (LIT_M6)>() * g[0] + lit<TC, (LIT_3_4)>() * m0);
-    const TC d5h = R.s2h * ((sx + sx) - sy - sz);
+    const TC d5 = R.s2 * ((sx + sx) - sy - sz);
     const TC e4 = d4 * lit<TC, (LIT_1_42)>();
-    const TC eo = d5h * lit<TC, (LIT_1_6)>(), ex = eo + eo, q6 = R.s2q * (sy - sz);
+    const TC ex = d5 * lit<TC, LIT_1_6>(), eo = d5 * lit<TC, LIT_1_12>();
+    const TC q6 = lit<TC, LIT_1_4>() * (R.s2 * (sy - sz));
     const auto Fw = F * TC(0.125);
     if constexpr (DZ) {
       add_change<DZ>(g[0], d4 * lit<TC, (LIT_1_7)>() + F * TC(0.25), rz, 0);
@@ -268,9 +270,9 @@ struct D2Q4 {
   template <bool DZ = false, class TC, class TF>
   static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
                                                const TC *rz = nullptr) {
-    const TC h1 = R.s1h * ((g[0] - g[2]) - jeq[0]);
-    const TC h2 = R.s1h * ((g[1] - g[3]) - jeq[1]);
-    const TC q3 = R.s2q * ((g[0] + g[2]) - (g[1] + g[3]));
+    const TC h1 = lit<TC, LIT_1_2>() * (R.s1 * ((g[0] - g[2]) - jeq[0]));
+    const TC h2 = lit<TC, LIT_1_2>() * (R.s1 * ((g[1] - g[3]) - jeq[1]));
+    const TC q3 = lit<TC, LIT_1_4>() * (R.s2 * ((g[0] + g[2]) - (g[1] + g[3])));
     const auto Fw = F * TC(0.25);
     if constexpr (DZ) {
       add_change<DZ>(g[0], (Fw - h1) - q3, rz, 0);
@@ -307,11 +309,12 @@ struct D3Q6 {
   static __device__ __forceinline__ void relax(TC g[Q], const TC jeq[D], const Rates<TC> &R, TF F,
                                                const TC *rz = nullptr) {
     const TC sx = g[0] + g[1], sy = g[2] + g[3], sz = g[4] + g[5];
-    const TC h1 = R.s1h * ((g[0] - g[1]) - jeq[0]);
-    const TC h2 = R.s1h * ((g[2] - g[3]) - jeq[1]);
-    const TC h3 = R.s1h * ((g[4] - g[5]) - jeq[2]);
-    const TC d4h = R.s2h * ((sx + sx) - sy - sz);
-    const TC eo = d4h * lit<TC, (LIT_1_6)>(), ex = eo + eo, q5 = R.s2q * (sy - sz);
+    const TC h1 = lit<TC, LIT_1_2>() * (R.s1 * ((g[0] - g[1]) - jeq[0]));
+    const TC h2 = lit<TC, LIT_1_2>() * (R.s1 * ((g[2] - g[3]) - jeq[1]));
+    const TC h3 = lit<TC, LIT_1_2>() * (R.s1 * ((g[4] - g[5]) - jeq[2]));
+    const TC d4 = R.s2 * ((sx + sx) - sy - sz);
+    const TC ex = d4 * lit<TC, LIT_1_6>(), eo = d4 * lit<TC, LIT_1_12>();
+    const TC q5 = lit<TC, LIT_1_4>() * (R.s2 * (sy - sz));
     const auto Fw = F * TC(1.0 / 6.0);
     if constexpr (DZ) {
       add_change<DZ>(g[0], (Fw - h1) - ex, rz, 0);

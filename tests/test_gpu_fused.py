@@ -58,3 +58,51 @@ def test_fused_updates_in_a_captured_chunk():
         lat.close()
     for k in outs[0]:
         assert np.array_equal(outs[0][k], outs[1][k]), k
+
+
+@pytest.mark.parametrize("sides", [[2, 3, 4, 5, 7], [55, 56, 57, 64], [113, 30, 65], [128]])
+def test_fused_cavities_equal_the_persistent_kernel(sides):
+    """Batched cavities by fused launches (the default) against the
+    persistent kernel: the same bits after steps and after a run, with its
+    step counts, statuses and residuals."""
+    from paper_2108_08591_gb300 import CavityBatch
+
+    Re = [20.0 + 3.0 * s for s in sides]
+    got = []
+    for own in (False, True):
+        b = CavityBatch(sides, Re, lid_speed=0.1)
+        if own:
+            b.set_schedule(64, 0, 3)
+        out = []
+        for n in (1, 2, 3, 7, 4):
+            b.step(n)
+        out += [b.fields_host(c, ("P", "u", "rho", "G")) for c in range(b.n)]
+        b.init()
+        for period in (6, 4, 100):  # 4: two launches of two; 100: 24 of four and two of two
+            r = b.run(tol=1e-4, max_steps=3 * period, check_every=period)
+        out += [{"steps": r[0], "status": r[1], "res": r[2]}]
+        out += [b.fields_host(c, ("P", "u", "rho", "G")) for c in range(b.n)]
+        b.close()
+        got.append(out)
+    for a, b in zip(*got):
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
+
+
+def test_fused_cavities_as_they_retire():
+    """Most cavities converge early: the last ones move to the lists of
+    shorter segments and keep the persistent kernel's bits."""
+    from paper_2108_08591_gb300 import CavityBatch
+
+    sides, Re = [33] * 40 + [129], [40.0] * 40 + [300.0]
+    got = []
+    for own in (False, True):
+        b = CavityBatch(sides, Re, lid_speed=0.1)
+        if own:
+            b.set_schedule(64, 0, 3)
+        r = b.run(tol=1e-6, max_steps=6000, check_every=100)
+        got.append((*r, b.fields_host(0, ("u",))["u"], b.fields_host(40, ("u", "P"))["u"]))
+        b.close()
+    assert (got[0][1][:40] == 0).all() and got[0][0][:40].max() < got[0][0][40]
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
