@@ -614,49 +614,73 @@ __device__ __forceinline__ void init_moments(const DevArgs &A, long long N, long
   M[L::D + 1] = 0.f;
 }
 
+// First pass: the node moments (u, P', rho' = 0), each seed narrowed once.
+template <class L>
+__global__ void __launch_bounds__(kMaxBlock) k_init_eq_moments(const DevArgs A) {
+  constexpr int D = L::D;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= A.nx) return;
+  const long long row = (long long)blockIdx.z * A.ny + blockIdx.y;
+  const long long N = (long long)A.nx * A.ny * A.nz;
+  float M0[D + 2];
+  init_moments<L>(A, N, row * A.nx + x, M0);
+  const int K = moment_slots(D, A.with_rho);
+  float *mout = static_cast<float *>(A.mout) + eq_off(A.px, row, x, K);
+#pragma unroll
+  for (int k = 0; k < D + 2; ++k)
+    if (k < K) mout[k * kEqTile] = M0[k];
+}
+
+// Second pass: the stored parts, from this node's moments and those of the
+// nodes its populations come to.  (In one pass every (set, direction) read
+// and narrowed its neighbour's FP64 seed again, 15 or 28 times a node: 1007
+// us at 2050 x 1998, now 154 for both.)
 template <class L, class TS, bool WALLS>
 __global__ void __launch_bounds__(kMaxBlock) k_init_eq(const DevArgs A) {
   constexpr int D = L::D, Q = L::Q;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= A.nx) return;
   const int y = blockIdx.y, z = blockIdx.z;
-  const long long idx = ((long long)z * A.ny + y) * A.px + x;
-  const long long N = (long long)A.nx * A.ny * A.nz;
-  const long long n = ((long long)z * A.ny + y) * A.nx + x;
-  const uint8_t m = WALLS ? A.mask[idx] : uint8_t(0);
-  float M0[D + 2];
-  init_moments<L>(A, N, n, M0);
-  float *mout = static_cast<float *>(A.mout);
-  const int K = moment_slots(D, A.with_rho);
   const long long row = (long long)z * A.ny + y;
-  for (int k = 0; k < K; ++k) mout[eq_off(A.px, row, x, K) + k * kEqTile] = M0[k];
-  TS *fout = static_cast<TS *>(A.fout);
-  const int nsets = D + A.with_rho;
-  TS *fn = fout + eq_off(A.px, row, x, nsets * Q);
-  for (int a = 0; a < nsets; ++a) {
-    const int alpha = a + 1 - A.with_rho;
+  const long long idx = row * A.px + x, N = (long long)A.nx * A.ny * A.nz, n = row * A.nx + x;
+  const uint8_t m = WALLS ? A.mask[idx] : uint8_t(0);
+  const int K = moment_slots(D, A.with_rho), NK = (D + A.with_rho) * Q;
+  const float *mom = static_cast<const float *>(A.mout);
+  auto moments = [&](long long r, int xx, float (&M)[D + 2]) {
+    const float *p = mom + eq_off(A.px, r, xx, K);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
+    for (int k = 0; k < D + 2; ++k) M[k] = k < K ? p[k * kEqTile] : 0.f;
+  };
+  float M0[D + 2];
+  moments(row, x, M0);
+  TS *fn = static_cast<TS *>(A.fout) + eq_off(A.px, row, x, NK);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const bool wall = WALLS && i != 0 && ((m >> i) & 1);
+    const int tx = wrap(x + L::c(i, 0), A.nx), ty = wrap(y + L::c(i, 1), A.ny);
+    const int tz = D == 3 ? wrap(z + L::c(i, 2), A.nz) : z;
+    const long long trow = (long long)tz * A.ny + ty;
+    float Mt[D + 2];
+    if (!wall) moments(trow, tx, Mt);
+#pragma unroll
+    for (int alpha = 0; alpha <= D; ++alpha) {
+      if (alpha == 0 && !A.with_rho) continue;
       float target;
       const bool half = A.scheme2 && alpha >= 1;
       const float *Fa = half ? static_cast<const float *>(A.force) + (alpha - 1) * A.plane : nullptr;
-      if (WALLS && i != 0 && ((m >> i) & 1)) {
+      if (wall) {
         target = -geq_m<L>(alpha, L::opp(i), M0);
         if (A.Gin) target -= narrow_f64(fne_at<L>(A, N, n, alpha, L::opp(i)));
-        if (alpha >= 1 && i == L::UP && (m & 0x80u)) target += float(2.0 * L::w(i) * A.lid_u[alpha - 1]);
+        if (alpha >= 1 && i == L::UP && (m & 0x80u))
+          target += float(2.0 * L::w(i) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
         if (half) target += float(0.5 * L::w(i)) * __ldg(Fa + idx);  // negated by the bounce-back
       } else {
-        const int tx = wrap(x + L::c(i, 0), A.nx);
-        const int ty = wrap(y + L::c(i, 1), A.ny);
-        const int tz = D == 3 ? wrap(z + L::c(i, 2), A.nz) : z;
-        const long long tn = ((long long)tz * A.ny + ty) * A.nx + tx;
-        float Mt[D + 2];
-        init_moments<L>(A, N, tn, Mt);
         target = geq_m<L>(alpha, i, Mt);
-        if (A.Gin) target += narrow_f64(fne_at<L>(A, N, tn, alpha, i));
-        if (half) target -= float(0.5 * L::w(i)) * __ldg(Fa + ((long long)tz * A.ny + ty) * A.px + tx);
+        if (A.Gin) target += narrow_f64(fne_at<L>(A, N, trow * A.nx + tx, alpha, i));
+        if (half) target -= float(0.5 * L::w(i)) * __ldg(Fa + trow * A.px + tx);
       }
-      Codec<TS>::store(fn + (a * Q + i) * kEqTile, (target - geq_m<L>(alpha, i, M0)) * EqScale<TS>::s);
+      Codec<TS>::store(fn + ((alpha - 1 + A.with_rho) * Q + i) * kEqTile,
+                       (target - geq_m<L>(alpha, i, M0)) * EqScale<TS>::s);
     }
   }
 }
