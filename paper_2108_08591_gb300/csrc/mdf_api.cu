@@ -233,6 +233,7 @@ mdf_status one_update(mdf_t h, int mode, const mdf_fields_t *out) {
 // the lattice has such a kernel, else 1.
 int fused_updates(const mdf_t h, long long n) {
   if (!h->fuse || n < 2) return 1;
+  if (h->d == 3) return 2;
   const int K = n >= 4 && h->ny >= 4 ? 4 : 2;
   return h->ny >= K ? K : 1;
 }
@@ -414,8 +415,8 @@ mdf_status mdf_create(mdf_t *out, const mdf_grid *g, int d, const mdf_rates *r,
   h->block = opts.block ? opts.block
                         : fit_block(row_threads, h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage));
   // a caller's own launch shape is that of the one-update kernel
-  h->fuse = lattice_launch(d, q)->fused && h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
-            !opts.block && h->plane < (1LL << 31) - 64;
+  h->fuse = h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
+            !opts.block && h->plane < (1LL << 31) - 64 && (d == 2 || fuse3_pays(h->nx, h->ny, h->nz, h->walls));
 
   const size_t pb = h->pop_bytes();
   cudaError_t e = cudaMalloc(&h->buf[0], pb);

@@ -38,7 +38,6 @@
 namespace mdf {
 
 constexpr int kFuseWarps = 2;  // independent warps per block
-constexpr int kSMs = 152;      // of a GB300
 template <int K> constexpr int fuse_halo() { return (K + 1) / 2 * 2; }
 template <int K> constexpr int fuse_out() { return 64 - 2 * fuse_halo<K>(); }
 

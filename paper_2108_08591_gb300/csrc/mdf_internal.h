@@ -89,11 +89,41 @@ cudaError_t launch_reduce_d3q6(int storage, bool walls, int kind, const DevArgs 
 cudaError_t launch_mask_d3q6(const int wall[3], int lid, const DevArgs &a, uint8_t *mask,
                              cudaStream_t s);
 
-// K = 2 or 4 updates in one launch (FP32, two buffers, all d + 1 sets, ny >= K).
+// Two fused updates of a 3D lattice (mdf_fuse3d.cuh): planes per z segment,
+// and whether they pay.  Blocks of kFuse3Rows rows (two fewer stored) x 64
+// columns (60 stored), two per SM; a block takes about 5.2 us per plane and
+// 1.2 planes to fill, the single update 34.5 ps per node (1.25 x that with
+// walls, whose mask it reads): 128^3 (92 us fused, 74 single) and smaller
+// boxes stay single, 60 x 60 x 200 (31 / 37) and 190 x 202 x 178 (242 / 255)
+// go fused.
+constexpr int kSMs = 152;  // of a GB300
+constexpr int kFuse3Rows = 8;
+struct Fuse3Plan {
+  int seg;
+  double us;  // of two updates
+};
+inline Fuse3Plan fuse3_plan(int nx, int ny, int nz) {
+  const long long tiles = (long long)((nx + 59) / 60) * ((ny + kFuse3Rows - 3) / (kFuse3Rows - 2));
+  Fuse3Plan p{nz, 0.0};
+  for (int k = nz; k >= 1; k = k > 1 ? (k * 15 / 16 > 1 ? k * 15 / 16 : 1) : 0) {
+    const long long blocks = tiles * ((nz + k - 1) / k);
+    const double us = 5.2 * (double)((blocks + 2 * kSMs - 1) / (2 * kSMs)) * (k + 1.2);
+    if (p.us == 0.0 || us < p.us) p = {k, us};
+  }
+  return p;
+}
+inline bool fuse3_pays(int nx, int ny, int nz, bool walls) {
+  return fuse3_plan(nx, ny, nz).us < 69e-6 * (walls ? 1.25 : 1.0) * nx * (double)ny * nz;
+}
+
+// K updates in one launch (FP32, two buffers, all d + 1 sets): 2 or 4 in 2D
+// (ny >= K), 2 in 3D.
 cudaError_t launch_fused_d2q5(int K, bool walls, const DevArgs &a, cudaStream_t s);
 cudaError_t launch_fused_d2q4(int K, bool walls, const DevArgs &a, cudaStream_t s);
+cudaError_t launch_fused_d3q7(int K, bool walls, const DevArgs &a, cudaStream_t s);
+cudaError_t launch_fused_d3q6(int K, bool walls, const DevArgs &a, cudaStream_t s);
 
-// The launchers of one lattice (fused: null where it is not built).
+// The launchers of one lattice.
 struct LatticeLaunch {
   cudaError_t (*update)(int storage, int mode, bool walls, const DevArgs &a, cudaStream_t s);
   cudaError_t (*init)(int storage, bool walls, const DevArgs &a, cudaStream_t s);
@@ -104,10 +134,12 @@ struct LatticeLaunch {
 inline const LatticeLaunch *lattice_launch(int d, int q) {
   static const LatticeLaunch d2q5{launch_update_d2q5, launch_init_d2q5, launch_reduce_d2q5, launch_mask_d2q5,
                                   launch_fused_d2q5};
-  static const LatticeLaunch d3q7{launch_update_d3q7, launch_init_d3q7, launch_reduce_d3q7, launch_mask_d3q7, nullptr};
+  static const LatticeLaunch d3q7{launch_update_d3q7, launch_init_d3q7, launch_reduce_d3q7, launch_mask_d3q7,
+                                  launch_fused_d3q7};
   static const LatticeLaunch d2q4{launch_update_d2q4, launch_init_d2q4, launch_reduce_d2q4, launch_mask_d2q4,
                                   launch_fused_d2q4};
-  static const LatticeLaunch d3q6{launch_update_d3q6, launch_init_d3q6, launch_reduce_d3q6, launch_mask_d3q6, nullptr};
+  static const LatticeLaunch d3q6{launch_update_d3q6, launch_init_d3q6, launch_reduce_d3q6, launch_mask_d3q6,
+                                  launch_fused_d3q6};
   if (d == 2) return q == 5 ? &d2q5 : q == 4 ? &d2q4 : nullptr;
   if (d == 3) return q == 7 ? &d3q7 : q == 6 ? &d3q6 : nullptr;
   return nullptr;

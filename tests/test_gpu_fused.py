@@ -41,6 +41,41 @@ def test_fused_updates_equal_single_updates(shape, forcing, q):
             assert torch.equal(a, b), (wall, lid)
 
 
+# boxes large enough for the fused kernel to be chosen (single updates below);
+# tile edges (60 of 64 columns, 6 of 8 rows), odd rows, one segment and many
+SHAPES3 = [(119, 61, 151), (59, 59, 211), (300, 120, 25), (960, 6, 200)]
+BCS3 = [((0, 0, 0), False), ((1, 0, 0), False), ((0, 1, 0), False), ((0, 0, 1), True), ((1, 1, 1), True)]
+
+
+@pytest.mark.parametrize("q", [0, 6])
+@pytest.mark.parametrize("forcing", ["none", "eq3-21", "scheme2"])
+@pytest.mark.parametrize("shape", SHAPES3)
+def test_fused_3d_updates_equal_single_updates(shape, forcing, q):
+    import torch
+    from paper_2108_08591_gb300 import Lattice
+
+    N = int(np.prod(shape))
+    rng = np.random.default_rng([*shape, q])
+    P = 1.0 + 1e-3 * rng.standard_normal(N)
+    u, F = 0.01 * rng.standard_normal((3, N)), 1e-5 * rng.standard_normal((3, N))
+    for wall, lid in BCS3:
+        outs = []
+        for kw in ({}, {"vx": 1}):
+            lat = Lattice(shape, s1=1.8, s2=1.0, wall=wall, lid=lid, lid_u=(0.05, 0.01, 0.0), q=q, **kw)
+            if forcing != "none":
+                lat.set_forcing(forcing)
+                lat.set_force(F)
+            lat.init(P, u)
+            got = []
+            for n in (2, 3, 1, 6):
+                lat.step(n)
+                got += [v.clone() for v in lat.fields(("P", "u", "rho", "G")).values()]
+            lat.close()
+            outs.append(got)
+        for a, b in zip(*outs):
+            assert torch.equal(a, b), (wall, lid)
+
+
 def test_fused_updates_in_a_captured_chunk():
     import torch
     from paper_2108_08591_gb300 import Lattice
