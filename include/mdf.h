@@ -90,9 +90,10 @@ typedef struct {
                                 16-bit, FP64) or 2 (FP32, *EQ);
                                 mdf_info reports the width in use.  A width that
                                 does not divide nx falls back to 1.  With vx = 0
-                                and block = 0, runs of updates of a 2D FP32 lattice
-                                go several to a launch (the same bits); a width or
-                                block of the caller's own keeps to one. */
+                                and block = 0, runs of updates of an FP32 lattice go
+                                several to a launch where that is faster (the same
+                                bits); a width or block of the caller's own keeps
+                                to one. */
     int block;               /* threads per block of the update kernel: 0 = tuned
                                 default, else a multiple of 32 in [32, 256] */
     int q;                   /* directions per set: 0 = D2Q5 / D3Q7 (default), 4 = D2Q4,

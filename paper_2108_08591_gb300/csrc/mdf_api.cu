@@ -125,6 +125,7 @@ struct mdf_s {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // chunk starting from buffer 0 / 1
   void *buf[2] = {nullptr, nullptr};
   bool fuse = false;     // runs of updates go by fused launches (see mdf_create)
+  int resident = 0;      // runs of at least this many updates keep the lattice on chip (0: none)
   bool inplace = false;  // one buffer, AA pattern (buf[1] unused)
   int parity = 0;        // AA layout of the current state: 0 even, 1 odd
   void *mac[2] = {nullptr, nullptr};  // node moments of equilibrium-shifted storage
@@ -285,6 +286,14 @@ mdf_status build_graph(mdf_t h, int which) {
 }
 
 mdf_status run_steps(mdf_t h, long long n) {
+  while (h->resident && n >= h->resident) {
+    const int s = (int)std::min<long long>(n, 1 << 14);
+    CU(h, launch_set_clock(h->clock, (int)h->step, h->stream));
+    CU(h, lattice_launch(h->d, h->q)->resident(s, h->walls, base_args(h), h->stream));
+    std::swap(h->cur, h->nxt);
+    h->step += s;
+    n -= s;
+  }
   // Graph chunks only on a real (non-legacy) stream: capture is not allowed
   // on the legacy default stream.
   const bool use_graph = h->stream != nullptr && n >= kGraphChunk;
@@ -417,6 +426,8 @@ mdf_status mdf_create(mdf_t *out, const mdf_grid *g, int d, const mdf_rates *r,
   // a caller's own launch shape is that of the one-update kernel
   h->fuse = h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
             !opts.block && h->plane < (1LL << 31) - 64 && (d == 2 || fuse3_pays(h->nx, h->ny, h->nz, h->walls));
+  if (d == 2 && h->storage == MDF_F32 && !h->inplace && !opts.vx && !opts.block)
+    h->resident = lattice_launch(d, q)->resident_steps(h->nx, h->ny, h->nsets);
 
   const size_t pb = h->pop_bytes();
   cudaError_t e = cudaMalloc(&h->buf[0], pb);

@@ -291,15 +291,9 @@ __device__ __forceinline__ void fuse_march(const FuseLattice &A, int strip, int 
   }
 }
 
-template <int K, int Q> constexpr int fuse_slots() { return (K - 1) * 3 * Q * 32; }  // float2 per warp
-
-template <class L, int K, bool WALLS, int FORCE>
-__global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
-    k_update_fused2d(const DevArgs A, int strips, int seg_rows, int nseg) {
-  extern __shared__ float2 fuse_smem[];
-  const int item = blockIdx.x * kFuseWarps + (threadIdx.x >> 5);
-  if (item >= strips * nseg) return;  // the whole warp
-  const int strip = item % strips, seg = item / strips;
+// The lattice of a launch's arguments.
+template <class L>
+__device__ __forceinline__ FuseLattice fuse_lattice(const DevArgs &A) {
   FuseLattice G;
   G.fin = static_cast<const float *>(A.fin);
   G.fout = static_cast<float *>(A.fout);
@@ -319,7 +313,19 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
   G.key0 = (uint32_t)A.key_base;
   G.t0 = launch_step(A);
   G.usave = nullptr;
-  fuse_march<L, K, WALLS, FORCE, false>(G, strip, seg * seg_rows, min((seg + 1) * seg_rows, A.ny),
+  return G;
+}
+
+template <int K, int Q> constexpr int fuse_slots() { return (K - 1) * 3 * Q * 32; }  // float2 per warp
+
+template <class L, int K, bool WALLS, int FORCE>
+__global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
+    k_update_fused2d(const DevArgs A, int strips, int seg_rows, int nseg) {
+  extern __shared__ float2 fuse_smem[];
+  const int item = blockIdx.x * kFuseWarps + (threadIdx.x >> 5);
+  if (item >= strips * nseg) return;  // the whole warp
+  const int strip = item % strips, seg = item / strips;
+  fuse_march<L, K, WALLS, FORCE, false>(fuse_lattice<L>(A), strip, seg * seg_rows, min((seg + 1) * seg_rows, A.ny),
                                         fuse_smem + (threadIdx.x >> 5) * fuse_slots<K, L::Q>() + (threadIdx.x & 31));
 }
 

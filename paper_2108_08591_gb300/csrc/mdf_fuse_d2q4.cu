@@ -1,12 +1,21 @@
-// D2Q4 instantiations of the fused multi-update kernel (a translation unit of
-// its own so that it compiles beside the lattice's other kernels).
-#include "mdf_fuse2d.cuh"
+// D2Q4 instantiations of the fused and the resident multi-update kernels (a
+// translation unit of their own, to compile beside the lattice's others).
+#include "mdf_res2d.cuh"
 
 namespace mdf {
 
 cudaError_t launch_fused_d2q4(int K, bool walls, const DevArgs &a, cudaStream_t s) {
   return K == 4 ? update_fused2d<D2Q4, 4>(walls, a, s)
        : K == 2 ? update_fused2d<D2Q4, 2>(walls, a, s) : cudaErrorInvalidValue;
+}
+
+cudaError_t launch_resident_d2q4(int steps, bool walls, const DevArgs &a, cudaStream_t s) {
+  return update_resident2d<D2Q4>(walls, a, steps, s);
+}
+int resident_steps_d2q4(int nx, int ny, int nsets) {
+  static const bool available = res_available(k_resident2d<D2Q4, true, FORCE_EQ321, true>);
+  const ResShape r = res_shape(nx, ny, D2Q4::Q, nsets);
+  return available && r.ctas ? res_min_steps(r.rows * nx) : 0;
 }
 
 }  // namespace mdf

@@ -123,23 +123,33 @@ cudaError_t launch_fused_d2q4(int K, bool walls, const DevArgs &a, cudaStream_t 
 cudaError_t launch_fused_d3q7(int K, bool walls, const DevArgs &a, cudaStream_t s);
 cudaError_t launch_fused_d3q6(int K, bool walls, const DevArgs &a, cudaStream_t s);
 
-// The launchers of one lattice.
+// `steps` updates (at most 16384) of a small 2D FP32 lattice in one launch of
+// one thread-block cluster (mdf_res2d.cuh), and the fewest updates for which
+// that pays (0: it does not fit).
+cudaError_t launch_resident_d2q5(int steps, bool walls, const DevArgs &a, cudaStream_t s);
+cudaError_t launch_resident_d2q4(int steps, bool walls, const DevArgs &a, cudaStream_t s);
+int resident_steps_d2q5(int nx, int ny, int nsets);
+int resident_steps_d2q4(int nx, int ny, int nsets);
+
+// The launchers of one lattice (resident: 2D only).
 struct LatticeLaunch {
   cudaError_t (*update)(int storage, int mode, bool walls, const DevArgs &a, cudaStream_t s);
   cudaError_t (*init)(int storage, bool walls, const DevArgs &a, cudaStream_t s);
   cudaError_t (*reduce)(int storage, bool walls, int kind, const DevArgs &a, cudaStream_t s);
   cudaError_t (*mask)(const int wall[3], int lid, const DevArgs &a, uint8_t *mask, cudaStream_t s);
   cudaError_t (*fused)(int K, bool walls, const DevArgs &a, cudaStream_t s);
+  cudaError_t (*resident)(int steps, bool walls, const DevArgs &a, cudaStream_t s);
+  int (*resident_steps)(int nx, int ny, int nsets);
 };
 inline const LatticeLaunch *lattice_launch(int d, int q) {
   static const LatticeLaunch d2q5{launch_update_d2q5, launch_init_d2q5, launch_reduce_d2q5, launch_mask_d2q5,
-                                  launch_fused_d2q5};
+                                  launch_fused_d2q5, launch_resident_d2q5, resident_steps_d2q5};
   static const LatticeLaunch d3q7{launch_update_d3q7, launch_init_d3q7, launch_reduce_d3q7, launch_mask_d3q7,
-                                  launch_fused_d3q7};
+                                  launch_fused_d3q7, nullptr, nullptr};
   static const LatticeLaunch d2q4{launch_update_d2q4, launch_init_d2q4, launch_reduce_d2q4, launch_mask_d2q4,
-                                  launch_fused_d2q4};
+                                  launch_fused_d2q4, launch_resident_d2q4, resident_steps_d2q4};
   static const LatticeLaunch d3q6{launch_update_d3q6, launch_init_d3q6, launch_reduce_d3q6, launch_mask_d3q6,
-                                  launch_fused_d3q6};
+                                  launch_fused_d3q6, nullptr, nullptr};
   if (d == 2) return q == 5 ? &d2q5 : q == 4 ? &d2q4 : nullptr;
   if (d == 3) return q == 7 ? &d3q7 : q == 6 ? &d3q6 : nullptr;
   return nullptr;

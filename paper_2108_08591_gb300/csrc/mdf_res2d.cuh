@@ -1,0 +1,319 @@
+// A small 2D FP32 lattice kept on chip for all updates of a call.
+//
+// What bounds a small lattice is not memory but the launch and the latency
+// of each update (64^2: 4.2 us per update in launches of one, 3.1 in fused
+// launches of four, for 0.03 us of arithmetic).  Here one thread-block cluster
+// holds the whole lattice: each CTA a run of rows, all populations in two
+// buffers of its shared memory.  An update pulls from one buffer, its edge
+// rows from the neighbouring CTAs' shared memory, collides and stores into
+// the other; one cluster barrier ends it.  Global memory is read once before
+// the first update and written once after the last.
+//
+// The arithmetic per node is the scalar kernel's (collide_node with the same
+// dither draws), so the bits are those of single updates.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "mdf_fuse2d.cuh"
+
+namespace mdf {
+
+constexpr int kResThreads = 512;
+constexpr int kResMaxCluster = 16;                // needs the non-portable size
+// Most nodes of a CTA.  Up to here the resident kernel is the faster one: us
+// per update against fused launches, 16^2 0.62 / 3.1, 64^2 0.75 / 3.1 (and
+// 4.2 in launches of one), 96^2 1.47 / 3.1, 128^2 (1024 nodes a CTA) 1.98 /
+// 3.2; at 144^2 (1296) 2.95 / 3.2 and at 170^2 3.37 / 3.4 it no longer pays
+// for its start.
+constexpr int kResMaxNodes = 1200;
+constexpr size_t kResMaxSmem = 2ull * 15 * kResMaxNodes * sizeof(float);  // of a CTA
+// Fewest updates that pay for reading and writing the lattice once more than
+// a fused launch would: with two nodes a thread four (128^2: 4.7 us per update
+// against 5.8 of single ones; with two updates 8.4 against 7.5).
+inline int res_min_steps(int nodes) { return nodes > kResThreads ? 4 : 2; }
+
+// CTAs of a cluster for nx x ny nodes, and the shared memory of each; 0 when
+// it does not fit.
+struct ResShape {
+  int ctas, rows;  // rows: the most of a CTA
+  size_t smem;
+};
+inline ResShape res_shape(int nx, int ny, int q, int nsets) {
+  const int c = std::min(ny, kResMaxCluster), rows = (ny + c - 1) / c;
+  if ((long long)rows * nx > kResMaxNodes) return {0, 0, 0};
+  return {c, rows, 2ull * nsets * q * rows * (size_t)nx * sizeof(float)};
+}
+
+// Where a node's populations come from: one pointer per direction (set 0,
+// current buffer; local or of a neighbouring CTA), and what the walls make of
+// the value.
+template <int Q> struct ResPull {
+  const float *q[Q];
+  unsigned neg;  // bit i: bounced back, negated
+  bool lid;      // the -y direction bounces off the lid
+};
+
+// `steps` updates of lattice G by this thread's cluster; rcap: rows a CTA's
+// buffers are laid out for.  PAIR: a thread takes its nodes two at a time as
+// the lanes of an FP32 pair (any two: every access is a 4-byte one), for CTAs
+// with more nodes than threads, which the issue slots bound; with a node a
+// thread the latency of one collision does, and the scalar form is shorter.
+template <class L, bool WALLS, int FORCE, bool PAIR>
+__device__ __forceinline__ void res_run(const FuseLattice &G, bool with_rho, int steps, bool save, int rcap,
+                                        float *buf) {
+  namespace cg = cooperative_groups;
+  using TC = typename std::conditional<PAIR, F2, float>::type;
+  constexpr int Q = L::Q, NP = PAIR ? 2 : 1;
+  const cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int base = G.ny / C, extra = G.ny - base * C;
+  const int rows = base + (rank < extra ? 1 : 0), y0 = rank * base + min(rank, extra);
+  const int lo = rank == 0 ? C - 1 : rank - 1, hi = rank == C - 1 ? 0 : rank + 1;
+  const int lo_last = base + (lo < extra ? 1 : 0) - 1;
+  const bool wx = WALLS && G.wx, wy = WALLS && G.wy;
+  const int stride = rcap * G.nx;  // of a direction
+  const int pops = (2 + (with_rho ? 1 : 0)) * Q;
+  const int half = pops * stride;  // of a buffer
+  const int T = (int)blockDim.x, tid = (int)threadIdx.x;
+  const int nodes = rows * G.nx;
+  const int dy = T / G.nx, dx = T - dy * G.nx;  // a thread's step through its nodes
+  const int yf = tid / G.nx, xf = tid - yf * G.nx;
+  auto advance = [&](int &x, int &y) {
+    x += dx;
+    y += dy;
+    if (x >= G.nx) { x -= G.nx; ++y; }
+  };
+
+  {
+    int y = yf, x = xf;
+    for (int k = tid; k < nodes; k += T, advance(x, y)) {
+      const float *src = G.fin + (long long)(y0 + y) * G.px + x;
+      float v[3 * Q];
+#pragma unroll
+      for (int p = 0; p < 3 * Q; ++p) v[p] = p < pops ? __ldg(src + (long long)p * G.plane) : 0.f;
+#pragma unroll
+      for (int p = 0; p < 3 * Q; ++p)
+        if (p < pops) buf[p * stride + k] = v[p];
+    }
+  }
+  cl.sync();
+  const float *const rlo = cl.map_shared_rank(buf, lo) + lo_last * G.nx;  // row y0 - 1
+  const float *const rhi = cl.map_shared_rank(buf, hi);                   // row y0 + rows
+  const Rates<TC> R(TC(G.s1), TC(G.s2));
+
+  for (int s = 0; s < steps; ++s) {
+    const int b = (s & 1) * half;
+    float *const out = buf + (half - b);
+    int y = yf, x = xf;
+    for (int k = tid; k < nodes;) {
+      ResPull<Q> P[NP];
+      int kk[NP], node[NP];
+      uint32_t key[NP];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        const bool past = j > 0 && k >= nodes;  // an odd last node: its pair repeats it
+        if (past) {
+          kk[j] = kk[0];
+          node[j] = node[0];
+          key[j] = key[0];
+          P[j] = P[0];
+          continue;
+        }
+        const float *const r0 = buf + b + (k - x);
+        const float *const rm = y > 0 ? r0 - G.nx : rlo + b;
+        const float *const rp = y < rows - 1 ? r0 + G.nx : rhi + b;
+        const int xm = x == 0 ? G.nx - 1 : x - 1, xp = x == G.nx - 1 ? 0 : x + 1;
+        P[j].neg = 0u;
+        P[j].lid = false;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const float *p = (L::c(i, 1) == 1 ? rm : L::c(i, 1) == -1 ? rp : r0) +
+                           (L::c(i, 0) == 1 ? xm : L::c(i, 0) == -1 ? xp : x) + i * stride;
+          if (WALLS && moving<L>(i)) {  // the node's own opposite direction, negated
+            const bool wall = L::c(i, 0) == 1    ? wx && x == 0
+                              : L::c(i, 0) == -1 ? wx && x == G.nx - 1
+                              : L::c(i, 1) == 1  ? wy && y0 + y == 0
+                                                 : wy && y0 + y == G.ny - 1;
+            if (wall) {
+              p = r0 + x + L::opp(i) * stride;
+              P[j].neg |= 1u << i;
+              if (L::c(i, 1) == -1) P[j].lid = G.lid;
+            }
+          }
+          P[j].q[i] = p;
+        }
+        kk[j] = k;
+        node[j] = (y0 + y) * G.px + x;
+        key[j] = node_key(G.key0 + (uint32_t)((y0 + y) * G.nx + x), G.t0 + s);
+        k += T;
+        advance(x, y);
+      }
+      TC g[2][Q], h[Q];
+      auto pull = [&](TC(&v)[Q], int set, int e) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          float w[NP];
+#pragma unroll
+          for (int j = 0; j < NP; ++j) {
+            w[j] = P[j].q[i][set * Q * stride];
+            if (WALLS && moving<L>(i)) {
+              if ((P[j].neg >> i) & 1u) w[j] = -w[j];
+              if (e >= 0 && L::c(i, 1) == -1 && P[j].lid) w[j] += G.lid_u[e >= 0 ? e : 0];
+            }
+          }
+          if constexpr (PAIR) v[i] = F2(w[0], w[1]);
+          else v[i] = w[0];
+        }
+      };
+      pull(g[0], with_rho ? 1 : 0, 0);
+      pull(g[1], with_rho ? 2 : 1, 1);
+      if (with_rho) pull(h, 0, -1);
+      typename NodeKey<TC>::T kt;
+      if constexpr (PAIR) kt = make_uint2(key[0], key[1]);
+      else kt = key[0];
+      TC u[2], Pp;
+      auto relax = [&](const auto &F) {
+        node_moments<L, TC, FORCE == FORCE_SCHEME2>(g, F, u, Pp);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) relax_velocity_set<L, TC, true>(g[a], a, u, Pp, R, F[a], kt);
+      };
+      if constexpr (FORCE == FORCE_NONE) {
+        const NoForce F[2] = {};
+        relax(F);
+      } else {
+        TC F[2];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const float *f = G.force + a * G.plane;
+          if constexpr (PAIR) F[a] = F2(__ldg(f + node[0]), __ldg(f + node[1]));
+          else F[a] = __ldg(f + node[0]);
+        }
+        relax(F);
+      }
+      if (with_rho) {
+        TC r;
+        relax_rho_set<L, TC>(h, u, R, r);
+      }
+      auto lane = [](TC v, int j) {
+        if constexpr (PAIR) return j == 0 ? v.x : v.y;
+        else return v;
+      };
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        if (save && s == 0) {
+#pragma unroll
+          for (int a = 0; a < 2; ++a) G.usave[a * G.plane + node[j]] = lane(u[a], j);
+        }
+        float *o = out + kk[j];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          o[((with_rho ? 1 : 0) * Q + i) * stride] = lane(g[0][i], j);
+          o[((with_rho ? 2 : 1) * Q + i) * stride] = lane(g[1][i], j);
+          if (with_rho) o[i * stride] = lane(h[i], j);
+        }
+      }
+    }
+    cl.sync();  // every pull of this update is done, every store visible
+  }
+
+  const float *const last = buf + (steps & 1) * half;
+  int y = yf, x = xf;
+  for (int k = tid; k < nodes; k += T, advance(x, y)) {
+    float *dst = G.fout + (long long)(y0 + y) * G.px + x;
+#pragma unroll
+    for (int p = 0; p < 3 * Q; ++p)
+      if (p < pops) dst[(long long)p * G.plane] = last[p * stride + k];
+  }
+}
+
+template <class L, bool WALLS, int FORCE, bool PAIR>
+__global__ void __launch_bounds__(kResThreads) k_resident2d(const DevArgs A, int steps, int rcap) {
+  extern __shared__ float res_smem[];
+  res_run<L, WALLS, FORCE, PAIR>(fuse_lattice<L>(A), A.with_rho != 0, steps, false, rcap, res_smem);
+}
+
+// Threads of a CTA for its nodes: whole warps, a node each, or two each (as a
+// pair) beyond the limit.
+inline bool res_pairs(int nodes) { return nodes > kResThreads; }
+inline int res_threads(int nodes) {
+  const int n = res_pairs(nodes) ? (nodes + 1) / 2 : nodes;
+  return std::min(kResThreads, (n + 31) / 32 * 32);
+}
+
+template <class Kernel, class... Args>
+cudaError_t res_launch(Kernel kernel, int clusters, const ResShape &r, int threads, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * r.ctas));
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = r.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)r.ctas;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// Shared memory and cluster size beyond the defaults.
+template <class Kernel>
+cudaError_t res_configure(Kernel kernel) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
+// Whether the device schedules clusters of the largest size and memory.
+template <class Kernel>
+bool res_available(Kernel kernel) {
+  if (res_configure(kernel) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kResMaxCluster);
+  cfg.blockDim = dim3(kResThreads);
+  cfg.dynamicSmemBytes = kResMaxSmem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kResMaxCluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n > 0;
+}
+
+template <class L, bool WALLS, int FORCE, bool PAIR>
+cudaError_t launch_resident2d_p(const ResShape &r, const DevArgs &a, int steps, cudaStream_t s) {
+  static const cudaError_t set = res_configure(k_resident2d<L, WALLS, FORCE, PAIR>);
+  if (set != cudaSuccess) return set;
+  return res_launch(k_resident2d<L, WALLS, FORCE, PAIR>, 1, r, res_threads(r.rows * a.nx), s, a, steps, r.rows);
+}
+
+template <class L, bool WALLS, int FORCE>
+cudaError_t launch_resident2d(const DevArgs &a, int steps, cudaStream_t s) {
+  const ResShape r = res_shape(a.nx, a.ny, L::Q, 2 + a.with_rho);
+  if (!r.ctas) return cudaErrorInvalidValue;
+  return res_pairs(r.rows * a.nx) ? launch_resident2d_p<L, WALLS, FORCE, true>(r, a, steps, s)
+                                  : launch_resident2d_p<L, WALLS, FORCE, false>(r, a, steps, s);
+}
+
+template <class L>
+cudaError_t update_resident2d(bool walls, const DevArgs &a, int steps, cudaStream_t s) {
+  if (a.scheme2)
+    return walls ? launch_resident2d<L, true, FORCE_SCHEME2>(a, steps, s)
+                 : launch_resident2d<L, false, FORCE_SCHEME2>(a, steps, s);
+  if (a.force)
+    return walls ? launch_resident2d<L, true, FORCE_EQ321>(a, steps, s)
+                 : launch_resident2d<L, false, FORCE_EQ321>(a, steps, s);
+  return walls ? launch_resident2d<L, true, FORCE_NONE>(a, steps, s)
+               : launch_resident2d<L, false, FORCE_NONE>(a, steps, s);
+}
+
+}  // namespace mdf

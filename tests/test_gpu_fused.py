@@ -1,14 +1,17 @@
-"""Fused updates (several per launch, 2D FP32) against single updates: the
-same bits for every boundary, force scheme, width and number of steps."""
+"""Fused updates (several per pass over memory, FP32) and the resident kernel
+(small 2D lattices kept on chip) against single updates: the same bits for
+every boundary, force scheme, width and number of steps."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 
-# strip edges (56 and 60 stored columns of 64), odd and even rows, rows too
-# short for the deeper kernels, one to several strips
-SHAPES = [(2, 4), (3, 5), (24, 7), (55, 9), (56, 2), (57, 4), (60, 33), (61, 12), (64, 64), (113, 17),
-          (128, 3), (129, 130), (300, 41)]
+# kept on chip by a cluster: fewer rows than CTAs, odd rows, the largest that fit
+RESIDENT = [(2, 4), (3, 5), (24, 7), (57, 2), (64, 64), (129, 130), (300, 41), (1200, 16), (60, 319)]
+# beyond that: strip edges (56 and 60 stored columns of 64), odd and even rows,
+# rows too short for the deeper kernels, one to several strips
+SHAPES = RESIDENT + [(1201, 16), (95, 310), (2000, 2), (1999, 3), (1921, 4), (2019, 9), (55, 560), (56, 550), (57, 545), (60, 512),
+                     (61, 511), (113, 301), (128, 257), (300, 131)]
 BCS = [((0, 0), False), ((1, 0), False), ((0, 1), True), ((1, 1), True)]
 
 
@@ -32,7 +35,7 @@ def test_fused_updates_equal_single_updates(shape, forcing, q):
                 lat.set_force(F)
             lat.init(P, u)
             got = []
-            for n in (1, 2, 3, 4, 7):  # 1: single; 2, 3: one launch of two; 4, 7: of four
+            for n in (1, 2, 3, 4, 7):  # fused: 1: single; 2, 3: one launch of two; 4, 7: of four
                 lat.step(n)
                 got += [v.clone() for v in lat.fields(("P", "u", "rho", "G")).values()]
             lat.close()
@@ -76,16 +79,34 @@ def test_fused_3d_updates_equal_single_updates(shape, forcing, q):
             assert torch.equal(a, b), (wall, lid)
 
 
-def test_fused_updates_in_a_captured_chunk():
+def test_resident_updates_without_the_continuity_set():
     import torch
     from paper_2108_08591_gb300 import Lattice
 
-    P = np.ones(97 * 50)
-    u = 0.01 * np.random.default_rng(1).standard_normal((2, 97 * 50))
+    P, u = np.ones(70 * 33), 0.01 * np.random.default_rng(2).standard_normal((2, 70 * 33))
+    outs = []
+    for kw in ({}, {"vx": 1}):
+        lat = Lattice((70, 33), s1=1.7, with_rho=False, wall=(0, 1), **kw)
+        lat.init(P, u)
+        lat.step(40000)  # three launches
+        lat.step(3)
+        outs.append(lat.fields(("P", "u", "G")))
+        lat.close()
+    for k in outs[0]:
+        assert torch.equal(outs[0][k], outs[1][k]), k
+
+
+@pytest.mark.parametrize("nx", [97, 777])
+def test_fused_updates_in_a_captured_chunk(nx):
+    import torch
+    from paper_2108_08591_gb300 import Lattice
+
+    P = np.ones(nx * 50)
+    u = 0.01 * np.random.default_rng(1).standard_normal((2, nx * 50))
     outs = []
     for kw in ({}, {"vx": 1}):
         s = torch.cuda.Stream()
-        lat = Lattice((97, 50), s1=1.7, stream=s, **kw)
+        lat = Lattice((nx, 50), s1=1.7, stream=s, **kw)
         lat.init(P, u)
         lat.step(64 * 2 + 3)
         lat.step(64 + 1)
