@@ -25,7 +25,7 @@
 #include <vector>
 
 #include "mdf.h"
-#include "mdf_fuse2d.cuh"
+#include "mdf_res2d.cuh"
 
 namespace mdf {
 
@@ -406,6 +406,53 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
       G, it.strip, it.y0, it.y1, fuse_smem + (threadIdx.x >> 5) * fuse_slots<K, L::Q>() + (threadIdx.x & 31));
 }
 
+// `steps` updates of small D2Q5 cavities kept on chip (mdf_res2d.cuh): a
+// cluster of 16 CTAs holds one or more cavities, each in a team of them (seat:
+// cavity, first CTA and CTAs of its team; cavity -1: an empty seat, which only
+// joins the barriers).  What bounds a batch of a few
+// small boxes is the latency of an update: 12 boxes of 65^2 .. 129^2 took 7.2
+// us per update in fused launches, 10.0 in the persistent kernel, and take 3.5.
+struct BatchSeat {
+  int cav, first, ctas;
+};
+template <bool PAIR>
+__global__ void __launch_bounds__(kResThreads)
+    k_batch_resident(BatchArgs B, const BatchSeat *seats, int cur, int tk, int steps, int save, int all) {
+  using L = D2Q5;
+  extern __shared__ float res_smem[];
+  const BatchSeat st = seats[blockIdx.x];
+  FuseLattice G;
+  G.nx = 1;
+  G.ny = G.px = 0;
+  G.plane = B.tot;
+  G.fin = B.f[cur];
+  G.fout = B.f[cur ^ 1];
+  G.pairs = false;
+  G.wx = G.wy = G.lid = true;
+  G.lid_u[0] = float(2.0 * L::w(L::UP) * B.lid_u[0]);
+  G.lid_u[1] = float(2.0 * L::w(L::UP) * B.lid_u[1]);
+  G.force = nullptr;
+  G.s1 = G.s2 = 1.f;
+  G.key0 = 0u;
+  G.t0 = __ldg(B.clock) + tk;
+  G.usave = B.usave;
+  int rank = 0, ctas = 1, first = 0, rcap = 0;
+  if (st.cav >= 0 && (all || B.status[st.cav] == CAV_RUNNING)) {
+    const CavParam C = B.cav[st.cav];
+    G.nx = G.ny = G.px = C.N;
+    G.fin += C.base;
+    G.fout += C.base;
+    G.usave += C.base;
+    G.s1 = C.s1;
+    G.s2 = C.s2;
+    first = st.first;
+    ctas = st.ctas;
+    rank = (int)(blockIdx.x % kResMaxCluster) - first;
+    rcap = (C.N + ctas - 1) / ctas;
+  }
+  res_run<L, true, FORCE_NONE, PAIR>(G, B.with_rho != 0, steps, save != 0, rcap, res_smem, first, ctas, rank);
+}
+
 // Rest state of every cavity: P = P0, u = 0, so all shifted populations are
 // zero but those behind the lid, whose bounce-back must return zero.
 template <class L>
@@ -644,6 +691,11 @@ struct mdf_batch_s {
   bool fuse = false; // runs go by fused launches (D2Q5, d + 1 sets, no schedule of the caller's own)
   BatchItems items{};
   BatchItem *item_mem = nullptr;
+  int seats = 0;     // CTAs of the resident kernel's launch (0: the batch does not go that way)
+  bool seat_pair = false;
+  int seat_threads = 0;
+  size_t seat_smem = 0;
+  BatchSeat *seat_mem = nullptr;
   int *host_live = nullptr;
   cudaGraphExec_t graph = nullptr;
   int graph_period = 0, graph_cur = 0;
@@ -801,9 +853,84 @@ cudaError_t launch_fused(mdf_batch_t b, int K, int cur, int tk, bool save, int a
   return save ? launch_fused_t<2, true>(b, cur, tk, all) : launch_fused_t<2, false>(b, cur, tk, all);
 }
 
+// Seats of the resident kernel: every cavity in a team of the fewest CTAs
+// that hold it at `limit` nodes each, the largest teams first, each into the
+// first cluster with room.  The smallest limit at which the GPU holds all
+// clusters at once (7 of 16 CTAs with over 114 KB each); none: the batch fills
+// the GPU better with fused launches.
+cudaError_t build_seats(mdf_batch_t b) {
+  static const bool available = res_available(k_batch_resident<true>) && res_available(k_batch_resident<false>);
+  if (!available) return cudaSuccess;
+  for (int limit : {600, 900, 1200, 1500, kResMaxTeamNodes}) {
+    std::vector<std::pair<int, int>> teams;  // CTAs, cavity
+    int nodes = 0;
+    for (int c = 0; c < b->ncav; ++c) {
+      const int N = b->cav[c].N;
+      int t = 1;
+      while (t <= std::min(N, kResMaxCluster) && (N + t - 1) / t * N > limit) ++t;
+      if (t > std::min(N, kResMaxCluster)) break;
+      nodes = std::max(nodes, (N + t - 1) / t * N);
+      teams.push_back({t, c});
+    }
+    if ((int)teams.size() < b->ncav) continue;
+    std::stable_sort(teams.begin(), teams.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+    std::vector<BatchSeat> seats;
+    std::vector<int> used;  // seats taken of each cluster
+    for (const auto &t : teams) {
+      size_t k = 0;
+      while (k < used.size() && used[k] + t.first > kResMaxCluster) ++k;
+      if (k == used.size()) {
+        used.push_back(0);
+        seats.resize(seats.size() + kResMaxCluster, BatchSeat{-1, 0, 1});
+      }
+      for (int i = 0; i < t.first; ++i) seats[k * kResMaxCluster + used[k] + i] = {t.second, used[k], t.first};
+      used[k] += t.first;
+    }
+    const size_t smem = 2ull * 3 * D2Q5::Q * nodes * sizeof(float);
+    int clusters = 0;
+    cudaError_t e = res_clusters(k_batch_resident<true>, res_threads(nodes), smem, &clusters);
+    if (e != cudaSuccess) return e;
+    // one CTA per SM: two would take turns
+    if ((int)used.size() > std::min(clusters, kSMs / kResMaxCluster)) continue;
+    e = cudaMalloc(&b->seat_mem, seats.size() * sizeof(BatchSeat));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b->seat_mem, seats.data(), seats.size() * sizeof(BatchSeat), cudaMemcpyHostToDevice,
+                          b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // `seats` leaves scope
+    if (e != cudaSuccess) return e;
+    b->seats = (int)seats.size();
+    b->seat_smem = smem;
+    b->seat_pair = res_pairs(nodes);
+    b->seat_threads = res_threads(nodes);
+    return cudaSuccess;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_resident(mdf_batch_t b, int cur, int tk, int steps, bool save, int all) {
+  static const cudaError_t set1 = res_configure(k_batch_resident<true>), set0 = res_configure(k_batch_resident<false>);
+  if (set1 != cudaSuccess || set0 != cudaSuccess) return set1 != cudaSuccess ? set1 : set0;
+  const ResShape r{kResMaxCluster, 0, b->seat_smem};
+  const BatchSeat *seats = b->seat_mem;
+  return b->seat_pair ? res_launch(k_batch_resident<true>, b->seats / kResMaxCluster, r, b->seat_threads, b->stream, b->B,
+                                   seats, cur, tk, steps, (int)save, all)
+                      : res_launch(k_batch_resident<false>, b->seats / kResMaxCluster, r, b->seat_threads, b->stream, b->B,
+                                   seats, cur, tk, steps, (int)save, all);
+}
+
 // An even number of launches of four and two updates that make `period`
 // (even, >= 4) updates, so that the state ends in the buffer it started in.
 cudaError_t fused_period(mdf_batch_t b, int period) {
+  if (b->seats) {  // an even number of launches, for the same reason
+    const int n = 2 * ((period / 2 + (1 << 14) - 1) >> 14);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0, t = 0; k < n && e == cudaSuccess; ++k) {
+      const int s = (period - t) / (n - k);
+      e = launch_resident(b, b->cur ^ (k & 1), t, s, k == 0, 0);
+      t += s;
+    }
+    return e;
+  }
   int four = period / 4, two = (period & 3) / 2;
   if ((four + two) & 1) {
     --four;
@@ -953,6 +1080,7 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
   if (e == cudaSuccess) e = max_grid(b, b->threads, b->sched, &b->grid);
   if (e == cudaSuccess && d == 2 && b->with_rho) {
     e = build_items(b);
+    if (e == cudaSuccess) e = build_seats(b);
     b->fuse = e == cudaSuccess;
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -976,6 +1104,7 @@ void mdf_batch_destroy(mdf_batch_t b) {
   cudaFree(B.live); cudaFree(B.n_live); cudaFree(B.usave); cudaFree(B.part); cudaFree(B.badtile);
   cudaFree(B.status); cudaFree(B.steps); cudaFree(B.res); cudaFree(B.bar); cudaFree(B.err);
   cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem);
+  cudaFree(b->seat_mem);
   cudaFreeHost(b->host_live);
   delete b;
 }
@@ -1116,7 +1245,11 @@ mdf_status mdf_batch_step(mdf_batch_t b, long long n) {
   while (n > 0) {
     const bool fused = b->fuse && n >= 2;
     int s = (int)std::min<long long>(n, chunk), k = 0;
-    if (fused) {
+    if (fused && b->seats) {
+      s = std::min(s, 1 << 14);
+      BCU(b, launch_resident(b, b->cur, 0, s, false, 1));
+      b->cur ^= 1;
+    } else if (fused) {
       for (; s - k >= 2; b->cur ^= 1) {
         const int K = s - k >= 4 ? 4 : 2;
         BCU(b, launch_fused(b, K, b->cur, k, false, 1));
@@ -1290,7 +1423,8 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
   bool fuse = b->fuse;
   if (st == MDF_OK && fuse) {  // the fused launches against the best of them
     cudaError_t e = cudaEventRecord(e0, b->stream);
-    for (int k = 0; k < reps && e == cudaSuccess; k += reps - k >= 4 ? 4 : 2)
+    if (b->seats && e == cudaSuccess) e = launch_resident(b, b->cur, 0, reps, false, 1);
+    for (int k = 0; k < reps && e == cudaSuccess && !b->seats; k += reps - k >= 4 ? 4 : 2)
       e = launch_fused(b, reps - k >= 4 ? 4 : 2, b->cur, k, false, 1);
     if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);

@@ -27,7 +27,8 @@ constexpr int kResMaxCluster = 16;                // needs the non-portable size
 // 3.2; at 144^2 (1296) 2.95 / 3.2 and at 170^2 3.37 / 3.4 it no longer pays
 // for its start.
 constexpr int kResMaxNodes = 1200;
-constexpr size_t kResMaxSmem = 2ull * 15 * kResMaxNodes * sizeof(float);  // of a CTA
+constexpr int kResMaxTeamNodes = 1800;  // of a CTA in a batch of cavities
+constexpr size_t kResMaxSmem = 2ull * 15 * kResMaxTeamNodes * sizeof(float);  // of a CTA
 // Fewest updates that pay for reading and writing the lattice once more than
 // a fused launch would: with two nodes a thread four (128^2: 4.7 us per update
 // against 5.8 of single ones; with two updates 8.4 against 7.5).
@@ -59,14 +60,16 @@ template <int Q> struct ResPull {
 // the lanes of an FP32 pair (any two: every access is a 4-byte one), for CTAs
 // with more nodes than threads, which the issue slots bound; with a node a
 // thread the latency of one collision does, and the scalar form is shorter.
+// The lattice is held by CTAs first .. first + C - 1 of the cluster, of which
+// this is CTA first + rank; the barriers are the whole cluster's.  nodes = 0
+// (G.ny = 0) takes part in them alone.
 template <class L, bool WALLS, int FORCE, bool PAIR>
 __device__ __forceinline__ void res_run(const FuseLattice &G, bool with_rho, int steps, bool save, int rcap,
-                                        float *buf) {
+                                        float *buf, int first, int C, int rank) {
   namespace cg = cooperative_groups;
   using TC = typename std::conditional<PAIR, F2, float>::type;
   constexpr int Q = L::Q, NP = PAIR ? 2 : 1;
   const cg::cluster_group cl = cg::this_cluster();
-  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int base = G.ny / C, extra = G.ny - base * C;
   const int rows = base + (rank < extra ? 1 : 0), y0 = rank * base + min(rank, extra);
   const int lo = rank == 0 ? C - 1 : rank - 1, hi = rank == C - 1 ? 0 : rank + 1;
@@ -98,8 +101,8 @@ __device__ __forceinline__ void res_run(const FuseLattice &G, bool with_rho, int
     }
   }
   cl.sync();
-  const float *const rlo = cl.map_shared_rank(buf, lo) + lo_last * G.nx;  // row y0 - 1
-  const float *const rhi = cl.map_shared_rank(buf, hi);                   // row y0 + rows
+  const float *const rlo = cl.map_shared_rank(buf, first + lo) + lo_last * G.nx;  // row y0 - 1
+  const float *const rhi = cl.map_shared_rank(buf, first + hi);                 // row y0 + rows
   const Rates<TC> R(TC(G.s1), TC(G.s2));
 
   for (int s = 0; s < steps; ++s) {
@@ -230,7 +233,9 @@ __device__ __forceinline__ void res_run(const FuseLattice &G, bool with_rho, int
 template <class L, bool WALLS, int FORCE, bool PAIR>
 __global__ void __launch_bounds__(kResThreads) k_resident2d(const DevArgs A, int steps, int rcap) {
   extern __shared__ float res_smem[];
-  res_run<L, WALLS, FORCE, PAIR>(fuse_lattice<L>(A), A.with_rho != 0, steps, false, rcap, res_smem);
+  const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  res_run<L, WALLS, FORCE, PAIR>(fuse_lattice<L>(A), A.with_rho != 0, steps, false, rcap, res_smem, 0,
+                                 (int)cl.num_blocks(), (int)cl.block_rank());
 }
 
 // Threads of a CTA for its nodes: whole warps, a node each, or two each (as a
@@ -264,25 +269,25 @@ cudaError_t res_configure(Kernel kernel) {
   return e;
 }
 
-// Whether the device schedules clusters of the largest size and memory.
+// Clusters of the largest size that the device holds at once.
 template <class Kernel>
-bool res_available(Kernel kernel) {
-  if (res_configure(kernel) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
+cudaError_t res_clusters(Kernel kernel, int threads, size_t smem, int *n) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kResMaxCluster);
-  cfg.blockDim = dim3(kResThreads);
-  cfg.dynamicSmemBytes = kResMaxSmem;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kResMaxCluster;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+}
+template <class Kernel>
+bool res_available(Kernel kernel) {
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+  if (res_configure(kernel) != cudaSuccess || res_clusters(kernel, kResThreads, kResMaxSmem, &n) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -116,9 +116,12 @@ def test_fused_updates_in_a_captured_chunk(nx):
         assert np.array_equal(outs[0][k], outs[1][k]), k
 
 
-@pytest.mark.parametrize("sides", [[2, 3, 4, 5, 7], [55, 56, 57, 64], [113, 30, 65], [128]])
+# on chip: one CTA each, teams of several sizes and empty seats, the largest
+# team; by fused launches: boxes beyond that, alone and with small ones
+@pytest.mark.parametrize("sides", [[2, 3, 4, 5, 7], [55, 36, 57, 64, 37], [113, 30, 65], [128],
+                                   [65] * 3 + [97] * 5 + [129] * 4, [175, 20], [2, 267, 56]])
 def test_fused_cavities_equal_the_persistent_kernel(sides):
-    """Batched cavities by fused launches (the default) against the
+    """Batched cavities on chip or by fused launches (the default) against the
     persistent kernel: the same bits after steps and after a run, with its
     step counts, statuses and residuals."""
     from paper_2108_08591_gb300 import CavityBatch
@@ -145,12 +148,14 @@ def test_fused_cavities_equal_the_persistent_kernel(sides):
             assert np.array_equal(a[k], b[k]), k
 
 
-def test_fused_cavities_as_they_retire():
-    """Most cavities converge early: the last ones move to the lists of
-    shorter segments and keep the persistent kernel's bits."""
+@pytest.mark.parametrize("last", [129, 177])
+def test_fused_cavities_as_they_retire(last):
+    """Most cavities converge early: the last one goes on alone in its cluster,
+    or on the lists of shorter segments, and keeps the persistent kernel's
+    bits."""
     from paper_2108_08591_gb300 import CavityBatch
 
-    sides, Re = [33] * 40 + [129], [40.0] * 40 + [300.0]
+    sides, Re = [33] * 40 + [last], [40.0] * 40 + [300.0]
     got = []
     for own in (False, True):
         b = CavityBatch(sides, Re, lid_speed=0.1)
