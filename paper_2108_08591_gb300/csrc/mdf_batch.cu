@@ -21,6 +21,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -696,6 +697,9 @@ struct mdf_batch_s {
   int seat_threads = 0;
   size_t seat_smem = 0;
   BatchSeat *seat_mem = nullptr;
+  double *stage = nullptr;  // device staging of host seeds and fields, grown when needed
+  size_t stage_bytes = 0;
+  std::mutex stage_mu;      // held from the use of `stage` to the synchronisation
   int *host_live = nullptr;
   cudaGraphExec_t graph = nullptr;
   int graph_period = 0, graph_cur = 0;
@@ -725,6 +729,24 @@ mdf_status bfail(mdf_batch_t b, mdf_status st, const char *fmt, ...) {
     if (e_ != cudaSuccess)                                                               \
       return bfail((b), MDF_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_));     \
   } while (0)
+
+// Device staging of at least `bytes`, kept with the batch: allocated from the
+// stream's pool on each call, it was mapped and returned to the system at
+// every synchronisation.
+mdf_status ensure_stage(mdf_batch_t b, size_t bytes) {
+  if (b->stage_bytes >= bytes) return MDF_OK;
+  BCU(b, cudaStreamSynchronize(b->stream));
+  cudaFree(b->stage);
+  b->stage = nullptr;
+  b->stage_bytes = 0;
+  const cudaError_t e = cudaMalloc(&b->stage, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return bfail(b, MDF_ENOMEM, "staging %zu bytes: %s", bytes, cudaGetErrorString(e));
+  }
+  b->stage_bytes = bytes;
+  return MDF_OK;
+}
 
 template <class L, int T, int S>
 cudaError_t launch_chunk_t(mdf_batch_t b, int steps, int save_first) {
@@ -1104,7 +1126,7 @@ void mdf_batch_destroy(mdf_batch_t b) {
   cudaFree(B.live); cudaFree(B.n_live); cudaFree(B.usave); cudaFree(B.part); cudaFree(B.badtile);
   cudaFree(B.status); cudaFree(B.steps); cudaFree(B.res); cudaFree(B.bar); cudaFree(B.err);
   cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem);
-  cudaFree(b->seat_mem);
+  cudaFree(b->seat_mem); cudaFree(b->stage);
   cudaFreeHost(b->host_live);
   delete b;
 }
@@ -1128,13 +1150,14 @@ mdf_status mdf_batch_seed(mdf_batch_t b, int cavity, const double *P, const doub
     BCU(b, cudaStreamSynchronize(b->stream));
     return MDF_OK;
   }
+  std::lock_guard<std::mutex> lock(b->stage_mu);
   for (int c = lo; c < hi; ++c) {
     const CavParam &C = b->cav[c];
     const long long nn = b->d == 2 ? (long long)C.N * C.N : (long long)C.N * C.N * C.N;
     const size_t bytes = sizeof(double) * (size_t)nn;
-    double *dP = nullptr, *du = nullptr;
-    BCU(b, cudaMallocAsync(&dP, bytes, b->stream));
-    BCU(b, cudaMallocAsync(&du, bytes * b->d, b->stream));
+    const mdf_status st = ensure_stage(b, bytes * (1 + b->d));
+    if (st != MDF_OK) return st;
+    double *const dP = b->stage, *const du = b->stage + nn;
     if (P && u) {
       const cudaMemcpyKind kind = where == MDF_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
       BCU(b, cudaMemcpyAsync(dP, P, bytes, kind, b->stream));
@@ -1150,8 +1173,6 @@ mdf_status mdf_batch_seed(mdf_batch_t b, int cavity, const double *P, const doub
     if (b->d == 2) k_batch_init<D2Q5><<<blocks, kTile, 0, b->stream>>>(b->B, b->cur, c, dP, du, ne);
     else k_batch_init<D3Q7><<<blocks, kTile, 0, b->stream>>>(b->B, b->cur, c, dP, du, ne);
     BCU(b, cudaGetLastError());
-    BCU(b, cudaFreeAsync(dP, b->stream));
-    BCU(b, cudaFreeAsync(du, b->stream));
   }
   BCU(b, cudaStreamSynchronize(b->stream));
   return MDF_OK;
@@ -1287,12 +1308,16 @@ mdf_status mdf_batch_fields(mdf_batch_t b, int cavity, const mdf_fields_t *out) 
   A.s1 = C.s1d;
   A.with_rho = b->with_rho;
   double **slot[8] = {&A.P, &A.u, &A.rho, &A.G, &A.div, &A.S, &A.sigma, &A.omega};
-  double *stage = nullptr;
   size_t total = 0;
   for (int k = 0; k < 8; ++k)
     if (host[k]) total += count[k];
-  if (out->where == MDF_HOST && total) BCU(b, cudaMallocAsync(&stage, total * sizeof(double), b->stream));
-  double *p = stage;
+  std::unique_lock<std::mutex> lock(b->stage_mu, std::defer_lock);
+  if (out->where == MDF_HOST && total) {
+    lock.lock();
+    const mdf_status st = ensure_stage(b, total * sizeof(double));
+    if (st != MDF_OK) return st;
+  }
+  double *p = b->stage;
   for (int k = 0; k < 8; ++k)
     if (host[k]) {
       *slot[k] = out->where == MDF_HOST ? p : host[k];
@@ -1306,7 +1331,6 @@ mdf_status mdf_batch_fields(mdf_batch_t b, int cavity, const mdf_fields_t *out) 
     for (int k = 0; k < 8; ++k)
       if (host[k])
         BCU(b, cudaMemcpyAsync(host[k], *slot[k], count[k] * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-    if (stage) BCU(b, cudaFreeAsync(stage, b->stream));
     BCU(b, cudaStreamSynchronize(b->stream));
   }
   return MDF_OK;
