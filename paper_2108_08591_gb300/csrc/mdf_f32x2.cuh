@@ -50,35 +50,28 @@ struct F2 {
 };
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(vadd(a.f2(), b.f2())); }
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(vsub(a.f2(), b.f2())); }
-// Constants of the collision, as both lanes of an f32x2 operand in constant
-// memory: as immediates each use costs the moves that build the register
-// pair.
-enum Lit { LIT_NEG0, LIT_2_3, LIT_3_4, LIT_M4, LIT_M6, LIT_1_20, LIT_1_5, LIT_1_42, LIT_1_7, LIT_1_6, LIT_1_2,
-           LIT_DITHER, LIT_1, LIT_1_4, LIT_1_3, LIT_1_12, LITS };
-#define MDF_LITS                                                                                              \
-  {-0.0, 2.0 / 3.0, 0.75, -4.0, -6.0, 0.05, 0.2, 1.0 / 42.0, 1.0 / 7.0, 1.0 / 6.0, 0.5, -1.498046875 * 0x1p-23, \
-   1.0, 0.25, 1.0 / 3.0, 1.0 / 12.0}
-constexpr double kLit[LITS] = MDF_LITS;
-#define MDF_PAIR(k) {(float)kLit[k], (float)kLit[k]}
-static __constant__ float2 kLit2[LITS] = {MDF_PAIR(0),  MDF_PAIR(1),  MDF_PAIR(2),  MDF_PAIR(3),  MDF_PAIR(4),
-                                          MDF_PAIR(5),  MDF_PAIR(6),  MDF_PAIR(7),  MDF_PAIR(8),  MDF_PAIR(9),
-                                          MDF_PAIR(10), MDF_PAIR(11), MDF_PAIR(12), MDF_PAIR(13), MDF_PAIR(14),
-                                          MDF_PAIR(15)};
-#undef MDF_PAIR
+// Constants of the collision.
+enum Lit { LIT_2_3, LIT_3_4, LIT_M4, LIT_M6, LIT_1_20, LIT_1_5, LIT_1_42, LIT_1_7, LIT_1_6, LIT_1_2, LIT_DITHER,
+           LIT_1, LIT_1_4, LIT_1_3, LIT_1_12, LITS };
+constexpr double kLit[LITS] = {2.0 / 3.0,  0.75,      -4.0, -6.0, 0.05, 0.2, 1.0 / 42.0, 1.0 / 7.0, 1.0 / 6.0,
+                               0.5,        -1.498046875 * 0x1p-23,  1.0,  0.25, 1.0 / 3.0,  1.0 / 12.0};
 template <class T, Lit K> __device__ __forceinline__ T lit() {
   constexpr double v = kLit[K];
-  if constexpr (std::is_same<T, F2>::value) return F2(kLit2[K]);
-  else return T(v);
+  return T(v);
 }
-// The product is a * b + (-0), with the -0 read from constant memory: a sum
-// of a mul.rn.f32x2 and another value was compiled into one fused f32x2
-// operation (measured: other bits than mul and add, also with -fmad=false),
-// and the scalar kernels, whose bits these must be, round the product.
-// -0 known to the compiler is simplified back into the plain product.
-__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(vfma(a.f2(), b.f2(), kLit2[LIT_NEG0])); }
+// A product is two scalar ones.  A sum of a mul.rn.f32x2 and another value was
+// compiled into one fused f32x2 operation (measured: other bits than mul and
+// add, also with -fmad=false), and the scalar kernels, whose bits these must
+// be, round the product.  The f32x2 forms take two slots of the FP32 pipe, so
+// a pair of scalar products costs it nothing more, and most of them multiply
+// by an immediate.  (As a f32x2 fma with -0 and with the constants, both read
+// from constant memory: 158 us per update at 4096^2 against 152; the dither's
+// FMAs as scalar ones too: 148.)
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)); }
 // b + c a for a power of two c: the product is exact, so one rounding either way
 template <Lit K, class T> __device__ __forceinline__ T add_scaled(T b, T a) {
-  if constexpr (std::is_same<T, F2>::value) return F2(vfma(a.f2(), kLit2[K], b.f2()));
+  constexpr float c = (float)kLit[K];
+  if constexpr (std::is_same<T, F2>::value) return F2(vfma(a.f2(), make_float2(c, c), b.f2()));
   else return b + lit<T, K>() * a;
 }
 __device__ __forceinline__ F2 operator-(F2 a) { return F2(-a.x, -a.y); }

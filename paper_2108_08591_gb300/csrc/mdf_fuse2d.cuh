@@ -26,8 +26,8 @@
 // so the bits are those of K single updates.
 //
 // Measured (GB300, K = 4, us per update against one update per launch):
-// 4096^2 158 / 302, 2048^2 43.7 / 80, 1024^2 14.5 / 22.6, 256^2 3.7 / 6.2;
-// 4095^2 159 / (scalar kernel) 330; walls and lid 172 at 4096^2.  K = 4 is
+// 4096^2 148 / 302, 2048^2 40.9 / 80, 1024^2 13.9 / 22.6, 256^2 3.7 / 6.2;
+// 4095^2 149 / (scalar kernel) 330; walls and lid 166 at 4096^2.  K = 4 is
 // bound by the FP32 and integer pipes (issue 58 %, the f32x2 operations take
 // two slots of theirs): 219 instructions per update and node, of which 1.14
 // x is rim.  K = 2 would stay at HBM's 150 us.

@@ -23,8 +23,8 @@
 // type F2, the same dither draws), so the bits are those of two single
 // updates.
 //
-// Measured (GB300, us per update against the single one): 512^3 3647 / 4633,
-// 480 x 480 x 200 1226 / 1590, 256^3 536 / 584, 190 x 202 x 178 with walls
+// Measured (GB300, us per update against the single one): 512^3 3637 / 4633,
+// 480 x 480 x 200 1226 / 1590, 256^3 534 / 584, 190 x 202 x 178 with walls
 // and a lid 269 / 351, periodic 242 / 255.  Bound by the FP32 and integer
 // pipes (590 instructions per update and node at 256^3, where the tiles do
 // 1.5 x the work) and by the barriers: issue 47 %.  Requesting the next plane

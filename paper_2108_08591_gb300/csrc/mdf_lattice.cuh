@@ -100,10 +100,8 @@ __device__ __forceinline__ float dithered_change(float dl, float v, float r) {
   return __fmaf_rn(r, p2, __fmaf_rn(-1.498046875f * 0x1p-23f, p2, dl));
 }
 
-__device__ __forceinline__ F2 dithered_change(F2 dl, F2 v, F2 r) {  // lane by lane the same
-  const float2 p2 = make_float2(__int_as_float(__float_as_int(v.x) & 0x7f800000),
-                                __int_as_float(__float_as_int(v.y) & 0x7f800000));
-  return F2(vfma(r.f2(), p2, vfma(kLit2[LIT_DITHER], p2, dl.f2())));
+__device__ __forceinline__ F2 dithered_change(F2 dl, F2 v, F2 r) {
+  return F2(dithered_change(dl.x, v.x, r.x), dithered_change(dl.y, v.y, r.y));
 }
 
 // Random keys of one node (float) or of a pair of nodes (F2), and their
