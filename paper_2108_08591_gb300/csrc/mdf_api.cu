@@ -85,15 +85,19 @@ int default_block(int d, int storage) {
   return d == 3 ? 256 : 128;
 }
 
-// The block that leaves the fewest of a row's threads idle, between 64 and the
-// default (at least 128), the default on a tie.  190 x 202 x 178 BF16
+// The block that leaves the fewest of a row's threads idle, between `least` and
+// the default (at least 128), the default on a tie.  190 x 202 x 178 BF16
 // equilibrium-shifted (95 threads a row): 191 us per update with 96, 207 with
 // 128; 100^3 FP16 55 / 97, in place FP32 47 / 127; no shape measured slower by
-// more than 1 %.
-int fit_block(int threads, int dflt) {
+// more than 1 %.  `least` is 64 but where one node per thread leaves a 3D row
+// one busy warp: blocks of two warps then put all busy warps on the same two
+// of an SM's four schedulers, blocks of three do not (29 x 124 x 157 FP16:
+// 37 us with 64, 21 with 96, 23 with 128; FP32 with 32 nodes a row 41 / 27 /
+// 29; with 40 nodes 42 / 43 / 45).
+int fit_block(int threads, int dflt, int least) {
   const auto padded = [&](int b) { return (threads + b - 1) / b * b; };
   int best = dflt;
-  for (int b = std::max(dflt, 128); b >= 64; b -= 32)
+  for (int b = std::max(dflt, 128); b >= least; b -= 32)
     if (padded(b) < padded(best)) best = b;
   return best;
 }
@@ -124,7 +128,7 @@ struct mdf_s {
   long long key_base = 0;   // global index of local node 0 (slabs of a larger lattice)
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // chunk starting from buffer 0 / 1
   void *buf[2] = {nullptr, nullptr};
-  bool fuse = false;     // runs of updates go by fused launches (see mdf_create)
+  bool fuse[2] = {false, false};  // runs of updates go by fused launches [without / with a force] (see mdf_create)
   int resident = 0;      // runs of at least this many updates keep the lattice on chip (0: none)
   bool inplace = false;  // one buffer, AA pattern (buf[1] unused)
   int parity = 0;        // AA layout of the current state: 0 even, 1 odd
@@ -233,7 +237,7 @@ mdf_status one_update(mdf_t h, int mode, const mdf_fields_t *out) {
 // Updates the next launch of a run of n should make: 4 or 2 fused ones where
 // the lattice has such a kernel, else 1.
 int fused_updates(const mdf_t h, long long n) {
-  if (!h->fuse || n < 2) return 1;
+  if (!h->fuse[h->force != nullptr] || n < 2) return 1;
   if (h->d == 3) return 2;
   const int K = n >= 4 && h->ny >= 4 ? 4 : 2;
   return h->ny >= K ? K : 1;
@@ -422,10 +426,13 @@ mdf_status mdf_create(mdf_t *out, const mdf_grid *g, int d, const mdf_rates *r,
   h->vx = std::min(h->vx, max_vx(d, h->storage, h->inplace));
   const int row_threads = h->nx % h->vx == 0 ? h->nx / h->vx : h->nx;
   h->block = opts.block ? opts.block
-                        : fit_block(row_threads, h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage));
+                        : fit_block(row_threads, h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage),
+                                    d == 3 && !eq_storage(h->storage) && row_threads == h->nx && h->nx <= 32 ? 96 : 64);
   // a caller's own launch shape is that of the one-update kernel
-  h->fuse = h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
-            !opts.block && h->plane < (1LL << 31) - 64 && (d == 2 || fuse3_pays(h->nx, h->ny, h->nz, h->walls));
+  const bool can_fuse = h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
+                        !opts.block && h->plane < (1LL << 31) - 64;
+  for (int f = 0; f < 2; ++f)
+    h->fuse[f] = can_fuse && (d == 2 || fuse3_pays(h->nx, h->ny, h->nz, h->walls, f));
   if (d == 2 && h->storage == MDF_F32 && !h->inplace && !opts.vx && !opts.block)
     h->resident = lattice_launch(d, q)->resident_steps(h->nx, h->ny, h->nsets);
 

@@ -634,8 +634,8 @@ __global__ void __launch_bounds__(kMaxBlock) k_init_eq_moments(const DevArgs A) 
 // Second pass: the stored parts, from this node's moments and those of the
 // nodes its populations come to.  (In one pass every (set, direction) read
 // and narrowed its neighbour's FP64 seed again, 15 or 28 times a node: 1007
-// us at 2050 x 1998, now 154 for both.)
-template <class L, class TS, bool WALLS>
+// us at 2050 x 1998, then 154 for both.)  GRAD as for k_init: INITEQFIG
+template <class L, class TS, bool WALLS, bool GRAD>
 __global__ void __launch_bounds__(kMaxBlock) k_init_eq(const DevArgs A) {
   constexpr int D = L::D, Q = L::Q;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_init_eq(const DevArgs A) {
   auto moments = [&](long long r, int xx, float (&M)[D + 2]) {
     const float *p = mom + eq_off(A.px, r, xx, K);
 #pragma unroll
-    for (int k = 0; k < D + 2; ++k) M[k] = k < K ? p[k * kEqTile] : 0.f;
+    for (int k = 0; k < D + 2; ++k) M[k] = k < K ? __ldg(p + k * kEqTile) : 0.f;
   };
   float M0[D + 2];
   moments(row, x, M0);
@@ -670,13 +670,13 @@ __global__ void __launch_bounds__(kMaxBlock) k_init_eq(const DevArgs A) {
       const float *Fa = half ? static_cast<const float *>(A.force) + (alpha - 1) * A.plane : nullptr;
       if (wall) {
         target = -geq_m<L>(alpha, L::opp(i), M0);
-        if (A.Gin) target -= narrow_f64(fne_at<L>(A, N, n, alpha, L::opp(i)));
+        if (GRAD) target -= narrow_f64(fne_at<L>(A, N, n, alpha, L::opp(i)));
         if (alpha >= 1 && i == L::UP && (m & 0x80u))
           target += float(2.0 * L::w(i) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
         if (half) target += float(0.5 * L::w(i)) * __ldg(Fa + idx);  // negated by the bounce-back
       } else {
         target = geq_m<L>(alpha, i, Mt);
-        if (A.Gin) target += narrow_f64(fne_at<L>(A, N, trow * A.nx + tx, alpha, i));
+        if (GRAD) target += narrow_f64(fne_at<L>(A, N, trow * A.nx + tx, alpha, i));
         if (half) target -= float(0.5 * L::w(i)) * __ldg(Fa + trow * A.px + tx);
       }
       Codec<TS>::store(fn + ((alpha - 1 + A.with_rho) * Q + i) * kEqTile,

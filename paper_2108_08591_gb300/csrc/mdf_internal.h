@@ -91,11 +91,16 @@ cudaError_t launch_mask_d3q6(const int wall[3], int lid, const DevArgs &a, uint8
 
 // Two fused updates of a 3D lattice (mdf_fuse3d.cuh): planes per z segment,
 // and whether they pay.  Blocks of kFuse3Rows rows (two fewer stored) x 64
-// columns (60 stored), two per SM; a block takes about 5.2 us per plane and
-// 1.2 planes to fill, the single update 34.5 ps per node (1.25 x that with
-// walls, whose mask it reads): 128^3 (92 us fused, 74 single) and smaller
-// boxes stay single, 60 x 60 x 200 (31 / 37) and 190 x 202 x 178 (242 / 255)
-// go fused.
+// columns (60 stored), two per SM; a block is counted at 5.2 us per plane and
+// 1.2 planes to fill.  The lines are in that count per node, where the pair
+// and two single updates took the same time over 30 boxes of 49 .. 315 nodes
+// a side (D3Q7): 69 ps; 76 with walls, whose mask slows the single update
+// more (41 -> 49 ps a node at 235 x 118 x 161); 60 with a force, which slows the
+// pair by 13 % there and the two by 3 %; 66 with both.  128^3 (92 us the pair, 74 the
+// two) and smaller boxes stay single, 60 x 60 x 200 (31 / 37), 190 x 202 x 178
+// (242 / 255) and 145 x 267 x 175 (526 / 562) go fused; of walled boxes with a
+// force, 192 x 229 x 78 (358 / 301) stays single and 235 x 118 x 161
+// (388 / 437) goes fused.
 constexpr int kSMs = 152;  // of a GB300
 constexpr int kFuse3Rows = 8;
 struct Fuse3Plan {
@@ -112,8 +117,9 @@ inline Fuse3Plan fuse3_plan(int nx, int ny, int nz) {
   }
   return p;
 }
-inline bool fuse3_pays(int nx, int ny, int nz, bool walls) {
-  return fuse3_plan(nx, ny, nz).us < 69e-6 * (walls ? 1.25 : 1.0) * nx * (double)ny * nz;
+inline bool fuse3_pays(int nx, int ny, int nz, bool walls, bool force) {
+  const double ps = walls ? (force ? 66.0 : 76.0) : (force ? 60.0 : 69.0);
+  return fuse3_plan(nx, ny, nz).us < 1e-6 * ps * nx * (double)ny * nz;
 }
 
 // K updates in one launch (FP32, two buffers, all d + 1 sets): 2 or 4 in 2D

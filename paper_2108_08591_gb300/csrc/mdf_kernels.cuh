@@ -799,9 +799,12 @@ template <class TS> __device__ __forceinline__ typename ComputeOf<TS>::T round_t
 // seed read, every population written); the sets are unrolled so that the
 // moments stay in registers, and the pushed offset is formed once per
 // direction: with a loop over the sets, which indexed u by a run-time alpha,
-// 256^3 D3Q7 FP32 took 918 us, now 728; 4096^2 D2Q5
-// 730 -> 451.
-template <class L, class TS, bool WALLS>
+// 256^3 D3Q7 FP32 took 918 us and 4096^2 D2Q5 730.  GRAD (a seed gradient is
+// given) is a template argument because its FP64 code, unrolled for every set
+// and direction, is most of the kernel; with a run-time test in place of it
+// 256^3 took 728 us, now 507, 4096^2 451 -> 292 (floor 222), and
+// 19 x 202 x 226 FP16 with walls 250 -> 60.
+template <class L, class TS, bool WALLS, bool GRAD>
 __global__ void __launch_bounds__(kMaxBlock) k_init(const DevArgs A) {
   using TC = typename ComputeOf<TS>::T;
   constexpr int D = L::D, Q = L::Q;
@@ -835,12 +838,12 @@ __global__ void __launch_bounds__(kMaxBlock) k_init(const DevArgs A) {
       const bool lid = WALLS && wall && alpha >= 1 && o == L::UP && (m & 0x80u);
       if (A.aa && !lid) {  // in-place AA, even layout: slot i of x holds the arriving f_i(x)
         v = geq_v<L, TC>(alpha, i, u, Pp);
-        if (A.Gin) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+        if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
         if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
         dst = i * A.plane + idx;
       } else if (wall) {  // stored in slot o at x, negated by the bounce-back
         v = -geq_v<L, TC>(alpha, i, u, Pp);
-        if (A.Gin) v -= narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+        if (GRAD) v -= narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
         if (lid) v += TC(2.0 * L::w(o) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
         if (A.scheme2 && alpha >= 1) v = v + TC(0.5 * L::w(o)) * Fa;
         dst = o * A.plane + idx;
@@ -853,7 +856,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_init(const DevArgs A) {
         }
       } else {  // stored in slot i at x - c_i
         v = geq_v<L, TC>(alpha, i, u, Pp);
-        if (A.Gin) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+        if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
         if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
         dst = i * A.plane + src;
       }
@@ -964,8 +967,13 @@ namespace mdf {
 // ---------------------------------------------------------------------------
 // Host-side dispatch over storage / mode / walls for one lattice.
 // ---------------------------------------------------------------------------
-inline dim3 node_grid(const DevArgs &a) {
-  return dim3((unsigned)((a.nx + kBlockX - 1) / kBlockX), (unsigned)a.ny, (unsigned)a.nz);
+// Block for one thread per node of a row: 96 .. kBlockX, whichever leaves the
+// fewest threads idle, 96 for rows of one warp (two-warp blocks would put every
+// busy warp on two of an SM's four schedulers).
+inline int row_block(int nx) { return (nx + 95) / 96 * 96 < (nx + kBlockX - 1) / kBlockX * kBlockX ? 96 : kBlockX; }
+
+inline dim3 node_grid(const DevArgs &a, int b = kBlockX) {
+  return dim3((unsigned)((a.nx + b - 1) / b), (unsigned)a.ny, (unsigned)a.nz);
 }
 
 template <class L, class TS>
@@ -1108,16 +1116,30 @@ cudaError_t update_lattice(int storage, int mode, bool walls, const DevArgs &a, 
 
 template <class L, class TS>
 cudaError_t init_t(bool walls, const DevArgs &a, cudaStream_t s) {
-  if (walls) k_init<L, TS, true><<<node_grid(a), kBlockX, 0, s>>>(a);
-  else k_init<L, TS, false><<<node_grid(a), kBlockX, 0, s>>>(a);
+  const int b = row_block(a.nx);
+  const dim3 grid = node_grid(a, b);
+  if (a.Gin) {
+    if (walls) k_init<L, TS, true, true><<<grid, b, 0, s>>>(a);
+    else k_init<L, TS, false, true><<<grid, b, 0, s>>>(a);
+  } else {
+    if (walls) k_init<L, TS, true, false><<<grid, b, 0, s>>>(a);
+    else k_init<L, TS, false, false><<<grid, b, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
 template <class L, class TS>
 cudaError_t init_eq_t(bool walls, const DevArgs &a, cudaStream_t s) {
-  k_init_eq_moments<L><<<node_grid(a), kBlockX, 0, s>>>(a);
-  if (walls) k_init_eq<L, TS, true><<<node_grid(a), kBlockX, 0, s>>>(a);
-  else k_init_eq<L, TS, false><<<node_grid(a), kBlockX, 0, s>>>(a);
+  const int b = row_block(a.nx);
+  const dim3 grid = node_grid(a, b);
+  k_init_eq_moments<L><<<grid, b, 0, s>>>(a);
+  if (a.Gin) {
+    if (walls) k_init_eq<L, TS, true, true><<<grid, b, 0, s>>>(a);
+    else k_init_eq<L, TS, false, true><<<grid, b, 0, s>>>(a);
+  } else {
+    if (walls) k_init_eq<L, TS, true, false><<<grid, b, 0, s>>>(a);
+    else k_init_eq<L, TS, false, false><<<grid, b, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
