@@ -235,11 +235,16 @@ mdf_status one_update(mdf_t h, int mode, const mdf_fields_t *out) {
 }
 
 // Updates the next launch of a run of n should make: 4 or 2 fused ones where
-// the lattice has such a kernel, else 1.
+// the lattice has such a kernel, else 1.  2D lattices of fewer than 750 000
+// nodes take 2: with few rows for each warp the 12 extra row updates that fill
+// and drain the deeper pipeline cost more than a pass over memory that is in
+// L2 (230 x 500 with a force 6.3 us per update by fours, 5.2 by twos; 700 x 500
+// 8.1 / 7.3, 700 x 1024 12.5 / 11.4; 1024 x 830 13.4 / 13.5, 1024^2 15.6 /
+// 16.4, with walls and a force 17.2 / 18.7).
 int fused_updates(const mdf_t h, long long n) {
   if (!h->fuse[h->force != nullptr] || n < 2) return 1;
   if (h->d == 3) return 2;
-  const int K = n >= 4 && h->ny >= 4 ? 4 : 2;
+  const int K = n >= 4 && h->ny >= 4 && (long long)h->nx * h->ny >= 750000 ? 4 : 2;
   return h->ny >= K ? K : 1;
 }
 

@@ -26,11 +26,13 @@
 // so the bits are those of K single updates.
 //
 // Measured (GB300, K = 4, us per update against one update per launch):
-// 4096^2 148 / 302, 2048^2 40.9 / 80, 1024^2 13.9 / 22.6, 256^2 3.7 / 6.2;
+// 4096^2 148 / 302, 2048^2 40.9 / 80, 1024^2 13.9 / 22.6;
 // 4095^2 149 / (scalar kernel) 330; walls and lid 166 at 4096^2.  K = 4 is
 // bound by the FP32 and integer pipes (issue 58 %, the f32x2 operations take
 // two slots of theirs): 219 instructions per update and node, of which 1.14
-// x is rim.  K = 2 would stay at HBM's 150 us.
+// x is rim.  K = 2 would stay at HBM's 150 us; it serves lattices of fewer than
+// 750 000 nodes, where the row updates that fill and drain the pipeline count
+// (509 x 515 with walls: 5.9 us per update, 6.9 with K = 4, 10.0 single).
 #pragma once
 
 #include "mdf_kernels.cuh"

@@ -12,6 +12,8 @@ RESIDENT = [(2, 4), (3, 5), (24, 7), (57, 2), (64, 64), (129, 130), (300, 41), (
 # rows too short for the deeper kernels, one to several strips
 SHAPES = RESIDENT + [(1201, 16), (95, 310), (2000, 2), (1999, 3), (1921, 4), (2019, 9), (55, 560), (56, 550), (57, 545), (60, 512),
                      (61, 511), (113, 301), (128, 257), (300, 131)]
+# from 750 000 nodes on: by fours
+SHAPES += [(400001, 2), (250001, 3), (190001, 4), (150001, 5), (55, 13637), (56, 13400), (57, 13159), (113, 6638), (1003, 751)]
 BCS = [((0, 0), False), ((1, 0), False), ((0, 1), True), ((1, 1), True)]
 
 
@@ -35,7 +37,7 @@ def test_fused_updates_equal_single_updates(shape, forcing, q):
                 lat.set_force(F)
             lat.init(P, u)
             got = []
-            for n in (1, 2, 3, 4, 7):  # fused: 1: single; 2, 3: one launch of two; 4, 7: of four
+            for n in (1, 2, 3, 4, 7):  # fused: 1: single; the others by twos, or fours and a two
                 lat.step(n)
                 got += [v.clone() for v in lat.fields(("P", "u", "rho", "G")).values()]
             lat.close()
@@ -46,7 +48,7 @@ def test_fused_updates_equal_single_updates(shape, forcing, q):
 
 # boxes large enough for the fused kernel to be chosen (single updates below);
 # tile edges (60 of 64 columns, 6 of 8 rows), odd rows, one segment and many
-SHAPES3 = [(119, 61, 151), (59, 59, 211), (300, 120, 25), (960, 6, 200)]
+SHAPES3 = [(119, 61, 151), (59, 59, 211), (300, 120, 25), (960, 6, 200), (119, 121, 151)]
 BCS3 = [((0, 0, 0), False), ((1, 0, 0), False), ((0, 1, 0), False), ((0, 0, 1), True), ((1, 1, 1), True)]
 
 
@@ -96,7 +98,7 @@ def test_resident_updates_without_the_continuity_set():
         assert torch.equal(outs[0][k], outs[1][k]), k
 
 
-@pytest.mark.parametrize("nx", [97, 777])
+@pytest.mark.parametrize("nx", [97, 777, 15777])
 def test_fused_updates_in_a_captured_chunk(nx):
     import torch
     from paper_2108_08591_gb300 import Lattice
