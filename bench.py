@@ -53,6 +53,9 @@ TG3D_S2 = 1.0
 S2 = -1.0  # the workload's s2 (negative: the paper's rule); set in main()
 KERNEL_SOURCES = ("paper_2108_08591_gb300/csrc/mdf_kernels.cuh",
                   "paper_2108_08591_gb300/csrc/mdf_lattice.cuh")
+# sources of the fused FP32 update
+FUSED_SOURCES = KERNEL_SOURCES + ("paper_2108_08591_gb300/csrc/mdf_fuse2d.cuh",
+                                  "paper_2108_08591_gb300/csrc/mdf_f32x2.cuh")
 # sources of the equilibrium-shifted update (its recorded traffic is keyed
 # by their hash)
 EQ_SOURCES = KERNEL_SOURCES + ("paper_2108_08591_gb300/csrc/mdf_eq.cuh",
@@ -117,6 +120,21 @@ def _traffic(kernel_sha: str, leg: str = ""):
     if t.get("kernel_sha") != kernel_sha:
         return None
     return t.get("dram_bytes_per_launch_4096")
+
+
+def _fused_launches(n: int, shape, storage: str, single: bool = False):
+    """(updates per fused launch, launches) of a run of n plain updates on the
+    library's default launch shape: FP32 with two buffers runs 4 updates per
+    launch on 2D lattices from 750 000 nodes (then 2, then 1 for the rest) and 2
+    on the 3D workload's box; every other storage, a streaming in place and a
+    caller's own launch shape (`single`) one."""
+    nodes = math.prod(shape)
+    if storage != "f32" or single:
+        return 1, n
+    if len(shape) == 3:
+        return 2, n // 2 + n % 2
+    K = 4 if nodes >= 750000 else 2
+    return K, n // K + (n % K) // 2 + n % 2
 
 
 def _peaks():
@@ -359,15 +377,18 @@ def storage_leg(shape, s1, P, u, storage, steps=5, warmup=3, q=0, oracle_check=T
     lat.close()
     del fields
     peak, kind = _peaks()
-    achieved = info.bytes_per_update * N / (plain_ms / 1e3) / 1e9
+    # bytes each launch cannot do without, over all launches of the plain updates
+    per_launch, launches = _fused_launches(EPI_EVERY - 1, shape, storage)
+    achieved = info.bytes_per_update * N * launches / ((EPI_EVERY - 1) * plain_ms / 1e3) / 1e9
     sha = _kernel_sha(EQ_SOURCES) if storage.endswith("eq") else _kernel_sha()
     traffic = _traffic(sha, storage) if (N_GRID == 4096 and len(shape) == 2) else None
     out = {"storage": storage, "value": steps * EPI_EVERY * N / (ms / 1e3) / 1e6, "unit": "MLUPS",
            "steps": steps, "warmup": warmup,
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": traffic, "kernel_sha": sha,
-                        "bytes_per_node": info.bytes_per_update,
-                        "avg_launch_ms": plain_ms, "vx": info.vx, "block": info.block,
+                        "bytes_per_node": info.bytes_per_update, "updates_per_launch": per_launch,
+                        "avg_launch_ms": plain_ms * (EPI_EVERY - 1) / launches,
+                        "ms_per_update": plain_ms, "vx": info.vx, "block": info.block,
                         "peak_source": f"{kind} hbm_gbs (MEASURED_PEAKS.json)"}}
     if oracle_check:
         out["fp64_oracle_error"] = sampled_oracle_error(shape, s1, P, u, storage,
@@ -393,7 +414,7 @@ def tg3d_leg(oracle_check=True):
         out["workload"] = (f"3D Taylor-Green vortex, periodic 512^3, D3Q7 x 4 sets, U0 = {TG3D_U0}, "
                            f"Re = {TG3D_RE:.0f}, s2 = {TG3D_S2:g}, FP32 rest-shifted storage, "
                            "epilogue every 200 steps")
-        out["kernel"] = "k_update<D3Q7,float,MODE_STEP,periodic>"
+        out["kernel"] = "k_update_fused3d<D3Q7,2,periodic>"
         return out
     finally:
         S2, EPI_EVERY = saved
@@ -498,8 +519,11 @@ def run_mdf(args):
 
     peak, peak_kind = _peaks()
     bytes_per_launch = info.bytes_per_update * N
-    achieved = bytes_per_launch / (plain_ms / 1e3) / 1e9
-    sha = _kernel_sha()
+    # several updates share a pass over memory: bytes count per launch
+    per_launch, launches = _fused_launches(EPI_EVERY - 1, shape, args.storage,
+                                           args.inplace or bool(args.vx or args.block))
+    achieved = bytes_per_launch * launches / ((EPI_EVERY - 1) * plain_ms / 1e3) / 1e9
+    sha = _kernel_sha(FUSED_SOURCES if per_launch > 1 else KERNEL_SOURCES)
     default_lattice = args.q in (0, 5 if d == 2 else 7) and not args.inplace
     traffic = _traffic(sha) if (args.workload == "tg2d" and N_GRID == 4096
                                 and args.storage == "f32" and default_lattice) else None
@@ -526,6 +550,8 @@ def run_mdf(args):
                   else f"k_update_aa<{kname},{tname},even+odd,MODE_STEP,periodic>")
     elif args.storage.endswith("eq"):
         kernel = f"k_update_eq<{kname},{tname},VX={info.vx},MODE_STEP,periodic>"
+    elif per_launch > 1:
+        kernel = f"k_update_fused{d}d<{kname},{per_launch},periodic>"
     elif info.vx == 4 and args.storage == "f32":
         kernel = f"k_update_vec_f32x4<{kname},MODE_STEP,periodic>"
     elif info.vx > 1 and d == 3 and args.storage in ("f16", "bf16"):
@@ -547,7 +573,9 @@ def run_mdf(args):
                      "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)",
                      "kernel": kernel, "block": info.block,
                      "algorithmic_bytes_per_launch": bytes_per_launch,
-                     "avg_launch_ms": plain_ms, "kernel_sha": sha},
+                     "updates_per_launch": per_launch,
+                     "avg_launch_ms": plain_ms * (EPI_EVERY - 1) / launches,
+                     "ms_per_update": plain_ms, "kernel_sha": sha},
         "fp64_oracle_error": oerr,
         "storage_f16eq": extra,
         "workload_tg3d": leg3d,
@@ -557,7 +585,7 @@ def run_mdf(args):
                 "d2h_bytes_per_step": int(outP.nbytes + outu.nbytes),
                 "path": "C-ABI host buffers: mdf_init(MDF_HOST) from pinned memory, the step, "
                         "mdf_fields(MDF_HOST) into pinned memory; serial, host clock"},
-        "gpu_launches": args.steps * EPI_EVERY,
+        "gpu_launches": args.steps * (1 + launches),
         "clocks": clocks,
     }
     print(json.dumps(line), flush=True)
@@ -618,8 +646,10 @@ def run_cavities(args):
         "ms_per_step": ms, "nodes": int(nodes.sum()), "cavities": len(sides),
         "roofline": {"bound": "hbm", "achieved": mlups * 120 / 1e3, "peak": peak, "unit": "GB/s",
                      "frac": mlups * 120 / 1e3 / peak, "peak_source": f"{kind} hbm_gbs",
-                     "kernel": f"k_batch_chunk<D2Q5,{sched['threads']},{sched['sched']}> "
-                               "(persistent, cooperative)"},
+                     "kernel": "k_batch_fused<D2Q5,4> and k_batch_resident<D2Q5>, or where the autotuner "
+                               f"measured it faster k_batch_chunk<D2Q5,{sched['threads']},{sched['sched']}>",
+                     "bytes": "120 per node and update, as if every update were a pass of its own (4 updates "
+                              "share a pass, boxes on chip make none between checks): above 1 means shared passes"},
         "schedule": {"tuned": sched, "default": sched_default, "autotune_s": tune_s,
                      "default_mlups": float(nodes.sum() / (ms_default / 1e3) / 1e6)},
         "to_steady": {"tol": 1e-8, "max_steps": args.max_steps, "seconds": run_s,

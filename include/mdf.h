@@ -517,8 +517,10 @@ mdf_status mdf_nn_conv_wgrad(const void *x, const void *dz, float *dw, float *pa
 mdf_status mdf_nn_conv_dgrad(const void *dz, const void *w, void *wt, void *dx, int B, int H, int W,
                              int Cin, int Cout, void *stream);
 /* Forward/dgrad convolution kernel, process-wide: which = 2 the tcgen05
- * kernel with one staged input halo per channel chunk reused by the nine
- * taps (the default; Cin % 16 != 0 falls back to 1), 1 the tcgen05 kernel
+ * kernels with one staged input halo per channel chunk reused by the nine
+ * taps (the default: persistent CTAs fed by TMA where the pointers are 16-byte
+ * aligned and no tile override is set, else one CTA per tile, the same bits;
+ * Cin % 16 != 0 falls back to 1), 1 the tcgen05 kernel
  * with im2col gathers, 0 the mma.sync kernel.  All accumulate in FP32. */
 mdf_status mdf_nn_set_conv_kernel(int which);
 
