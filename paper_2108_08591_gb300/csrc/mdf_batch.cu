@@ -940,6 +940,16 @@ cudaError_t launch_resident(mdf_batch_t b, int cur, int tk, int steps, bool save
                                    seats, cur, tk, steps, (int)save, all);
 }
 
+// Updates a fused launch should make: four for 750 000 nodes or more, else two
+// (as for single lattices: the rows that fill and drain the deeper march count;
+// four boxes of 300^2 10.9 us per update by fours, 10.0 by twos, twelve 21.4 /
+// 22.7).
+int fused_depth(mdf_batch_t b) {
+  long long nodes = 0;
+  for (const CavParam &c : b->cav) nodes += (long long)c.N * c.N;
+  return nodes >= 750000 ? 4 : 2;
+}
+
 // An even number of launches of four and two updates that make `period`
 // (even, >= 4) updates, so that the state ends in the buffer it started in.
 cudaError_t fused_period(mdf_batch_t b, int period) {
@@ -954,7 +964,10 @@ cudaError_t fused_period(mdf_batch_t b, int period) {
     return e;
   }
   int four = period / 4, two = (period & 3) / 2;
-  if ((four + two) & 1) {
+  if (fused_depth(b) == 2) {
+    four = (period / 2) & 1;
+    two = period / 2 - 2 * four;
+  } else if ((four + two) & 1) {
     --four;
     two += 2;
   }
@@ -1271,8 +1284,9 @@ mdf_status mdf_batch_step(mdf_batch_t b, long long n) {
       BCU(b, launch_resident(b, b->cur, 0, s, false, 1));
       b->cur ^= 1;
     } else if (fused) {
+      const int depth = fused_depth(b);
       for (; s - k >= 2; b->cur ^= 1) {
-        const int K = s - k >= 4 ? 4 : 2;
+        const int K = s - k >= 4 ? depth : 2;
         BCU(b, launch_fused(b, K, b->cur, k, false, 1));
         k += K;
       }
@@ -1448,8 +1462,9 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
   if (st == MDF_OK && fuse) {  // the fused launches against the best of them
     cudaError_t e = cudaEventRecord(e0, b->stream);
     if (b->seats && e == cudaSuccess) e = launch_resident(b, b->cur, 0, reps, false, 1);
-    for (int k = 0; k < reps && e == cudaSuccess && !b->seats; k += reps - k >= 4 ? 4 : 2)
-      e = launch_fused(b, reps - k >= 4 ? 4 : 2, b->cur, k, false, 1);
+    const int depth = fused_depth(b);
+    for (int k = 0; k < reps && e == cudaSuccess && !b->seats; k += reps - k >= 4 ? depth : 2)
+      e = launch_fused(b, reps - k >= 4 ? depth : 2, b->cur, k, false, 1);
     if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;

@@ -119,9 +119,10 @@ def test_fused_updates_in_a_captured_chunk(nx):
 
 
 # on chip: one CTA each, teams of several sizes and empty seats, the largest
-# team; by fused launches: boxes beyond that, alone and with small ones
+# team; by fused launches: boxes beyond that, alone and with small ones, by twos
+# and (750 000 nodes) by fours
 @pytest.mark.parametrize("sides", [[2, 3, 4, 5, 7], [55, 36, 57, 64, 37], [113, 30, 65], [128],
-                                   [65] * 3 + [97] * 5 + [129] * 4, [175, 20], [2, 267, 56]])
+                                   [65] * 3 + [97] * 5 + [129] * 4, [175, 20], [2, 267, 56], [2, 870, 56]])
 def test_fused_cavities_equal_the_persistent_kernel(sides):
     """Batched cavities on chip or by fused launches (the default) against the
     persistent kernel: the same bits after steps and after a run, with its
@@ -139,7 +140,7 @@ def test_fused_cavities_equal_the_persistent_kernel(sides):
             b.step(n)
         out += [b.fields_host(c, ("P", "u", "rho", "G")) for c in range(b.n)]
         b.init()
-        for period in (6, 4, 100):  # 4: two launches of two; 100: 24 of four and two of two
+        for period in (6, 4, 100):  # by twos with a four for 6 and 100, or by fours and twos
             r = b.run(tol=1e-4, max_steps=3 * period, check_every=period)
         out += [{"steps": r[0], "status": r[1], "res": r[2]}]
         out += [b.fields_host(c, ("P", "u", "rho", "G")) for c in range(b.n)]
@@ -150,7 +151,7 @@ def test_fused_cavities_equal_the_persistent_kernel(sides):
             assert np.array_equal(a[k], b[k]), k
 
 
-@pytest.mark.parametrize("last", [129, 177])
+@pytest.mark.parametrize("last", [129, 177, 866])
 def test_fused_cavities_as_they_retire(last):
     """Most cavities converge early: the last one goes on alone in its cluster,
     or on the lists of shorter segments, and keeps the persistent kernel's
