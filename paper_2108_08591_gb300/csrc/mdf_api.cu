@@ -872,7 +872,6 @@ namespace {
 constexpr size_t kNoallocStageDoubles = size_t(1) << 21;
 static __device__ __align__(256) double g_noalloc_stage[kNoallocStageDoubles];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
 double *g_noalloc_addr[kMaxDevices] = {};  // device address of the buffer, per GPU
 

@@ -881,8 +881,8 @@ cudaError_t launch_fused(mdf_batch_t b, int K, int cur, int tk, bool save, int a
 // clusters at once (7 of 16 CTAs with over 114 KB each); none: the batch fills
 // the GPU better with fused launches.
 cudaError_t build_seats(mdf_batch_t b) {
-  static const bool available = res_available(k_batch_resident<true>) && res_available(k_batch_resident<false>);
-  if (!available) return cudaSuccess;
+  static OncePerDevice once1, once0;
+  if (!res_available(once1, k_batch_resident<true>) || !res_available(once0, k_batch_resident<false>)) return cudaSuccess;
   for (int limit : {600, 900, 1200, 1500, kResMaxTeamNodes}) {
     std::vector<std::pair<int, int>> teams;  // CTAs, cavity
     int nodes = 0;
@@ -930,8 +930,6 @@ cudaError_t build_seats(mdf_batch_t b) {
 }
 
 cudaError_t launch_resident(mdf_batch_t b, int cur, int tk, int steps, bool save, int all) {
-  static const cudaError_t set1 = res_configure(k_batch_resident<true>), set0 = res_configure(k_batch_resident<false>);
-  if (set1 != cudaSuccess || set0 != cudaSuccess) return set1 != cudaSuccess ? set1 : set0;
   const ResShape r{kResMaxCluster, 0, b->seat_smem};
   const BatchSeat *seats = b->seat_mem;
   return b->seat_pair ? res_launch(k_batch_resident<true>, b->seats / kResMaxCluster, r, b->seat_threads, b->stream, b->B,

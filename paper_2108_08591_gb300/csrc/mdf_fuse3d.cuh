@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(32 * kF3Rows, kF3Blocks)
 template <class L, bool WALLS, int FORCE>
 cudaError_t launch_fused3d(const DevArgs &a, cudaStream_t s) {
   constexpr size_t smem = (size_t)kF3Rows * fuse3_slots<L>() * 32 * sizeof(float2);
-  static const cudaError_t set = cudaFuncSetAttribute(k_update_fused3d<L, WALLS, FORCE>,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static OncePerDevice once;
+  const cudaError_t set = allow_smem(once, k_update_fused3d<L, WALLS, FORCE>, smem);
   if (set != cudaSuccess) return set;
   const int tx = (a.nx + fuse_out<2>() - 1) / fuse_out<2>(), ty = (a.ny + kF3Out - 1) / kF3Out;
   const int seg = fuse3_plan(a.nx, a.ny, a.nz).seg;

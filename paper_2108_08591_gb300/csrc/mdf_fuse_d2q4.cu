@@ -13,9 +13,9 @@ cudaError_t launch_resident_d2q4(int steps, bool walls, const DevArgs &a, cudaSt
   return update_resident2d<D2Q4>(walls, a, steps, s);
 }
 int resident_steps_d2q4(int nx, int ny, int nsets) {
-  static const bool available = res_available(k_resident2d<D2Q4, true, FORCE_EQ321, true>);
+  static OncePerDevice once;
   const ResShape r = res_shape(nx, ny, D2Q4::Q, nsets);
-  return available && r.ctas ? res_min_steps(r.rows * nx) : 0;
+  return r.ctas && res_available(once, k_resident2d<D2Q4, true, FORCE_EQ321, true>) ? res_min_steps(r.rows * nx) : 0;
 }
 
 }  // namespace mdf

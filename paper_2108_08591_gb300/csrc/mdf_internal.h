@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "mdf_device.h"
+
 namespace mdf {
 
 // Everything a kernel launch needs, as plain pointers and sizes.

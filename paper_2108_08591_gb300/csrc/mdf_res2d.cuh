@@ -284,19 +284,24 @@ cudaError_t res_clusters(Kernel kernel, int threads, size_t smem, int *n) {
   cfg.numAttrs = 1;
   return cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
 }
+// Whether the current device runs clusters of the largest size (configures
+// the kernel for them).
 template <class Kernel>
-bool res_available(Kernel kernel) {
-  int n = 0;
-  if (res_configure(kernel) != cudaSuccess || res_clusters(kernel, kResThreads, kResMaxSmem, &n) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return n > 0;
+bool res_available(OncePerDevice &once, Kernel kernel) {
+  const cudaError_t e = once([&] {
+    int n = 0;
+    cudaError_t s = res_configure(kernel);
+    if (s == cudaSuccess) s = res_clusters(kernel, kResThreads, kResMaxSmem, &n);
+    return s != cudaSuccess || n > 0 ? s : cudaErrorNotSupported;
+  });
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
 }
 
 template <class L, bool WALLS, int FORCE, bool PAIR>
 cudaError_t launch_resident2d_p(const ResShape &r, const DevArgs &a, int steps, cudaStream_t s) {
-  static const cudaError_t set = res_configure(k_resident2d<L, WALLS, FORCE, PAIR>);
+  static OncePerDevice once;
+  const cudaError_t set = once([] { return res_configure(k_resident2d<L, WALLS, FORCE, PAIR>); });
   if (set != cudaSuccess) return set;
   return res_launch(k_resident2d<L, WALLS, FORCE, PAIR>, 1, r, res_threads(r.rows * a.nx), s, a, steps, r.rows);
 }

@@ -27,6 +27,7 @@
 #include <mutex>
 
 #include "mdf.h"
+#include "mdf_device.h"
 #include "mdf_nn.cuh"
 #include "mdf_nn_wgrad_tc.cuh"
 #include "mdf_nn_pers.cuh"
@@ -139,15 +140,11 @@ int g_tc_bn = 0, g_tc_stages = 0;  // tile override of the tcgen05 kernel (0 = a
 
 template <int BN, int S>
 cudaError_t launch_tc(cudaStream_t s, const ConvArgs &a, long long M, int *err) {
-  static bool configured = false;
+  static mdf::OncePerDevice once;
   const size_t smem = tc_smem_bytes<BN, S>();
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_fwd_tc<BN, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  const cudaError_t e = mdf::allow_smem(once, k_conv_fwd_tc<BN, S>, smem);
+  if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((a.Cout + BN - 1) / BN));
   k_conv_fwd_tc<BN, S><<<grid, TC_THREADS, smem, s>>>(a, err);
   return cudaGetLastError();
@@ -176,15 +173,11 @@ void tc_tile(long long M, int Cout, int &bn, int &stages) {
 template <int BN, int KC, int MT>
 cudaError_t launch_halo(cudaStream_t s, const ConvArgs &a, int *err) {
   constexpr int S = 4;
-  static bool configured = false;
+  static mdf::OncePerDevice once;
   const size_t smem = halo_smem_bytes<BN, KC, MT, S>();
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_fwd_halo<BN, KC, MT, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  const cudaError_t e = mdf::allow_smem(once, k_conv_fwd_halo<BN, KC, MT, S>, smem);
+  if (e != cudaSuccess) return e;
   const HaloGeom g = halo_geom(a.H, a.W, MT);
   const long long nx = (long long)a.B * g.strips * g.tiles;
   if (nx > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -374,13 +367,9 @@ PersPlan pers_plan(const ConvArgs &a, int sms) {
 template <int KC, int MT>
 cudaError_t launch_pers(cudaStream_t s, const ConvArgs &a, const PersPlan &p, const CUtensorMap &xm,
                         const CUtensorMap &wm, int *err) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_conv_fwd_pers<KC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemOptin);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static mdf::OncePerDevice once;
+  const cudaError_t e = mdf::allow_smem(once, k_conv_fwd_pers<KC, MT>, kMaxSmemOptin);
+  if (e != cudaSuccess) return e;
   k_conv_fwd_pers<KC, MT><<<dim3((unsigned)p.grid, (unsigned)p.nb), PC_THREADS, p.smem, s>>>(xm, wm, a, p.g, err);
   return cudaGetLastError();
 }
@@ -438,13 +427,9 @@ int pix_per_split(long long M) { return M >= 8192 ? 2048 : 256; }
 template <bool SWAP, int KC, int BN, int S>
 cudaError_t launch_wgrad_tma(cudaStream_t s, const CUtensorMap &xm, const CUtensorMap &dm, const WgradTmaArgs &a,
                              int *err) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_tma<SWAP, KC, BN, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemOptin);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static mdf::OncePerDevice once;
+  const cudaError_t e = mdf::allow_smem(once, k_conv_wgrad_tma<SWAP, KC, BN, S>, kMaxSmemOptin);
+  if (e != cudaSuccess) return e;
   const int nn = SWAP ? a.Cout : a.Cin, mm = SWAP ? a.Cin : a.Cout;
   dim3 grid((unsigned)((nn + BN - 1) / BN), (unsigned)((mm + 127) / 128), (unsigned)(3 * a.splits));
   k_conv_wgrad_tma<SWAP, KC, BN, S>

@@ -1,0 +1,65 @@
+"""Loads the library's host code linked against fake_cudart.cpp in the place of
+the CUDA runtime, so that plans, dispatch and error paths are tested without a
+GPU."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+from paper_2108_08591_gb300 import _build, _lib
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+def link(out):
+    """Link the built objects with the stand-in into `out`."""
+    _build.build()
+    objs = sorted(glob.glob(os.path.join(_build.BUILD, "mdf_*.o")))
+    if len(objs) != len(_build._sources()):
+        _build.build(force=True)
+        objs = sorted(glob.glob(os.path.join(_build.BUILD, "mdf_*.o")))
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build._nvcc()))), "include")
+    # -Bsymbolic: the library's calls bind to the stand-in also where a real runtime is loaded
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", inc,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", str(out)], check=True)
+
+
+class Fake:
+    """One copy of the library and its stand-in (each copy has its own state)."""
+
+    def __init__(self, linked, path):
+        shutil.copy(linked, path)
+        self.lib = ctypes.CDLL(str(path))
+        for name, (res, args) in _lib.SIGNATURES.items():
+            fn = getattr(self.lib, name)
+            fn.restype, fn.argtypes = res, args
+        self.lib.fake_launch.restype = ctypes.c_char_p
+        self.lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double, ctypes.c_double]
+
+    def launches(self):
+        """Recorded launches as (kernel, device, blocks, threads, cluster)."""
+        out = []
+        for k in range(self.lib.fake_launches()):
+            v = [ctypes.c_uint() for _ in range(4)]
+            name = self.lib.fake_launch(k, *(ctypes.byref(x) for x in v)).decode()
+            out.append((name, *(x.value for x in v)))
+        self.lib.fake_clear()
+        return out
+
+    def lattice(self, shape, storage="f32", **opts):
+        h = ctypes.c_void_p()
+        g = _lib.Grid(*shape, *([1] if len(shape) == 2 else []))
+        r = _lib.Rates(1.0, 1.7, -1.0)
+        o = _lib.Opts(_lib.STORAGE[storage], 1, None, *(opts.get(k, 0) for k in ("vx", "block", "q", "inplace")))
+        st = self.lib.mdf_create(ctypes.byref(h), ctypes.byref(g), len(shape), ctypes.byref(r), None, ctypes.byref(o))
+        assert st == _lib.OK, self.lib.mdf_last_error(None)
+        return h
+
+    def batch(self, sides):
+        h = ctypes.c_void_p()
+        side = (ctypes.c_int * len(sides))(*sides)
+        Re = (ctypes.c_double * len(sides))(*[100.0] * len(sides))
+        st = self.lib.mdf_batch_create(ctypes.byref(h), 2, len(sides), side, Re, 0.1, None)
+        assert st == _lib.OK, self.lib.mdf_batch_last_error(None)
+        return h

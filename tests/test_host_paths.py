@@ -1,0 +1,56 @@
+"""Host-side paths of the library that need no GPU: per-device state, fallbacks
+and launch plans, against a stand-in for the CUDA runtime (fake_cudart.cpp)."""
+import ctypes
+import shutil
+
+import numpy as np
+import pytest
+
+from paper_2108_08591_gb300 import _lib
+
+pytestmark = pytest.mark.skipif(not shutil.which("g++"), reason="g++ not found")
+
+
+@pytest.fixture(scope="module")
+def linked(tmp_path_factory):
+    from _fakecuda import link
+    out = tmp_path_factory.mktemp("fake") / "libmdf_fake.so"
+    link(out)
+    return out
+
+
+@pytest.fixture
+def fake(linked, tmp_path):
+    from _fakecuda import Fake
+    return Fake(linked, tmp_path / "libmdf_fake.so")
+
+
+def test_kernel_attributes_are_set_on_every_device(fake):
+    """Shared memory and cluster sizes beyond the defaults are a device's own:
+    a handle on a second GPU of the process launches as on the first."""
+    lib = fake.lib
+    conv = [np.zeros(8 * 8 * 64 * 64, np.float32) for _ in range(3)]
+    x, w, y = ((a.ctypes.data + 63) // 64 * 64 for a in conv)
+    got = []
+    for dev in (0, 1):
+        lib.fake_set_device(dev)
+        for shape, q in (((64, 64), 0), ((40, 60), 4), ((60, 60, 200), 0), ((60, 60, 200), 6)):
+            h = fake.lattice(shape, q=q)
+            assert lib.mdf_step(h, 6) == _lib.OK, (dev, shape, lib.mdf_last_error(h))
+            lib.mdf_destroy(h)
+        b = fake.batch([65, 97, 129])
+        assert lib.mdf_batch_step(b, 10) == _lib.OK, (dev, lib.mdf_batch_last_error(b))
+        lib.mdf_batch_destroy(b)
+        for which in (2, 1):
+            assert lib.mdf_nn_set_conv_kernel(which) == _lib.OK
+            assert lib.mdf_nn_conv_fwd(x, w, None, y, None, 1, 64, 64, 32, 32, 0, None) == _lib.OK, (dev, which)
+        assert lib.mdf_nn_set_conv_kernel(2) == _lib.OK
+        assert lib.mdf_nn_set_halo_tile(2, 16) == _lib.OK
+        assert lib.mdf_nn_conv_fwd(x, w, None, y, None, 1, 64, 64, 32, 32, 0, None) == _lib.OK, dev
+        assert lib.mdf_nn_set_halo_tile(0, 0) == _lib.OK
+        assert lib.mdf_nn_conv_wgrad(x, x, y, w, 1, 64, 64, 32, 32, None) == _lib.OK, dev
+        got.append([(n, *rest) for n, d, *rest in fake.launches() if d == dev])
+    assert got[0] == got[1]
+    for kernel in ("k_resident2d", "k_update_fused3d", "k_batch_resident", "k_conv_fwd_pers", "k_conv_fwd_halo",
+                   "k_conv_fwd_tc", "k_conv_wgrad_tma"):
+        assert any(kernel in n for n, *_ in got[1]), kernel
