@@ -825,7 +825,8 @@ cudaError_t max_grid(mdf_batch_t b, int threads, int sched, int *grid) {
   return e;
 }
 
-// The item lists of the fused kernel (see BatchItems).
+// The item lists of the fused kernel (see BatchItems).  On an error the batch
+// keeps to the persistent kernel.
 cudaError_t build_items(mdf_batch_t b) {
   constexpr int K = 4, OUT = fuse_out<K>();
   static_assert(fuse_out<2>() >= OUT, "the strips of four updates serve two as well");
@@ -879,7 +880,8 @@ cudaError_t launch_fused(mdf_batch_t b, int K, int cur, int tk, bool save, int a
 // that hold it at `limit` nodes each, the largest teams first, each into the
 // first cluster with room.  The smallest limit at which the GPU holds all
 // clusters at once (7 of 16 CTAs with over 114 KB each); none: the batch fills
-// the GPU better with fused launches.
+// the GPU better with fused launches, as it does where a query or the
+// allocation fails.
 cudaError_t build_seats(mdf_batch_t b) {
   static OncePerDevice once1, once0;
   if (!res_available(once1, k_batch_resident<true>) || !res_available(once0, k_batch_resident<false>)) return cudaSuccess;
@@ -919,7 +921,7 @@ cudaError_t build_seats(mdf_batch_t b) {
       e = cudaMemcpyAsync(b->seat_mem, seats.data(), seats.size() * sizeof(BatchSeat), cudaMemcpyHostToDevice,
                           b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // `seats` leaves scope
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;  // b->seats stays 0
     b->seats = (int)seats.size();
     b->seat_smem = smem;
     b->seat_pair = res_pairs(nodes);
@@ -1111,10 +1113,11 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
     e = cudaMemcpyAsync((void *)B.tile_cav, tile_cav.data(), sizeof(int) * b->ntiles,
                         cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = max_grid(b, b->threads, b->sched, &b->grid);
+  // what only the fused and the resident launches need does not fail the
+  // batch: without it the next slower path takes its updates
   if (e == cudaSuccess && d == 2 && b->with_rho) {
-    e = build_items(b);
-    if (e == cudaSuccess) e = build_seats(b);
-    b->fuse = e == cudaSuccess;
+    b->fuse = build_items(b) == cudaSuccess;
+    if (!b->fuse || build_seats(b) != cudaSuccess) cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {

@@ -54,3 +54,41 @@ def test_kernel_attributes_are_set_on_every_device(fake):
     for kernel in ("k_resident2d", "k_update_fused3d", "k_batch_resident", "k_conv_fwd_pers", "k_conv_fwd_halo",
                    "k_conv_fwd_tc", "k_conv_wgrad_tma"):
         assert any(kernel in n for n, *_ in got[1]), kernel
+
+
+def _step_kernels(fake, b):
+    fake.launches()
+    assert fake.lib.mdf_batch_step(b, 8) == _lib.OK, fake.lib.mdf_batch_last_error(b)
+    return {n for n, *_ in fake.launches() if "batch_tick" not in n}
+
+
+def test_batch_falls_back_where_its_faster_path_cannot_be_set_up(fake):
+    """A cluster query or an allocation that only the fused launches need does
+    not fail the creation of a batch: it goes by fused launches, or by the
+    persistent kernel."""
+    lib = fake.lib
+    b = fake.batch([65, 97])
+    assert all("k_batch_resident" in n for n in _step_kernels(fake, b))
+    lib.mdf_batch_destroy(b)
+    lib.fake_fail_clusters(1)
+    b = fake.batch([65, 97])
+    assert all("k_batch_fused" in n for n in _step_kernels(fake, b))
+    lib.mdf_batch_destroy(b)
+    lib.fake_fail_clusters(0)
+    side, Re = (ctypes.c_int * 2)(65, 97), (ctypes.c_double * 2)(100.0, 100.0)
+    got = []
+    for k in range(1, 40):  # the k-th allocation fails
+        lib.fake_fail_malloc(k)
+        b = ctypes.c_void_p()
+        st = lib.mdf_batch_create(ctypes.byref(b), 2, 2, side, Re, 0.1, None)
+        lib.fake_fail_malloc(0)
+        if st != _lib.OK:
+            assert st == _lib.ENOMEM
+            got.append("refused")
+            continue
+        kinds = _step_kernels(fake, b)
+        got.append(next(n for n in ("chunk", "fused", "resident") if any(n in x for x in kinds)))
+        lib.mdf_batch_destroy(b)
+    # the state's own, the lists of fused launches, the seats on chip, none
+    order = [g for k, g in enumerate(got) if k == 0 or g != got[k - 1]]
+    assert order == ["refused", "chunk", "fused", "resident"], got
