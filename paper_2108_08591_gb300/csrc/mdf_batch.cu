@@ -361,10 +361,11 @@ __global__ void __launch_bounds__(T, SCHED == 3 ? batch_min_blocks<L, T>() : 0)
 // rows of odd boxes are not 8-byte aligned, so their pairs move as two
 // 4-byte accesses.
 //
-// Segment lengths: item lists are laid out for the whole batch at three
-// lengths (fuse_rows', half and a quarter); as cavities retire, the kernel
-// moves to a shorter one that still fits one wave, so that the last ones
-// spread over more SMs.
+// Item lists are laid out for the whole batch, for launches of two updates
+// (strips of 60 columns) and of four (56), at three segment lengths
+// (fuse_rows', half and a quarter); as cavities retire, the kernel moves to a
+// shorter one that still fits one wave, so that the last ones spread over more
+// SMs.
 struct BatchItem {
   int cav, strip, y0, y1;
 };
@@ -690,8 +691,8 @@ struct mdf_batch_s {
   int threads = 64;  // threads per block (kTile / threads nodes per thread)
   int sched = 3;     // 0: round-robin, 1: contiguous runs, 2: neighbour waits, 3: claimed tail
   bool fuse = false; // runs go by fused launches (D2Q5, d + 1 sets, no schedule of the caller's own)
-  BatchItems items{};
-  BatchItem *item_mem = nullptr;
+  BatchItems items[2] = {};  // of launches of two and of four updates
+  BatchItem *item_mem[2] = {};
   int seats = 0;     // CTAs of the resident kernel's launch (0: the batch does not go that way)
   bool seat_pair = false;
   int seat_threads = 0;
@@ -827,9 +828,11 @@ cudaError_t max_grid(mdf_batch_t b, int threads, int sched, int *grid) {
 
 // The item lists of the fused kernel (see BatchItems).  On an error the batch
 // keeps to the persistent kernel.
+template <int K>
 cudaError_t build_items(mdf_batch_t b) {
-  constexpr int K = 4, OUT = fuse_out<K>();
-  static_assert(fuse_out<2>() >= OUT, "the strips of four updates serve two as well");
+  constexpr int OUT = fuse_out<K>();
+  BatchItems &items = b->items[K / 4];
+  BatchItem *&mem = b->item_mem[K / 4];
   constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, D2Q5::Q>() * sizeof(float2);
   int per = 0, nmax = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_fused<K, false>, 32 * kFuseWarps, smem);
@@ -852,23 +855,24 @@ cudaError_t build_items(mdf_batch_t b) {
       for (int y = 0; y < N; y += rows)
         for (int s = 0; s * OUT < N; ++s) all.push_back({c, s, y, std::min(N, y + rows)});
     }
-    b->items.n[l] = (int)(all.size() - first[l]);
+    items.n[l] = (int)(all.size() - first[l]);
   }
-  b->items.wave = std::max(b->items.n[0], 4 * kSMs);
-  e = cudaMalloc(&b->item_mem, all.size() * sizeof(BatchItem));
+  items.wave = std::max(items.n[0], 4 * kSMs);
+  e = cudaMalloc(&mem, all.size() * sizeof(BatchItem));
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->item_mem, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(mem, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // `all` leaves scope
-  for (int l = 0; l < kItemLists; ++l) b->items.list[l] = b->item_mem + first[l];
+  for (int l = 0; l < kItemLists; ++l) items.list[l] = mem + first[l];
   return e;
 }
 
 template <int K, bool SAVE>
 cudaError_t launch_fused_t(mdf_batch_t b, int cur, int tk, int all) {
   constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, D2Q5::Q>() * sizeof(float2);
-  const int most = std::max(b->items.n[0], std::max(b->items.n[1], b->items.n[2]));
+  const BatchItems &items = b->items[K / 4];
+  const int most = std::max(items.n[0], std::max(items.n[1], items.n[2]));
   k_batch_fused<K, SAVE><<<(unsigned)((most + kFuseWarps - 1) / kFuseWarps), 32 * kFuseWarps, smem, b->stream>>>(
-      b->B, b->items, cur, tk, all);
+      b->B, items, cur, tk, all);
   return cudaGetLastError();
 }
 cudaError_t launch_fused(mdf_batch_t b, int K, int cur, int tk, bool save, int all) {
@@ -1116,7 +1120,7 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
   // what only the fused and the resident launches need does not fail the
   // batch: without it the next slower path takes its updates
   if (e == cudaSuccess && d == 2 && b->with_rho) {
-    b->fuse = build_items(b) == cudaSuccess;
+    b->fuse = build_items<2>(b) == cudaSuccess && build_items<4>(b) == cudaSuccess;
     if (!b->fuse || build_seats(b) != cudaSuccess) cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -1139,8 +1143,8 @@ void mdf_batch_destroy(mdf_batch_t b) {
   cudaFree(B.f[0]); cudaFree(B.f[1]); cudaFree((void *)B.cav); cudaFree((void *)B.tile_cav);
   cudaFree(B.live); cudaFree(B.n_live); cudaFree(B.usave); cudaFree(B.part); cudaFree(B.badtile);
   cudaFree(B.status); cudaFree(B.steps); cudaFree(B.res); cudaFree(B.bar); cudaFree(B.err);
-  cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem);
-  cudaFree(b->seat_mem); cudaFree(b->stage);
+  cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem[0]);
+  cudaFree(b->item_mem[1]); cudaFree(b->seat_mem); cudaFree(b->stage);
   cudaFreeHost(b->host_live);
   delete b;
 }

@@ -35,6 +35,7 @@ class Fake:
             fn = getattr(self.lib, name)
             fn.restype, fn.argtypes = res, args
         self.lib.fake_launch.restype = ctypes.c_char_p
+        self.lib.fake_watched.restype = ctypes.c_void_p
         self.lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double, ctypes.c_double]
 
     def launches(self):
@@ -46,6 +47,9 @@ class Fake:
             out.append((name, *(x.value for x in v)))
         self.lib.fake_clear()
         return out
+
+    def watched(self, ctype):
+        return ctype.from_buffer_copy(ctypes.string_at(self.lib.fake_watched(), ctypes.sizeof(ctype)))
 
     def lattice(self, shape, storage="f32", **opts):
         h = ctypes.c_void_p()

@@ -35,6 +35,9 @@ std::vector<Launch> g_log;
 std::vector<Cost> g_costs;
 std::map<cudaEvent_t, double> g_events;
 double g_now = 0.0;       // us
+std::string g_watch;      // kernel whose argument g_watch_arg is copied at each launch
+int g_watch_arg = 0;
+std::vector<char> g_watched;
 int g_clusters = 9;       // clusters that the device holds at once
 int g_fail_clusters = 0;  // cluster queries to fail
 int g_fail_malloc = 0;    // the allocation to fail, counted from now (0: none)
@@ -44,7 +47,7 @@ cudaStream_t g_stream;
 
 int attr(const void *f, int a) { return g_attr[{g_device, f}][a]; }
 
-cudaError_t record(const void *f, dim3 grid, dim3 block, size_t smem, unsigned cluster) {
+cudaError_t record(const void *f, dim3 grid, dim3 block, size_t smem, unsigned cluster, void **args) {
   if (smem > 48 * 1024 && (size_t)attr(f, cudaFuncAttributeMaxDynamicSharedMemorySize) < smem)
     return cudaErrorInvalidValue;
   if (cluster > 8 && !attr(f, cudaFuncAttributeNonPortableClusterSizeAllowed)) return cudaErrorInvalidClusterSize;
@@ -56,6 +59,8 @@ cudaError_t record(const void *f, dim3 grid, dim3 block, size_t smem, unsigned c
       break;
     }
   ++g_launched[f];
+  if (!g_watch.empty() && g_names[f].find(g_watch) != std::string::npos)
+    std::memcpy(g_watched.data(), args[g_watch_arg], g_watched.size());
   return cudaSuccess;
 }
 
@@ -81,6 +86,12 @@ void fake_clusters(int n) { g_clusters = n; }
 void fake_fail_clusters(int n) { g_fail_clusters = n; }
 void fake_fail_malloc(int n) { g_fail_malloc = n; }
 void fake_cost(const char *name, double us, double first) { g_costs.push_back({name, us, first}); }
+void fake_watch(const char *name, int arg, int bytes) {
+  g_watch = name;
+  g_watch_arg = arg;
+  g_watched.assign(bytes, 0);
+}
+const char *fake_watched() { return g_watched.data(); }
 void fake_clear() { g_log.clear(); }
 int fake_launches() { return (int)g_log.size(); }
 const char *fake_launch(int k, int *device, unsigned *grid, unsigned *block, unsigned *cluster) {
@@ -123,16 +134,16 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
   return cudaSuccess;
 }
 static cudaError_t g_last = cudaSuccess;
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **, size_t smem, cudaStream_t) {
-  const cudaError_t e = record(k, grid, block, smem, 1);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t) {
+  const cudaError_t e = record(k, grid, block, smem, 1, args);
   if (e != cudaSuccess) g_last = e;
   return e;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {
   unsigned cluster = 1;
   for (unsigned k = 0; k < c->numAttrs; ++k)
     if (c->attrs[k].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[k].val.clusterDim.x;
-  const cudaError_t e = record(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster);
+  const cudaError_t e = record(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster, args);
   if (e != cudaSuccess) g_last = e;
   return e;
 }

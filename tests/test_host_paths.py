@@ -92,3 +92,33 @@ def test_batch_falls_back_where_its_faster_path_cannot_be_set_up(fake):
     # the state's own, the lists of fused launches, the seats on chip, none
     order = [g for k, g in enumerate(got) if k == 0 or g != got[k - 1]]
     assert order == ["refused", "chunk", "fused", "resident"], got
+
+
+class _Items(ctypes.Structure):  # of the fused batch kernel: lists, their lengths
+    _fields_ = [("list", ctypes.c_void_p * 3), ("n", ctypes.c_int * 3), ("wave", ctypes.c_int)]
+
+
+@pytest.mark.parametrize("sides", [[300] * 4, [240, 175], [113, 267, 56], [870, 600], [61, 1100], [1921, 2]])
+@pytest.mark.parametrize("K", [2, 4])
+def test_fused_batch_items_cover_every_box_once(fake, sides, K):
+    """Each list of a fused launch of K updates covers every node once, with no
+    strip (64 columns less the K lost on each side) beyond its box."""
+    lib, out = fake.lib, {2: 60, 4: 56}[K]
+    lib.fake_clusters(0)  # boxes that would fit on chip as well
+    b = fake.batch(sides)
+    lib.fake_watch(b"k_batch_fusedILi%d" % K, 1, ctypes.sizeof(_Items))
+    # 16 updates make launches of the batch's depth, a period of 6 one of the other
+    assert lib.mdf_batch_step(b, 18) == _lib.OK
+    st = [np.zeros(len(sides), t) for t in (np.int64, np.int32, np.float64)]
+    lib.mdf_batch_run(b, 1e-8, 6, 6, *(v.ctypes.data for v in st))
+    it = fake.watched(_Items)
+    assert it.n[0] > 0
+    for l in range(3):
+        items = np.ctypeslib.as_array((ctypes.c_int * (4 * it.n[l])).from_address(it.list[l])).reshape(-1, 4)
+        cover = [np.zeros((N, N), np.int8) for N in sides]
+        for c, s, y0, y1 in items:
+            assert s * out < sides[c], (l, c, s)
+            assert 0 <= y0 < y1 <= sides[c]
+            cover[c][y0:y1, s * out:(s + 1) * out] += 1
+        assert all((v == 1).all() for v in cover), l
+    lib.mdf_batch_destroy(b)
