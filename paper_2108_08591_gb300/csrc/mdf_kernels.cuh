@@ -748,7 +748,12 @@ __device__ __forceinline__ TC geq_v(int alpha, int i, const TC (&u)[L::D], TC Pp
   if (alpha == 0) return wi * cu * ics2;
   const TC ua = u[alpha - 1];
   const TC cP = L::c(i, alpha - 1) > 0 ? Pp : (L::c(i, alpha - 1) < 0 ? -Pp : TC(0));
-  return wi * (ua + (cu * ua + cP) * ics2);
+  // 1 / c_s^2 is a power of two on D3Q7 and D2Q4: its product is exact, so one
+  // FMA rounds as the product and the sum do
+  if constexpr (std::is_same<TC, double>::value && (L::CS2 == 0.25 || L::CS2 == 0.5))
+    return wi * __fma_rn(cu * ua + cP, ics2, ua);
+  else
+    return wi * (ua + (cu * ua + cP) * ics2);
 }
 
 // First-order non-equilibrium part of set alpha along c_i at node n from
@@ -804,6 +809,14 @@ template <class TS> __device__ __forceinline__ typename ComputeOf<TS>::T round_t
 // and direction, is most of the kernel; with a run-time test in place of it
 // 256^3 took 728 us, now 507, 4096^2 451 -> 292 (floor 222), and
 // 19 x 202 x 226 FP16 with walls 250 -> 60.
+//
+// FP64 lattices are bound by the FP64 pipe, and the order of the loops decides
+// how much of it the compiler shares between populations: set by set without
+// a gradient, direction by direction with one.  190 x 202 x 178, us, set by set
+// against direction by direction: D3Q7 2038 / 3090 (both with the FMA of
+// geq_v; without it 2251 / 3587, and 3443 with a run-time loop over the sets),
+// without the alpha = 0 set 1800 / 2851; D3Q6 2050 / 3091; with a gradient 5739 /
+// 3580.
 template <class L, class TS, bool WALLS, bool GRAD>
 __global__ void __launch_bounds__(kMaxBlock) k_init(const DevArgs A) {
   using TC = typename ComputeOf<TS>::T;
@@ -818,49 +831,61 @@ __global__ void __launch_bounds__(kMaxBlock) k_init(const DevArgs A) {
   TC u[D], Pp;
   seed_at<L, TC>(A, N, n, u, Pp);
   TS *fout = static_cast<TS *>(A.fout);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int o = L::opp(i);
-    const bool wall = WALLS && moving<L>(i) && ((m >> o) & 1);  // arrives through a wall
-    // x - c_i as an offset from this node
+  // x - c_i as an offset from this node
+  auto pushed = [&](int i) {
     long long src = idx;
     if (L::c(i, 0) != 0) src += wrap(x - L::c(i, 0), A.nx) - x;
     if (L::c(i, 1) != 0) src += (long long)(wrap(y - L::c(i, 1), A.ny) - y) * A.px;
     if (D == 3 && L::c(i, 2) != 0) src += (long long)(wrap(z - L::c(i, 2), A.nz) - z) * A.ny * A.px;
-#pragma unroll
-    for (int alpha = 0; alpha <= D; ++alpha) {
-      if (alpha == 0 && !A.with_rho) continue;
-      TS *const set = fout + (long long)(alpha - 1 + A.with_rho) * Q * A.plane;
-      const TC Fa = (A.scheme2 && alpha >= 1)
-                        ? __ldg(static_cast<const TC *>(A.force) + (alpha - 1) * A.plane + idx) : TC(0);
-      TC v;
-      long long dst;
-      const bool lid = WALLS && wall && alpha >= 1 && o == L::UP && (m & 0x80u);
-      if (A.aa && !lid) {  // in-place AA, even layout: slot i of x holds the arriving f_i(x)
-        v = geq_v<L, TC>(alpha, i, u, Pp);
-        if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
-        if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
+    return src;
+  };
+  auto population = [&](int i, int alpha, long long src) {
+    if (alpha == 0 && !A.with_rho) return;
+    const int o = L::opp(i);
+    const bool wall = WALLS && moving<L>(i) && ((m >> o) & 1);  // arrives through a wall
+    TS *const set = fout + (long long)(alpha - 1 + A.with_rho) * Q * A.plane;
+    const TC Fa = (A.scheme2 && alpha >= 1)
+                      ? __ldg(static_cast<const TC *>(A.force) + (alpha - 1) * A.plane + idx) : TC(0);
+    TC v;
+    long long dst;
+    const bool lid = WALLS && wall && alpha >= 1 && o == L::UP && (m & 0x80u);
+    if (A.aa && !lid) {  // in-place AA, even layout: slot i of x holds the arriving f_i(x)
+      v = geq_v<L, TC>(alpha, i, u, Pp);
+      if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+      if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
+      dst = i * A.plane + idx;
+    } else if (wall) {  // stored in slot o at x, negated by the bounce-back
+      v = -geq_v<L, TC>(alpha, i, u, Pp);
+      if (GRAD) v -= narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+      if (lid) v += TC(2.0 * L::w(o) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
+      if (A.scheme2 && alpha >= 1) v = v + TC(0.5 * L::w(o)) * Fa;
+      dst = o * A.plane + idx;
+      if (A.aa) {
+        // the value the pull stream's first bounce-back delivers (the lid
+        // term does not cancel exactly in rounded arithmetic), so that
+        // both layouts start from the same state
+        v = -round_to<TS>(v) + TC(2.0 * L::w(i) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
         dst = i * A.plane + idx;
-      } else if (wall) {  // stored in slot o at x, negated by the bounce-back
-        v = -geq_v<L, TC>(alpha, i, u, Pp);
-        if (GRAD) v -= narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
-        if (lid) v += TC(2.0 * L::w(o) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
-        if (A.scheme2 && alpha >= 1) v = v + TC(0.5 * L::w(o)) * Fa;
-        dst = o * A.plane + idx;
-        if (A.aa) {
-          // the value the pull stream's first bounce-back delivers (the lid
-          // term does not cancel exactly in rounded arithmetic), so that
-          // both layouts start from the same state
-          v = -round_to<TS>(v) + TC(2.0 * L::w(i) * A.lid_u[alpha >= 1 ? alpha - 1 : 0]);
-          dst = i * A.plane + idx;
-        }
-      } else {  // stored in slot i at x - c_i
-        v = geq_v<L, TC>(alpha, i, u, Pp);
-        if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
-        if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
-        dst = i * A.plane + src;
       }
-      Codec<TS>::store(set + dst, v);
+    } else {  // stored in slot i at x - c_i
+      v = geq_v<L, TC>(alpha, i, u, Pp);
+      if (GRAD) v += narrow_to<TC>(fne_at<L>(A, N, n, alpha, i));
+      if (A.scheme2 && alpha >= 1) v = v - TC(0.5 * L::w(i)) * Fa;
+      dst = i * A.plane + src;
+    }
+    Codec<TS>::store(set + dst, v);
+  };
+  if constexpr (std::is_same<TC, double>::value && !GRAD) {
+#pragma unroll
+    for (int alpha = 0; alpha <= D; ++alpha)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) population(i, alpha, pushed(i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const long long src = pushed(i);
+#pragma unroll
+      for (int alpha = 0; alpha <= D; ++alpha) population(i, alpha, src);
     }
   }
 }
