@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_update_aa(const DevArgs A) {
   if (MODE != MODE_STEP) {
     const long long N = (long long)A.nx * A.ny * A.nz;
     const long long n = ((long long)z * A.ny + y) * A.nx + x;
-    write_fields<L, TC>(A, n, N, g, h, F);
+    write_fields<L, TC, MODE == MODE_STEP_FIELDS && sizeof(TS) == 8>(A, n, N, g, h, F);
     if (MODE == MODE_FIELDS) return;
   }
 

@@ -91,6 +91,21 @@ __device__ __forceinline__ void pull_set(const DevArgs &A, const TS *__restrict_
                            A.lid_u, g);
 }
 
+// Whether an update that writes fields forms the moments once for both (see
+// write_fields).  FP64 is bound by the FP64 pipe and always does.  The others
+// are bound by memory latency, and it is a matter of the registers that each
+// form leaves; us per update, shared / apart: D2Q5 FP16 with walls at 2050 x
+// 1998 107.5 / 114.2, BF16 107.1 / 120.3, FP32 125.6 / 115.1, FP16 without walls
+// 88.2 / 81.3; at 190 x 202 x 178 with walls D3Q7 FP32 377 / 401, FP16 405 / 424,
+// D3Q6 FP32 335 / 353, FP16 333 / 315, without walls D3Q7 FP16 251 / 238; FP64
+// D3Q7 4205 / 4583.
+template <class L, class TS, bool WALLS> constexpr bool shares_moments() {
+  if (sizeof(TS) == 8) return true;
+  if (!WALLS) return false;
+  if (L::D == 2) return L::Q == 5 && sizeof(TS) == 2;
+  return L::Q == 7 || sizeof(TS) == 4;
+}
+
 // Derived fields of Eq. 2-7, 3-15 .. 3-19 at one node from the pulled
 // (pre-collision) shifted populations, computed in the compute type TC and
 // written as FP64.  gv: the d velocity sets; h: the alpha = 0 set (ignored
@@ -100,7 +115,11 @@ __device__ __forceinline__ void pull_set(const DevArgs &A, const TS *__restrict_
 // sizes; the FP32 storage rounding of g dominates the error.  (GB300's FP64
 // throughput is too low for FP64 arithmetic here to stay HBM-bound; the
 // widening to FP64 is built on the integer pipe, leaving two FP64 adds.)
-template <class L, class TC>
+//
+// SHARED: the moments written as node_moments writes them, so that an update
+// that also collides forms them once; otherwise with sums that start from 0
+// (the same values), which the compiler keeps apart.
+template <class L, class TC, bool SHARED = false>
 __device__ __forceinline__ void write_fields(const DevArgs &A, long long n, long long N,
                                              const TC (&gv)[L::D][L::Q], const TC (&h)[L::Q],
                                              const TC (&F)[L::D]) {
@@ -108,33 +127,33 @@ __device__ __forceinline__ void write_fields(const DevArgs &A, long long n, long
   TC u[D], J[D][D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    TC s = TC(0);
+    TC s = SHARED ? gv[a][0] : TC(0);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) s += gv[a][i];
+    for (int i = SHARED ? 1 : 0; i < Q; ++i) s += gv[a][i];
     u[a] = A.scheme2 ? s + TC(0.5) * F[a] : s;  // Eq. 2-7a under Scheme II
 #pragma unroll
     for (int b = 0; b < D; ++b) {
-      TC t = TC(0);
+      TC t = TC(0), p{}, m{};  // p, m: the populations along +e_b and -e_b
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        if (L::c(i, b) > 0) t += gv[a][i];
-        if (L::c(i, b) < 0) t -= gv[a][i];
+        if (L::c(i, b) > 0) { t += gv[a][i]; p = gv[a][i]; }
+        if (L::c(i, b) < 0) { t -= gv[a][i]; m = gv[a][i]; }
       }
-      J[a][b] = t;  // sum_i c_{i,b} g_{i,a}
+      J[a][b] = SHARED ? p - m : t;  // sum_i c_{i,b} g_{i,a}
     }
   }
-  TC tr = TC(0), usq = TC(0);
+  TC tr = SHARED ? J[0][0] : TC(0), usq = SHARED ? u[0] * u[0] : TC(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) { tr += J[a][a]; usq += u[a] * u[a]; }
+  for (int a = SHARED ? 1 : 0; a < D; ++a) { tr += J[a][a]; usq += u[a] * u[a]; }
   const TC Pp = (tr - usq) * TC(1.0 / D);  // Eq. 3-15, P' = P - P0, R = 0
   if (A.P) A.P[n] = 1.0 + widen_f32(Pp);
   if (A.u)
 #pragma unroll
     for (int a = 0; a < D; ++a) A.u[a * N + n] = widen_f32(u[a]);
   if (A.rho && A.with_rho) {
-    TC s = TC(0);
+    TC s = SHARED ? h[0] : TC(0);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) s += h[i];
+    for (int i = SHARED ? 1 : 0; i < Q; ++i) s += h[i];
     A.rho[n] = 1.0 + widen_f32(s);
   }
   if (!(A.G || A.div || A.S || A.sigma || A.omega)) return;
@@ -309,7 +328,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_update(const DevArgs A) {
   if (MODE != MODE_STEP) {
     const long long N = (long long)A.nx * A.ny * A.nz;
     const long long n = ((long long)z * A.ny + y) * A.nx + x;
-    write_fields<L, TC>(A, n, N, g, h, F);
+    write_fields<L, TC, MODE == MODE_STEP_FIELDS && shares_moments<L, TS, WALLS>()>(A, n, N, g, h, F);
     if (MODE == MODE_FIELDS) return;
   }
 
