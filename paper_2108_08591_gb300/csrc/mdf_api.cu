@@ -93,7 +93,10 @@ int default_block(int d, int storage) {
 // one busy warp: blocks of two warps then put all busy warps on the same two
 // of an SM's four schedulers, blocks of three do not (29 x 124 x 157 FP16:
 // 37 us with 64, 21 with 96, 23 with 128; FP32 with 32 nodes a row 41 / 27 /
-// 29; with 40 nodes 42 / 43 / 45).
+// 29; with 40 nodes 42 / 43 / 45).  Walled 2D equilibrium-shifted lattices keep
+// their default of 64: wider blocks fit some rows better and are slower all the same
+// (FP16, 2050 x 1998 76.3 us with 64, 79.1 with 96; 2098 x 2000 77.8 / 80.0;
+// 1538 x 1500 47.1 / 49.6; without walls 67.0 / 66.1, 67.7 / 67.4, 41.0 / 41.1).
 int fit_block(int threads, int dflt, int least) {
   const auto padded = [&](int b) { return (threads + b - 1) / b * b; };
   int best = dflt;
@@ -430,9 +433,10 @@ mdf_status mdf_create(mdf_t *out, const mdf_grid *g, int d, const mdf_rates *r,
   h->vx = opts.vx ? opts.vx : (h->inplace ? default_vx_aa(d, h->storage) : default_vx(d, h->storage));
   h->vx = std::min(h->vx, max_vx(d, h->storage, h->inplace));
   const int row_threads = h->nx % h->vx == 0 ? h->nx / h->vx : h->nx;
+  const int dflt = h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage);
+  const int least = d == 3 && !eq_storage(h->storage) && row_threads == h->nx && h->nx <= 32 ? 96 : 64;
   h->block = opts.block ? opts.block
-                        : fit_block(row_threads, h->inplace ? default_block_aa(d, h->storage) : default_block(d, h->storage),
-                                    d == 3 && !eq_storage(h->storage) && row_threads == h->nx && h->nx <= 32 ? 96 : 64);
+             : d == 2 && eq_storage(h->storage) && h->walls ? dflt : fit_block(row_threads, dflt, least);
   // a caller's own launch shape is that of the one-update kernel
   const bool can_fuse = h->storage == MDF_F32 && h->with_rho && !h->inplace && !opts.vx &&
                         !opts.block && h->plane < (1LL << 31) - 64;

@@ -4,7 +4,6 @@ GPU."""
 import ctypes
 import glob
 import os
-import shutil
 import subprocess
 
 from paper_2108_08591_gb300 import _build, _lib
@@ -26,17 +25,24 @@ def link(out):
 
 
 class Fake:
-    """One copy of the library and its stand-in (each copy has its own state)."""
+    """The library on the stand-in.  What the library keeps per device stays for
+    the life of the process, so every test starts on a device of its own."""
 
-    def __init__(self, linked, path):
-        shutil.copy(linked, path)
-        self.lib = ctypes.CDLL(str(path))
+    def __init__(self, linked):
+        self.device = -1
+        self.lib = ctypes.CDLL(str(linked))
         for name, (res, args) in _lib.SIGNATURES.items():
             fn = getattr(self.lib, name)
             fn.restype, fn.argtypes = res, args
         self.lib.fake_launch.restype = ctypes.c_char_p
         self.lib.fake_watched.restype = ctypes.c_void_p
         self.lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double, ctypes.c_double]
+
+    def new_device(self):
+        """Make a device that nothing has been launched on the current one."""
+        self.device += 1
+        self.lib.fake_set_device(self.device)
+        return self.device
 
     def launches(self):
         """Recorded launches as (kernel, device, blocks, threads, cluster)."""
@@ -56,7 +62,10 @@ class Fake:
         g = _lib.Grid(*shape, *([1] if len(shape) == 2 else []))
         r = _lib.Rates(1.0, 1.7, -1.0)
         o = _lib.Opts(_lib.STORAGE[storage], 1, None, *(opts.get(k, 0) for k in ("vx", "block", "q", "inplace")))
-        st = self.lib.mdf_create(ctypes.byref(h), ctypes.byref(g), len(shape), ctypes.byref(r), None, ctypes.byref(o))
+        bc = _lib.BC()
+        bc.wall[:] = [int(opts.get("wall", False) and k < len(shape)) for k in range(3)]
+        st = self.lib.mdf_create(ctypes.byref(h), ctypes.byref(g), len(shape), ctypes.byref(r), ctypes.byref(bc),
+                                 ctypes.byref(o))
         assert st == _lib.OK, self.lib.mdf_last_error(None)
         return h
 

@@ -81,6 +81,14 @@ CUresult encode(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cu
 extern "C" {
 
 // ---- what the tests set and read
+void fake_reset() {
+  g_log.clear();
+  g_costs.clear();
+  g_launched.clear();
+  g_watch.clear();
+  g_clusters = 9;
+  g_fail_clusters = g_fail_malloc = 0;
+}
 void fake_set_device(int d) { g_device = d; }
 void fake_clusters(int n) { g_clusters = n; }
 void fake_fail_clusters(int n) { g_fail_clusters = n; }

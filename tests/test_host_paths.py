@@ -13,16 +13,17 @@ pytestmark = pytest.mark.skipif(not shutil.which("g++"), reason="g++ not found")
 
 @pytest.fixture(scope="module")
 def linked(tmp_path_factory):
-    from _fakecuda import link
+    from _fakecuda import Fake, link
     out = tmp_path_factory.mktemp("fake") / "libmdf_fake.so"
     link(out)
-    return out
+    return Fake(out)
 
 
 @pytest.fixture
-def fake(linked, tmp_path):
-    from _fakecuda import Fake
-    return Fake(linked, tmp_path / "libmdf_fake.so")
+def fake(linked):
+    linked.lib.fake_reset()
+    linked.new_device()
+    return linked
 
 
 def test_kernel_attributes_are_set_on_every_device(fake):
@@ -32,7 +33,7 @@ def test_kernel_attributes_are_set_on_every_device(fake):
     conv = [np.zeros(8 * 8 * 64 * 64, np.float32) for _ in range(3)]
     x, w, y = ((a.ctypes.data + 63) // 64 * 64 for a in conv)
     got = []
-    for dev in (0, 1):
+    for dev in (fake.device, fake.new_device()):
         lib.fake_set_device(dev)
         for shape, q in (((64, 64), 0), ((40, 60), 4), ((60, 60, 200), 0), ((60, 60, 200), 6)):
             h = fake.lattice(shape, q=q)
@@ -122,3 +123,16 @@ def test_fused_batch_items_cover_every_box_once(fake, sides, K):
             cover[c][y0:y1, s * out:(s + 1) * out] += 1
         assert all((v == 1).all() for v in cover), l
     lib.mdf_batch_destroy(b)
+
+
+@pytest.mark.parametrize("storage", ["f16eq", "bf16eq"])
+@pytest.mark.parametrize("shape,walled,open_", [((2050, 1998), 64, 96), ((2098, 40), 64, 96), ((1024, 64), 64, 64)])
+def test_walled_2d_equilibrium_shifted_rows_keep_their_block(fake, storage, shape, walled, open_):
+    got = []
+    for wall in (True, False):
+        h = fake.lattice(shape, storage, wall=wall)
+        fake.launches()
+        assert fake.lib.mdf_step(h, 1) == _lib.OK
+        got += [threads for n, _, _, threads, _ in fake.launches() if "k_update_eq" in n]
+        fake.lib.mdf_destroy(h)
+    assert got == [walled, open_]
