@@ -423,8 +423,8 @@ mdf_status mdf_batch_info(mdf_batch_t b, long long *nodes, int *tiles, int *grid
  * (default 4e9, about 2 s).  A barrier that waits longer makes every block of
  * the persistent kernel return and the call report MDF_ETIMEOUT; the batch
  * state is then undefined until the next mdf_batch_init.  Fused launches (see
- * mdf_batch_set_schedule) have no barrier; a limit keeps to the persistent
- * kernel. */
+ * mdf_batch_set_schedule) have no barrier; a limit other than the default
+ * keeps to the persistent kernel. */
 mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles);
 
 /* Scheduling of the batch's persistent kernel (mdf_batch_set_schedule,
@@ -445,8 +445,8 @@ mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles);
  * computes the same bits; only the speed differs.  MDF_EINVAL for other
  * values.  A new batch starts with 64 threads, schedule 3 and the largest
  * grid; a 2D one with the alpha = 0 set advances by ordinary launches of
- * several updates each instead (the same bits), until this call or
- * mdf_batch_set_timeout asks for the persistent kernel, or
+ * several updates each instead (the same bits), until this call or a limit
+ * (mdf_batch_set_timeout) asks for the persistent kernel, or
  * mdf_batch_autotune finds it faster. */
 mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sched);
 
@@ -456,8 +456,11 @@ mdf_status mdf_batch_get_schedule(mdf_batch_t b, int *threads, int *grid, int *s
 /* mdf_batch_autotune -- time `reps` (rounded up to even; < 2: 20) steps of
  * every schedule candidate (threads 128 / 64 / 32, schedules 0 .. 3, grids
  * of 1, 2, 3, 4, 6, 8, 12, 16, 24, 32 blocks per SM up to the co-resident limit) on
- * the current state with all cavities live, keep the fastest and restore
- * the state (bit for bit; step counts and statuses are not touched).
+ * the current state with all cavities live, keep the fastest, compare it over
+ * max(reps, 100) steps with the fused launches where the batch has them and
+ * no limit keeps it from them, choose the faster path (also after
+ * mdf_batch_set_schedule) and restore the state (bit for bit; step counts and
+ * statuses are not touched).
  * Needs one extra population pool of device memory while it runs. */
 mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads, int *grid, int *sched);
 

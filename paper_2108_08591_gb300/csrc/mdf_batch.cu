@@ -690,7 +690,10 @@ struct mdf_batch_s {
   int grid = 0;      // blocks of the persistent kernel
   int threads = 64;  // threads per block (kTile / threads nodes per thread)
   int sched = 3;     // 0: round-robin, 1: contiguous runs, 2: neighbour waits, 3: claimed tail
-  bool fuse = false; // runs go by fused launches (D2Q5, d + 1 sets, no schedule of the caller's own)
+  bool can_fuse = false;   // runs can go by fused or resident launches (D2Q5, d + 1 sets)
+  bool own_shape = false;  // they do not: a schedule was set, or autotuning found one faster
+  bool own_limit = false;  // nor with a barrier limit of the caller's own
+  bool fuse() const { return can_fuse && !own_shape && !own_limit; }
   BatchItems items[2] = {};  // of launches of two and of four updates
   BatchItem *item_mem[2] = {};
   int seats = 0;     // CTAs of the resident kernel's launch (0: the batch does not go that way)
@@ -712,6 +715,8 @@ struct mdf_batch_s {
 namespace {
 
 thread_local std::string g_batch_error = "no error";
+
+constexpr long long kDefaultTimeout = 4000000000LL;  // ~2 s at the GB300 clock
 
 mdf_status bfail(mdf_batch_t b, mdf_status st, const char *fmt, ...) {
   char msg[512];
@@ -954,6 +959,27 @@ int fused_depth(mdf_batch_t b) {
   return nodes >= 750000 ? 4 : 2;
 }
 
+// Enqueue n >= 2 updates from buffer *cur by fused or resident launches, and
+// move *cur to their result; returns in *made how many (an odd last one is left
+// to the persistent kernel).
+cudaError_t enqueue_fused(mdf_batch_t b, int n, int *cur, int *made) {
+  cudaError_t e = cudaSuccess;
+  int k = 0;
+  if (b->seats) {
+    k = std::min(n, 1 << 14);
+    e = launch_resident(b, *cur, 0, k, false, 1);
+    *cur ^= 1;
+  } else {
+    for (const int depth = fused_depth(b); n - k >= 2 && e == cudaSuccess; *cur ^= 1) {
+      const int K = n - k >= 4 ? depth : 2;
+      e = launch_fused(b, K, *cur, k, false, 1);
+      k += K;
+    }
+  }
+  *made = k;
+  return e;
+}
+
 // An even number of launches of four and two updates that make `period`
 // (even, >= 4) updates, so that the state ends in the buffer it started in.
 cudaError_t fused_period(mdf_batch_t b, int period) {
@@ -1007,7 +1033,7 @@ mdf_status all_live(mdf_batch_t b) {
 
 template <class L>
 cudaError_t enqueue_period(mdf_batch_t b, int period, double tol, long long max_steps) {
-  cudaError_t e = b->fuse && period >= 4 ? fused_period(b, period) : launch_chunk<L>(b, period, 1);
+  cudaError_t e = b->fuse() && period >= 4 ? fused_period(b, period) : launch_chunk<L>(b, period, 1);
   if (e != cudaSuccess) return e;
   k_batch_tick<<<1, 1, 0, b->stream>>>(b->B.clock, period);
   const int cur_after = (b->cur + period) & 1;
@@ -1083,7 +1109,7 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
   B.ntiles = b->ntiles;
   B.with_rho = b->with_rho;
   for (int k = 0; k < 3; ++k) B.lid_u[k] = b->lid_u[k];
-  B.timeout = 4000000000LL;  // ~2 s at the GB300 clock
+  B.timeout = kDefaultTimeout;
   const size_t popb = sizeof(float) * (size_t)nsets * Q * (size_t)b->tot;
   std::vector<int> tile_cav(b->ntiles);
   for (int c = 0; c < n; ++c)
@@ -1120,8 +1146,8 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
   // what only the fused and the resident launches need does not fail the
   // batch: without it the next slower path takes its updates
   if (e == cudaSuccess && d == 2 && b->with_rho) {
-    b->fuse = build_items<2>(b) == cudaSuccess && build_items<4>(b) == cudaSuccess;
-    if (!b->fuse || build_seats(b) != cudaSuccess) cudaGetLastError();
+    b->can_fuse = build_items<2>(b) == cudaSuccess && build_items<4>(b) == cudaSuccess;
+    if (!b->can_fuse || build_seats(b) != cudaSuccess) cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
@@ -1282,20 +1308,9 @@ mdf_status mdf_batch_step(mdf_batch_t b, long long n) {
   if (st != MDF_OK) return st;
   const int chunk = 1 << 20;
   while (n > 0) {
-    const bool fused = b->fuse && n >= 2;
-    int s = (int)std::min<long long>(n, chunk), k = 0;
-    if (fused && b->seats) {
-      s = std::min(s, 1 << 14);
-      BCU(b, launch_resident(b, b->cur, 0, s, false, 1));
-      b->cur ^= 1;
-    } else if (fused) {
-      const int depth = fused_depth(b);
-      for (; s - k >= 2; b->cur ^= 1) {
-        const int K = s - k >= 4 ? depth : 2;
-        BCU(b, launch_fused(b, K, b->cur, k, false, 1));
-        k += K;
-      }
-      s = k;
+    int s = (int)std::min<long long>(n, chunk);
+    if (b->fuse() && n >= 2) {
+      BCU(b, enqueue_fused(b, s, &b->cur, &s));
     } else {
       BCU(b, b->d == 2 ? launch_chunk<D2Q5>(b, s, 0) : launch_chunk<D3Q7>(b, s, 0));
       b->cur = (b->cur + s) & 1;
@@ -1370,7 +1385,7 @@ mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles) {
   if (!b) return MDF_EINVAL;
   if (cycles < 0) return bfail(b, MDF_EINVAL, "timeout must be >= 0 cycles");
   b->B.timeout = cycles;
-  b->fuse = false;  // a limit of the caller's own is the persistent kernel's
+  b->own_limit = cycles != kDefaultTimeout;  // a limit is the persistent kernel's
   drop_graph(b);  // the captured kernels hold the old value
   return MDF_OK;
 }
@@ -1387,7 +1402,7 @@ mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sche
   b->threads = threads;
   b->sched = sched;
   b->grid = grid ? grid : gmax;
-  b->fuse = false;  // the caller's own launch shape is the persistent kernel's
+  b->own_shape = true;  // the caller's own launch shape is the persistent kernel's
   drop_graph(b);  // the captured launch holds the old shape
   return MDF_OK;
 }
@@ -1463,19 +1478,33 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
         }
       }
     }
-  bool fuse = b->fuse;
-  if (st == MDF_OK && fuse) {  // the fused launches against the best of them
-    cudaError_t e = cudaEventRecord(e0, b->stream);
-    if (b->seats && e == cudaSuccess) e = launch_resident(b, b->cur, 0, reps, false, 1);
-    const int depth = fused_depth(b);
-    for (int k = 0; k < reps && e == cudaSuccess && !b->seats; k += reps - k >= 4 ? depth : 2)
-      e = launch_fused(b, reps - k >= 4 ? depth : 2, b->cur, k, false, 1);
-    if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+  // The fused launches against the best of them: both over as many updates as
+  // a convergence period makes, after a launch that is not timed (the first
+  // one of a kernel loads it), the best of three in turn.
+  bool own_shape = b->own_shape;
+  if (st == MDF_OK && b->can_fuse && !b->own_limit) {
+    const int n = std::min(1 << 14, std::max(reps, 100));
+    float t[2] = {1e30f, 1e30f};  // persistent, fused
+    cudaError_t e = cudaSuccess;
+    b->threads = best_threads;
+    b->sched = best_sched;
+    b->grid = best_grid;
+    for (int k = 0; k < 8 && e == cudaSuccess; ++k) {
+      int cur = b->cur, made = 0;
+      e = cudaMemsetAsync(b->B.bar, 0, sizeof(unsigned int) * kBarWords, b->stream);
+      if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+      if (e == cudaSuccess) e = k & 1 ? enqueue_fused(b, n, &cur, &made) : launch_chunk<D2Q5>(b, n, 0);
+      if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+      float ms = 0.f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+      if (k >= 2) t[k & 1] = std::min(t[k & 1], ms);
+    }
+    int err = 0;
+    if (e == cudaSuccess) e = cudaMemcpy(&err, b->B.err, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) st = bfail(b, MDF_ECUDA, "autotune: %s", cudaGetErrorString(e));
-    fuse = ms < best;
+    else if (err) st = bfail(b, MDF_ETIMEOUT, "autotune: grid barrier timed out");
+    own_shape = t[0] < t[1];
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
@@ -1488,7 +1517,7 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
     b->threads = best_threads;
     b->sched = best_sched;
     b->grid = best_grid;
-    b->fuse = fuse;
+    b->own_shape = own_shape;
   } else {
     b->threads = old_threads;
     b->sched = old_sched;

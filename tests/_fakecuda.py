@@ -36,7 +36,7 @@ class Fake:
             fn.restype, fn.argtypes = res, args
         self.lib.fake_launch.restype = ctypes.c_char_p
         self.lib.fake_watched.restype = ctypes.c_void_p
-        self.lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double, ctypes.c_double]
+        self.lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double, ctypes.c_double, ctypes.c_int]
 
     def new_device(self):
         """Make a device that nothing has been launched on the current one."""

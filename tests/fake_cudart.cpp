@@ -25,6 +25,7 @@ struct Launch {
 struct Cost {
   std::string name;
   double us, first;
+  int arg;  // >= 0: `us` is per unit of this int argument
 };
 
 int g_device = 0;
@@ -55,7 +56,7 @@ cudaError_t record(const void *f, dim3 grid, dim3 block, size_t smem, unsigned c
   g_log.push_back({g_device, g_names[f], grid.x * grid.y * grid.z, block.x, cluster, smem});
   for (const Cost &c : g_costs)
     if (g_names[f].find(c.name) != std::string::npos) {
-      g_now += c.us + (g_launched[f] ? 0.0 : c.first);
+      g_now += c.us * (c.arg < 0 ? 1 : *static_cast<int *>(args[c.arg])) + (g_launched[f] ? 0.0 : c.first);
       break;
     }
   ++g_launched[f];
@@ -93,7 +94,7 @@ void fake_set_device(int d) { g_device = d; }
 void fake_clusters(int n) { g_clusters = n; }
 void fake_fail_clusters(int n) { g_fail_clusters = n; }
 void fake_fail_malloc(int n) { g_fail_malloc = n; }
-void fake_cost(const char *name, double us, double first) { g_costs.push_back({name, us, first}); }
+void fake_cost(const char *name, double us, double first, int arg) { g_costs.push_back({name, us, first, arg}); }
 void fake_watch(const char *name, int arg, int bytes) {
   g_watch = name;
   g_watch_arg = arg;

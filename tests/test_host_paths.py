@@ -136,3 +136,33 @@ def test_walled_2d_equilibrium_shifted_rows_keep_their_block(fake, storage, shap
         got += [threads for n, _, _, threads, _ in fake.launches() if "k_update_eq" in n]
         fake.lib.mdf_destroy(h)
     assert got == [walled, open_]
+
+
+@pytest.mark.parametrize("sides,kernel,per_update,arg", [([300, 240], "k_batch_fused", 2 * 5.0, -1),
+                                                         ([65, 97, 129], "k_batch_resident", 5.0, 4)])
+def test_batch_autotune_weighs_warm_kernels(fake, sides, kernel, per_update, arg):
+    """The first launch of a kernel loads it.  That does not count against the
+    fused or on-chip launches, which stay in use when they are the faster ones,
+    also after a schedule of the caller's own."""
+    lib = fake.lib
+    lib.fake_cost(kernel.encode(), per_update, 1e5, arg)
+    lib.fake_cost(b"k_batch_chunk", 10.0, 1e5, 2)  # us per update
+    b = fake.batch(sides)
+    assert lib.mdf_batch_autotune(b, 20, None, None, None) == _lib.OK
+    assert all(kernel in n for n in _step_kernels(fake, b))
+    assert lib.mdf_batch_set_schedule(b, 64, 0, 3) == _lib.OK
+    assert all("k_batch_chunk" in n for n in _step_kernels(fake, b))
+    assert lib.mdf_batch_autotune(b, 20, None, None, None) == _lib.OK
+    assert all(kernel in n for n in _step_kernels(fake, b))
+    lib.mdf_batch_destroy(b)
+
+
+def test_batch_autotune_keeps_the_persistent_kernel_where_it_is_faster(fake):
+    lib = fake.lib
+    lib.fake_cost(b"k_batch_fused", 2 * 12.0, 0.0, -1)
+    lib.fake_cost(b"k_batch_chunk", 10.0, 0.0, 2)
+    b = fake.batch([300, 240])
+    assert all("k_batch_fused" in n for n in _step_kernels(fake, b))
+    assert lib.mdf_batch_autotune(b, 20, None, None, None) == _lib.OK
+    assert all("k_batch_chunk" in n for n in _step_kernels(fake, b))
+    lib.mdf_batch_destroy(b)
