@@ -316,6 +316,23 @@ mdf_status mdf_load(mdf_t h, const char *path);
 /* mdf_info -- static facts about h (host struct). */
 mdf_status mdf_info(mdf_t h, mdf_info_t *out);
 
+/* How updates are launched. */
+#define MDF_PATH_SINGLE 0     /* one update per launch */
+#define MDF_PATH_FUSED 1      /* several updates per pass over memory */
+#define MDF_PATH_RESIDENT 2   /* the lattice stays on chip over the updates of a launch */
+#define MDF_PATH_PERSISTENT 3 /* batches: one persistent kernel with a grid barrier */
+#define MDF_PATH_DEFAULT (-1) /* batches: as a new batch chooses */
+typedef struct {
+    int path;           /* of the launches that make the most updates */
+    int updates;        /* updates of each of those */
+    long long launches; /* update-kernel launches in all */
+    int threads;        /* per block of those of `path` */
+} mdf_plan_t;
+
+/* mdf_plan -- how mdf_step(h, n) launches its n >= 0 updates (host struct).
+ * Every path gives the same bits. */
+mdf_status mdf_plan(mdf_t h, long long n, mdf_plan_t *out);
+
 /*
  * mdf_autotune -- measure the update kernel's launch shapes for this handle
  * (one node per thread and each vector width built for the storage type
@@ -450,7 +467,21 @@ mdf_status mdf_batch_set_timeout(mdf_batch_t b, long long cycles);
  * mdf_batch_autotune finds it faster. */
 mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sched);
 
-/* mdf_batch_get_schedule -- the launch shape in use (any pointer may be NULL). */
+/* mdf_batch_set_path -- MDF_PATH_PERSISTENT: advance by the persistent kernel
+ * with the schedule in use; MDF_PATH_DEFAULT: as a new batch does (a barrier
+ * limit other than the default still keeps to the persistent kernel).
+ * MDF_EINVAL for other values. */
+mdf_status mdf_batch_set_path(mdf_batch_t b, int path);
+
+/* mdf_batch_get_path -- the path in use, MDF_PATH_FUSED, MDF_PATH_RESIDENT or
+ * MDF_PATH_PERSISTENT, and the updates of a fused launch (0 on the others: a
+ * launch makes those of a call or period); either pointer may be NULL.  Chunks
+ * of fewer than two steps and periods of two go by the persistent kernel on
+ * every path. */
+mdf_status mdf_batch_get_path(mdf_batch_t b, int *path, int *updates);
+
+/* mdf_batch_get_schedule -- the launch shape of the persistent kernel, used on
+ * MDF_PATH_PERSISTENT (any pointer may be NULL). */
 mdf_status mdf_batch_get_schedule(mdf_batch_t b, int *threads, int *grid, int *sched);
 
 /* mdf_batch_autotune -- time `reps` (rounded up to even; < 2: 20) steps of

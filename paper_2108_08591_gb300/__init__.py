@@ -242,6 +242,14 @@ class Lattice:
     def load(self, path: str):
         self._check(self._lib.mdf_load(self._h, path.encode()))
 
+    def plan(self, n: int) -> Dict[str, object]:
+        """How step(n) launches its updates: the path ('single', 'fused' or
+        'resident') of the launches that make the most updates, the updates
+        and threads per block of those, and the launches in all."""
+        p = _lib.Plan()
+        self._check(self._lib.mdf_plan(self._h, int(n), ctypes.byref(p)))
+        return {"path": _lib.PATHS[p.path], "updates": p.updates, "launches": p.launches, "threads": p.threads}
+
     def autotune(self, reps: int = 10):
         """Measure the update kernel's launch shapes and keep the fastest;
         the lattice state is unchanged.  Returns (vx, block)."""
@@ -386,8 +394,23 @@ class CavityBatch:
         self._check(self._lib.mdf_batch_set_timeout(self._h, int(cycles)))
 
     def set_schedule(self, threads: int = 128, grid: int = 0, sched: int = 0):
-        """Launch shape of the persistent step kernel (see mdf_batch_set_schedule)."""
+        """Advance by the persistent kernel with this launch shape (see
+        mdf_batch_set_schedule); set_path('default') goes back."""
         self._check(self._lib.mdf_batch_set_schedule(self._h, int(threads), int(grid), int(sched)))
+
+    def set_path(self, path: str):
+        """'persistent': advance by the persistent kernel; 'default': as a new
+        batch does (see mdf_batch_set_path)."""
+        code = {"default": _lib.PATH_DEFAULT, "persistent": _lib.PATH_PERSISTENT}[path]
+        self._check(self._lib.mdf_batch_set_path(self._h, code))
+
+    @property
+    def path(self) -> Dict[str, object]:
+        """The path in use, 'fused', 'resident' (boxes stay on chip) or
+        'persistent', and the updates of a fused launch (else 0)."""
+        v, k = ctypes.c_int(), ctypes.c_int()
+        self._check(self._lib.mdf_batch_get_path(self._h, ctypes.byref(v), ctypes.byref(k)))
+        return {"path": _lib.PATHS[v.value], "updates": k.value}
 
     def schedule(self) -> Dict[str, int]:
         v = np.zeros(3, np.int32)
@@ -396,8 +419,10 @@ class CavityBatch:
         return {"threads": int(v[0]), "grid": int(v[1]), "sched": int(v[2])}
 
     def autotune(self, reps: int = 20) -> Dict[str, int]:
-        """Time every schedule on the current state, keep the fastest, restore
-        the state; returns the chosen {threads, grid, sched}."""
+        """Time every schedule of the persistent kernel on the current state,
+        compare the fastest with the fused launches, choose the faster path (see
+        `path`) and restore the state; returns the persistent kernel's best
+        {threads, grid, sched}."""
         v = np.zeros(3, np.int32)
         self._check(self._lib.mdf_batch_autotune(self._h, int(reps), v[0:].ctypes.data, v[1:].ctypes.data,
                                                  v[2:].ctypes.data))

@@ -52,6 +52,16 @@ class Info(ctypes.Structure):
                 ("vx", ctypes.c_int), ("block", ctypes.c_int)]
 
 
+# MDF_PATH_* of a plan or batch
+PATHS = {0: "single", 1: "fused", 2: "resident", 3: "persistent"}
+PATH_DEFAULT, PATH_PERSISTENT = -1, 3
+
+
+class Plan(ctypes.Structure):
+    _fields_ = [("path", ctypes.c_int), ("updates", ctypes.c_int), ("launches", ctypes.c_longlong),
+                ("threads", ctypes.c_int)]
+
+
 H = ctypes.c_void_p
 DP = ctypes.c_void_p  # double* (host or device address)
 
@@ -84,6 +94,7 @@ SIGNATURES = {
     "mdf_save": (ctypes.c_int, [H, ctypes.c_char_p]),
     "mdf_load": (ctypes.c_int, [H, ctypes.c_char_p]),
     "mdf_info": (ctypes.c_int, [H, ctypes.POINTER(Info)]),
+    "mdf_plan": (ctypes.c_int, [H, ctypes.c_longlong, ctypes.POINTER(Plan)]),
     "mdf_autotune": (ctypes.c_int, [H, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                     ctypes.POINTER(ctypes.c_int)]),
     "mdf_sync": (ctypes.c_int, [H]),
@@ -101,6 +112,9 @@ SIGNATURES = {
     "mdf_batch_set_timeout": (ctypes.c_int, [H, ctypes.c_longlong]),
     "mdf_batch_set_schedule": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "mdf_batch_get_schedule": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
+    "mdf_batch_set_path": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
+    "mdf_batch_get_path": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int),
+                                          ctypes.POINTER(ctypes.c_int)]),
     "mdf_batch_autotune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
                                           ctypes.c_void_p]),
     "mdf_batch_last_error": (ctypes.c_char_p, [H]),

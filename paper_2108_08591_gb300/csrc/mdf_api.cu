@@ -251,6 +251,30 @@ int fused_updates(const mdf_t h, long long n) {
   return h->ny >= K ? K : 1;
 }
 
+// What run_steps makes of n updates, launch by launch.
+mdf_plan_t plan_of(const mdf_t h, long long n) {
+  mdf_plan_t p{MDF_PATH_SINGLE, 0, 0, 0};
+  while (n > 0) {
+    const bool resident = h->resident && n >= h->resident;
+    const int k = resident ? (int)std::min<long long>(n, kResMaxSteps) : fused_updates(h, n);
+    const long long times = n / k;
+    p.launches += times;
+    n -= times * k;
+    if (k <= p.updates) continue;
+    p.updates = k;
+    if (resident) {
+      p.path = MDF_PATH_RESIDENT;
+      p.threads = res_threads(res_shape(h->nx, h->ny, h->q, h->nsets).rows * h->nx);
+    } else if (k > 1) {
+      p.path = MDF_PATH_FUSED;
+      p.threads = 32 * (h->d == 2 ? kFuseWarps : kFuse3Rows);
+    } else {
+      p.threads = h->block;
+    }
+  }
+  return p;
+}
+
 // Enqueue the next launch of a run of n updates, `tk` updates into its
 // launch group, and move to its result; *k is the updates it makes.
 cudaError_t launch_next(mdf_t h, long long n, int tk, int *k) {
@@ -299,7 +323,7 @@ mdf_status build_graph(mdf_t h, int which) {
 
 mdf_status run_steps(mdf_t h, long long n) {
   while (h->resident && n >= h->resident) {
-    const int s = (int)std::min<long long>(n, 1 << 14);
+    const int s = (int)std::min<long long>(n, kResMaxSteps);
     CU(h, launch_set_clock(h->clock, (int)h->step, h->stream));
     CU(h, lattice_launch(h->d, h->q)->resident(s, h->walls, base_args(h), h->stream));
     std::swap(h->cur, h->nxt);
@@ -791,6 +815,13 @@ mdf_status mdf_info(mdf_t h, mdf_info_t *out) {
   out->vx = h->vx;
   out->block = h->block;
   out->s0 = h->s0; out->s1 = h->s1; out->s2 = h->s2;
+  return MDF_OK;
+}
+
+mdf_status mdf_plan(mdf_t h, long long n, mdf_plan_t *out) {
+  if (check_handle(h)) return MDF_EINVAL;
+  if (!out || n < 0) return fail(h, MDF_EINVAL, "plan: null output or n < 0");
+  *out = plan_of(h, n);
   return MDF_OK;
 }
 

@@ -966,7 +966,7 @@ cudaError_t enqueue_fused(mdf_batch_t b, int n, int *cur, int *made) {
   cudaError_t e = cudaSuccess;
   int k = 0;
   if (b->seats) {
-    k = std::min(n, 1 << 14);
+    k = std::min(n, kResMaxSteps);
     e = launch_resident(b, *cur, 0, k, false, 1);
     *cur ^= 1;
   } else {
@@ -984,7 +984,7 @@ cudaError_t enqueue_fused(mdf_batch_t b, int n, int *cur, int *made) {
 // (even, >= 4) updates, so that the state ends in the buffer it started in.
 cudaError_t fused_period(mdf_batch_t b, int period) {
   if (b->seats) {  // an even number of launches, for the same reason
-    const int n = 2 * ((period / 2 + (1 << 14) - 1) >> 14);
+    const int n = 2 * ((period / 2 + kResMaxSteps - 1) / kResMaxSteps);
     cudaError_t e = cudaSuccess;
     for (int k = 0, t = 0; k < n && e == cudaSuccess; ++k) {
       const int s = (period - t) / (n - k);
@@ -1407,6 +1407,22 @@ mdf_status mdf_batch_set_schedule(mdf_batch_t b, int threads, int grid, int sche
   return MDF_OK;
 }
 
+mdf_status mdf_batch_set_path(mdf_batch_t b, int path) {
+  if (!b) return MDF_EINVAL;
+  if (path != MDF_PATH_DEFAULT && path != MDF_PATH_PERSISTENT)
+    return bfail(b, MDF_EINVAL, "path must be MDF_PATH_DEFAULT or MDF_PATH_PERSISTENT (got %d)", path);
+  b->own_shape = path == MDF_PATH_PERSISTENT;
+  drop_graph(b);  // it holds launches of the other path
+  return MDF_OK;
+}
+
+mdf_status mdf_batch_get_path(mdf_batch_t b, int *path, int *updates) {
+  if (!b) return MDF_EINVAL;
+  if (path) *path = !b->fuse() ? MDF_PATH_PERSISTENT : b->seats ? MDF_PATH_RESIDENT : MDF_PATH_FUSED;
+  if (updates) *updates = b->fuse() && !b->seats ? fused_depth(b) : 0;
+  return MDF_OK;
+}
+
 mdf_status mdf_batch_get_schedule(mdf_batch_t b, int *threads, int *grid, int *sched) {
   if (!b) return MDF_EINVAL;
   if (threads) *threads = b->threads;
@@ -1483,7 +1499,7 @@ mdf_status mdf_batch_autotune(mdf_batch_t b, int reps, int *threads_out, int *gr
   // one of a kernel loads it), the best of three in turn.
   bool own_shape = b->own_shape;
   if (st == MDF_OK && b->can_fuse && !b->own_limit) {
-    const int n = std::min(1 << 14, std::max(reps, 100));
+    const int n = std::min(kResMaxSteps, std::max(reps, 100));
     float t[2] = {1e30f, 1e30f};  // persistent, fused
     cudaError_t e = cudaSuccess;
     b->threads = best_threads;

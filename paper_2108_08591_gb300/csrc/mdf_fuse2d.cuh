@@ -39,7 +39,6 @@
 
 namespace mdf {
 
-constexpr int kFuseWarps = 2;  // independent warps per block
 template <int K> constexpr int fuse_halo() { return (K + 1) / 2 * 2; }
 template <int K> constexpr int fuse_out() { return 64 - 2 * fuse_halo<K>(); }
 

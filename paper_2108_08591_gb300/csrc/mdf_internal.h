@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "mdf_device.h"
 
 namespace mdf {
@@ -122,6 +124,43 @@ inline Fuse3Plan fuse3_plan(int nx, int ny, int nz) {
 inline bool fuse3_pays(int nx, int ny, int nz, bool walls, bool force) {
   const double ps = walls ? (force ? 66.0 : 76.0) : (force ? 60.0 : 69.0);
   return fuse3_plan(nx, ny, nz).us < 1e-6 * ps * nx * (double)ny * nz;
+}
+
+constexpr int kFuseWarps = 2;  // independent warps per block of the 2D fused kernel
+
+// The resident kernel's launches (mdf_res2d.cuh).
+constexpr int kResThreads = 512;
+constexpr int kResMaxCluster = 16;                // needs the non-portable size
+// Most nodes of a CTA.  Up to here the resident kernel is the faster one: us
+// per update against fused launches, 16^2 0.62 / 3.1, 64^2 0.75 / 3.1 (and
+// 4.2 in launches of one), 96^2 1.47 / 3.1, 128^2 (1024 nodes a CTA) 1.98 /
+// 3.2; at 144^2 (1296) 2.95 / 3.2 and at 170^2 3.37 / 3.4 it no longer pays
+// for its start.
+constexpr int kResMaxNodes = 1200;
+constexpr int kResMaxSteps = 1 << 14;  // updates of one launch
+// Fewest updates that pay for reading and writing the lattice once more than
+// a fused launch would: with two nodes a thread four (128^2: 4.7 us per update
+// against 5.8 of single ones; with two updates 8.4 against 7.5).
+inline int res_min_steps(int nodes) { return nodes > kResThreads ? 4 : 2; }
+
+// CTAs of a cluster for nx x ny nodes, and the shared memory of each; 0 when
+// it does not fit.
+struct ResShape {
+  int ctas, rows;  // rows: the most of a CTA
+  size_t smem;
+};
+inline ResShape res_shape(int nx, int ny, int q, int nsets) {
+  const int c = std::min(ny, kResMaxCluster), rows = (ny + c - 1) / c;
+  if ((long long)rows * nx > kResMaxNodes) return {0, 0, 0};
+  return {c, rows, 2ull * nsets * q * rows * (size_t)nx * sizeof(float)};
+}
+
+// Threads of a CTA for its nodes: whole warps, a node each, or two each (as a
+// pair) beyond the limit.
+inline bool res_pairs(int nodes) { return nodes > kResThreads; }
+inline int res_threads(int nodes) {
+  const int n = res_pairs(nodes) ? (nodes + 1) / 2 : nodes;
+  return std::min(kResThreads, (n + 31) / 32 * 32);
 }
 
 // K updates in one launch (FP32, two buffers, all d + 1 sets): 2 or 4 in 2D

@@ -19,33 +19,8 @@
 
 namespace mdf {
 
-constexpr int kResThreads = 512;
-constexpr int kResMaxCluster = 16;                // needs the non-portable size
-// Most nodes of a CTA.  Up to here the resident kernel is the faster one: us
-// per update against fused launches, 16^2 0.62 / 3.1, 64^2 0.75 / 3.1 (and
-// 4.2 in launches of one), 96^2 1.47 / 3.1, 128^2 (1024 nodes a CTA) 1.98 /
-// 3.2; at 144^2 (1296) 2.95 / 3.2 and at 170^2 3.37 / 3.4 it no longer pays
-// for its start.
-constexpr int kResMaxNodes = 1200;
 constexpr int kResMaxTeamNodes = 1800;  // of a CTA in a batch of cavities
 constexpr size_t kResMaxSmem = 2ull * 15 * kResMaxTeamNodes * sizeof(float);  // of a CTA
-// Fewest updates that pay for reading and writing the lattice once more than
-// a fused launch would: with two nodes a thread four (128^2: 4.7 us per update
-// against 5.8 of single ones; with two updates 8.4 against 7.5).
-inline int res_min_steps(int nodes) { return nodes > kResThreads ? 4 : 2; }
-
-// CTAs of a cluster for nx x ny nodes, and the shared memory of each; 0 when
-// it does not fit.
-struct ResShape {
-  int ctas, rows;  // rows: the most of a CTA
-  size_t smem;
-};
-inline ResShape res_shape(int nx, int ny, int q, int nsets) {
-  const int c = std::min(ny, kResMaxCluster), rows = (ny + c - 1) / c;
-  if ((long long)rows * nx > kResMaxNodes) return {0, 0, 0};
-  return {c, rows, 2ull * nsets * q * rows * (size_t)nx * sizeof(float)};
-}
-
 // Where a node's populations come from: one pointer per direction (set 0,
 // current buffer; local or of a neighbouring CTA), and what the walls make of
 // the value.
@@ -236,14 +211,6 @@ __global__ void __launch_bounds__(kResThreads) k_resident2d(const DevArgs A, int
   const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   res_run<L, WALLS, FORCE, PAIR>(fuse_lattice<L>(A), A.with_rho != 0, steps, false, rcap, res_smem, 0,
                                  (int)cl.num_blocks(), (int)cl.block_rank());
-}
-
-// Threads of a CTA for its nodes: whole warps, a node each, or two each (as a
-// pair) beyond the limit.
-inline bool res_pairs(int nodes) { return nodes > kResThreads; }
-inline int res_threads(int nodes) {
-  const int n = res_pairs(nodes) ? (nodes + 1) / 2 : nodes;
-  return std::min(kResThreads, (n + 31) / 32 * 32);
 }
 
 template <class Kernel, class... Args>

@@ -166,3 +166,84 @@ def test_batch_autotune_keeps_the_persistent_kernel_where_it_is_faster(fake):
     assert lib.mdf_batch_autotune(b, 20, None, None, None) == _lib.OK
     assert all("k_batch_chunk" in n for n in _step_kernels(fake, b))
     lib.mdf_batch_destroy(b)
+
+
+def _count(fake, step):
+    """(update kernels launched, threads of the last) of a call."""
+    fake.launches()
+    assert step() == _lib.OK
+    return [(n, threads) for n, _, _, threads, _ in fake.launches() if "set_clock" not in n]
+
+
+@pytest.mark.parametrize("shape,storage,opts", [
+    ((64, 64), "f32", {}), ((1200, 16), "f32", {}), ((129, 130), "f32", {"q": 4}), ((300, 300), "f32", {}),
+    ((1003, 751), "f32", {}), ((400001, 2), "f32", {}), ((250001, 3), "f32", {}), ((1003, 751), "f32", {"vx": 1}),
+    ((1003, 751), "f32", {"inplace": 1}), ((1003, 751), "f16", {}), ((64, 64), "f64", {}), ((60, 60, 200), "f32", {}),
+    ((64, 64, 64), "f32", {}), ((60, 60, 200), "f16eq", {}), ((119, 121, 151), "f32", {"q": 6, "wall": True})])
+def test_plan_is_what_a_step_launches(fake, shape, storage, opts):
+    h = fake.lattice(shape, storage, **opts)
+    kernels = {0: "k_update", 1: "k_update_fused", 2: "k_resident2d"}
+    for n in (0, 1, 2, 3, 4, 7, 70):
+        p = _lib.Plan()
+        assert fake.lib.mdf_plan(h, n, ctypes.byref(p)) == _lib.OK
+        got = _count(fake, lambda: fake.lib.mdf_step(h, n))
+        assert p.launches == len(got), n
+        assert p.updates * p.launches >= n
+        if n:
+            assert kernels[p.path] in got[0][0] and got[0][1] == p.threads, (n, got)
+            assert ("fused" in got[0][0]) == (p.path == 1)
+    p = _lib.Plan()
+    assert fake.lib.mdf_plan(h, 10**12, ctypes.byref(p)) == _lib.OK and p.launches * p.updates >= 10**12
+    assert fake.lib.mdf_plan(h, -1, ctypes.byref(p)) == _lib.EINVAL
+    assert fake.lib.mdf_plan(h, 1, None) == _lib.EINVAL
+    fake.lib.mdf_destroy(h)
+
+
+def test_plan_of_a_long_run_on_chip(fake):
+    h = fake.lattice((64, 64))
+    p = _lib.Plan()
+    assert fake.lib.mdf_plan(h, 40001, ctypes.byref(p)) == _lib.OK
+    assert (p.path, p.updates, p.launches, p.threads) == (2, 16384, 3, 256)
+    assert len(_count(fake, lambda: fake.lib.mdf_step(h, 40001))) == 3
+    fake.lib.mdf_destroy(h)
+
+
+def test_plan_struct_matches_the_header(tmp_path):
+    """As tests/test_abi.py checks the other structs."""
+    import os
+    import subprocess
+    src = tmp_path / "layout.c"
+    src.write_text('#include <stdio.h>\n#include <stddef.h>\n#include "mdf.h"\nint main(void) {\n'
+                   + "".join(f'printf("%zu ", offsetof(mdf_plan_t, {f}));' for f, _ in _lib.Plan._fields_)
+                   + 'printf("%zu", sizeof(mdf_plan_t)); return 0; }\n')
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "include")
+    subprocess.run(["gcc", "-std=c99", "-I", inc, str(src), "-o", str(tmp_path / "layout")], check=True)
+    out = subprocess.run([str(tmp_path / "layout")], check=True, capture_output=True, text=True).stdout
+    assert [int(v) for v in out.split()] == [getattr(_lib.Plan, f).offset for f, _ in _lib.Plan._fields_] + [
+        ctypes.sizeof(_lib.Plan)]
+
+
+@pytest.mark.parametrize("sides,path,updates,kernel", [([300, 240], 1, 2, "k_batch_fused"), ([700] * 2, 1, 4, "k_batch_fused"),
+                                                       ([65, 97], 2, 0, "k_batch_resident")])
+def test_batch_path_is_reported_and_can_be_chosen(fake, sides, path, updates, kernel):
+    lib = fake.lib
+    b = fake.batch(sides)
+
+    def now():
+        p, k = ctypes.c_int(), ctypes.c_int()
+        assert lib.mdf_batch_get_path(b, ctypes.byref(p), ctypes.byref(k)) == _lib.OK
+        kinds = _step_kernels(fake, b)
+        assert all(("k_batch_chunk" if p.value == _lib.PATH_PERSISTENT else kernel) in n for n in kinds)
+        return p.value, k.value
+
+    default, persistent = (path, updates), (_lib.PATH_PERSISTENT, 0)
+    assert now() == default
+    for away in (lambda: lib.mdf_batch_set_schedule(b, 64, 0, 3), lambda: lib.mdf_batch_set_path(b, _lib.PATH_PERSISTENT)):
+        assert away() == _lib.OK and now() == persistent
+        assert lib.mdf_batch_set_path(b, _lib.PATH_DEFAULT) == _lib.OK and now() == default
+    assert lib.mdf_batch_set_timeout(b, 1000) == _lib.OK and now() == persistent
+    assert lib.mdf_batch_set_path(b, _lib.PATH_DEFAULT) == _lib.OK and now() == persistent  # the limit stays
+    assert lib.mdf_batch_set_timeout(b, 4_000_000_000) == _lib.OK and now() == default
+    for bad in (-2, 0, 1, 2, 4):
+        assert lib.mdf_batch_set_path(b, bad) == _lib.EINVAL
+    lib.mdf_batch_destroy(b)
