@@ -334,10 +334,13 @@ typedef struct {
 mdf_status mdf_plan(mdf_t h, long long n, mdf_plan_t *out);
 
 /*
- * mdf_autotune -- measure the update kernel's launch shapes for this handle
- * (one node per thread and each vector width built for the storage type
- * that divides nx, times 64/128/256 threads per block; `reps` timed updates
- * each, CUDA events on h's stream) and keep the fastest.  The candidates
+ * mdf_autotune -- measure the one-update kernel's launch shapes for this
+ * handle (the shape in use; one node per thread and each vector width built for
+ * the storage type that divides nx, times 64/128/256 threads per block; `reps`
+ * timed updates each, CUDA events on h's stream) and keep the fastest.  That is
+ * the kernel of every update of a handle on MDF_PATH_SINGLE; runs that go fused
+ * or stay on chip (mdf_plan) keep doing so, and take it for what is left of
+ * them.  The candidates
  * update out of place without advancing the state, so the lattice is left
  * as it was.  *vx, *block (nullable) receive the choice.  Synchronises.
  */

@@ -251,8 +251,9 @@ class Lattice:
         return {"path": _lib.PATHS[p.path], "updates": p.updates, "launches": p.launches, "threads": p.threads}
 
     def autotune(self, reps: int = 10):
-        """Measure the update kernel's launch shapes and keep the fastest;
-        the lattice state is unchanged.  Returns (vx, block)."""
+        """Measure the one-update kernel's launch shapes and keep the fastest
+        (runs that go fused or stay on chip keep doing so, see plan()); the
+        lattice state is unchanged.  Returns (vx, block)."""
         vx, block = ctypes.c_int(), ctypes.c_int()
         self._check(self._lib.mdf_autotune(self._h, int(reps), ctypes.byref(vx), ctypes.byref(block)))
         return vx.value, block.value

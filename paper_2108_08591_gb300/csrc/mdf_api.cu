@@ -830,8 +830,9 @@ mdf_status mdf_autotune(mdf_t h, int reps, int *vx_out, int *block_out) {
   if (h->inplace)  // its trial updates run out of place, and there is one buffer
     return fail(h, MDF_EUNSUPPORTED, "autotune needs the two-buffer layout");
   if (reps < 1) reps = 10;
-  // Candidates: one node per thread, and every vector width built for the
-  // storage type that divides nx; 64, 128 and 256 threads per block.
+  // Candidates: the shape in use, then one node per thread and every vector
+  // width built for the storage type that divides nx, each with 64, 128 and 256
+  // threads per block.  (The default block may be another, see fit_block.)
   int widths[4] = {1, 0, 0, 0}, nw = 1;
   // by MDF_F32, F16, BF16, F64, F16EQ, BF16EQ
   const int built[6][2] = {{2, 4}, {4, 8}, {4, 8}, {2, 2}, {2, 4}, {2, 4}};
@@ -848,10 +849,12 @@ mdf_status mdf_autotune(mdf_t h, int reps, int *vx_out, int *block_out) {
   float best = 1e30f;
   int best_vx = h->vx, best_block = h->block;
   mdf_status st = MDF_OK;
-  for (int w = 0; w < nw && st == MDF_OK; ++w)
-    for (int b = 0; b < 3 && st == MDF_OK; ++b) {
-      h->vx = widths[w];
-      h->block = blocks[b];
+  for (int w = -1; w < nw && st == MDF_OK; ++w)
+    for (int b = 0; b < (w < 0 ? 1 : 3) && st == MDF_OK; ++b) {
+      if (w >= 0) {
+        h->vx = widths[w];
+        h->block = blocks[b];
+      }
       // out-of-place updates cur -> nxt without swapping: the state is kept
       const DevArgs a = base_args(h);
       cudaError_t e = launch_update(h, MODE_STEP, a);
@@ -865,7 +868,7 @@ mdf_status mdf_autotune(mdf_t h, int reps, int *vx_out, int *block_out) {
         st = fail(h, MDF_ECUDA, "autotune: %s", cudaGetErrorString(e));
         break;
       }
-      if (ms < best) { best = ms; best_vx = widths[w]; best_block = blocks[b]; }
+      if (ms < best) { best = ms; best_vx = h->vx; best_block = h->block; }
     }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -247,3 +247,20 @@ def test_batch_path_is_reported_and_can_be_chosen(fake, sides, path, updates, ke
     for bad in (-2, 0, 1, 2, 4):
         assert lib.mdf_batch_set_path(b, bad) == _lib.EINVAL
     lib.mdf_batch_destroy(b)
+
+
+@pytest.mark.parametrize("shape,storage,own", [((29, 124, 157), "f16", (4, 96)), ((190, 40, 20), "bf16eq", (2, 96)),
+                                               ((700, 700), "f32", (4, 96)), ((64, 64), "f64", (2, 64))])
+def test_autotune_weighs_the_shape_in_use(fake, shape, storage, own):
+    """The launch shape of a handle is a candidate of its own, and stays where no
+    other is faster (here all take no time)."""
+    h = fake.lattice(shape, storage)
+    info = _lib.Info()
+    assert fake.lib.mdf_info(h, ctypes.byref(info)) == _lib.OK and (info.vx, info.block) == own
+    fake.launches()
+    v, b = ctypes.c_int(), ctypes.c_int()
+    assert fake.lib.mdf_autotune(h, 2, ctypes.byref(v), ctypes.byref(b)) == _lib.OK
+    assert own[1] in {threads for _, _, _, threads, _ in fake.launches()}
+    assert (v.value, b.value) == own
+    assert fake.lib.mdf_info(h, ctypes.byref(info)) == _lib.OK and (info.vx, info.block) == own
+    fake.lib.mdf_destroy(h)
