@@ -50,7 +50,9 @@ class Lattice:
     wall: per-axis halfway walls (anti-halfway bounce-back), lid: the + face
     of the last axis moves with lid_u.  storage: 'f32', 'f16', 'bf16', 'f64',
     'f16eq', 'bf16eq'.  vx / block: x-nodes per thread and threads per block
-    of the update kernel (0: the library's tuned default).  q: 0 for
+    of the one-update kernel (0, 0: the library's tuned default, with which runs
+    of updates of an FP32 lattice go several to a launch where that is faster,
+    see plan(); a value of one's own keeps to one).  q: 0 for
     D2Q5 / D3Q7, 4 for D2Q4, 6 for D3Q6 (rest-shifted storage types only).
     inplace: one population buffer streamed in place by the AA pattern
     (rest-shifted storage types; half the memory, the same results).
@@ -329,8 +331,11 @@ class Slabs:
 
 class CavityBatch:
     """Many lid-driven cavities (closed boxes, lid on the + face of the last
-    axis moving along x) advanced together to steady state by one persistent
-    kernel per convergence period (see mdf_batch_* in include/mdf.h)."""
+    axis moving along x) advanced together to steady state, a convergence
+    period at a time (see mdf_batch_* in include/mdf.h).  2D batches with the
+    alpha = 0 set stay on chip where they fit and otherwise advance by fused
+    launches; the others, and those given a schedule, by one persistent kernel
+    per period (see `path`)."""
 
     def __init__(self, sides: Sequence[int], Re: Sequence[float], lid_speed: float = 0.1,
                  d: int = 2, with_rho: bool = True, stream=None):
@@ -515,7 +520,9 @@ CONV_KERNELS = {"mma.sync": 0, "tcgen05": 1, "tcgen05-halo": 2}
 
 
 def set_conv_kernel(which: str):
-    """Forward/dgrad convolution kernel: 'tcgen05-halo' (default), 'tcgen05'
+    """Forward/dgrad convolution kernel: 'tcgen05-halo' (default: staged input
+    halos, by persistent TMA-fed CTAs for 16-byte aligned tensors without a
+    tile override, else one CTA per tile, with the same bits), 'tcgen05'
     (im2col gathers) or 'mma.sync'."""
     _lib.check(_lib.load().mdf_nn_set_conv_kernel(CONV_KERNELS[which]))
 

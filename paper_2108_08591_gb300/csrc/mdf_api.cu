@@ -241,9 +241,10 @@ mdf_status one_update(mdf_t h, int mode, const mdf_fields_t *out) {
 // the lattice has such a kernel, else 1.  2D lattices of fewer than 750 000
 // nodes take 2: with few rows for each warp the 12 extra row updates that fill
 // and drain the deeper pipeline cost more than a pass over memory that is in
-// L2 (230 x 500 with a force 6.3 us per update by fours, 5.2 by twos; 700 x 500
-// 8.1 / 7.3, 700 x 1024 12.5 / 11.4; 1024 x 830 13.4 / 13.5, 1024^2 15.6 /
-// 16.4, with walls and a force 17.2 / 18.7).
+// L2.  us per update by fours / twos: 230 x 500 4.08 / 3.12, 509 x 515 5.79 /
+// 4.83, 700 x 700 7.29 / 6.77, 700 x 1024 10.4 / 8.9, 866^2 (749 956 nodes) 10.5 /
+// 9.8; 1024 x 830 (849 920) 11.0 / 11.3, 1024^2 13.1 / 13.8, with walls and a force
+// 16.6 / 17.3, 2048^2 40.3 / 47.1.
 int fused_updates(const mdf_t h, long long n) {
   if (!h->fuse[h->force != nullptr] || n < 2) return 1;
   if (h->d == 3) return 2;

@@ -1,14 +1,25 @@
-// Batched lid-driven cavities advanced to steady state by one persistent
-// kernel per convergence period, captured in a CUDA graph.
+// Batched lid-driven cavities advanced to steady state, one convergence period
+// after the other, each captured in a CUDA graph.
 //
 // Every cavity is a closed box (anti-halfway bounce-back walls on all faces,
 // the + face of the last axis moving with the lid velocity, Sec. 4) with its
 // own side N and relaxation rates.  Nodes of all cavities live in one pool,
 // cavity after cavity, each cavity padded to whole tiles of kTile nodes, so a
 // tile belongs to exactly one cavity; populations are structure of arrays
-// f[set][i][pool node], rest-shifted FP32.  Per step the persistent kernel
-// walks the list of tiles of the cavities still running, with a bounded grid
-// barrier between steps.  Every R = `check` steps a residual pass (FP64:
+// f[set][i][pool node], rest-shifted FP32.
+//
+// The updates of a period take one of three paths, with the same bits:
+//   - resident (k_batch_resident): every cavity stays in the shared memory of a
+//     team of CTAs for the whole period; a 2D batch with the alpha = 0 set that
+//     fits on the GPU at once (build_seats);
+//   - fused (k_batch_fused): launches of two or four updates per pass over
+//     memory; every other 2D batch with the alpha = 0 set;
+//   - persistent (k_batch_chunk): one kernel walks the list of tiles of the
+//     cavities still running, with a bounded grid barrier between steps; 3D, two
+//     sets, periods of two, a schedule or barrier limit of the caller's own, or
+//     where mdf_batch_autotune measured it faster.
+//
+// Every R = `check` steps a residual pass (FP64:
 // r = |u^n - u^{n-R}|_2 / (R |u^n|_2) per cavity, the mean per-step relative
 // change over the period, which FP32 rounding noise does not floor near
 // 1e-7 as the single-step difference does), a status pass and a compaction
@@ -950,9 +961,12 @@ cudaError_t launch_resident(mdf_batch_t b, int cur, int tk, int steps, bool save
 }
 
 // Updates a fused launch should make: four for 750 000 nodes or more, else two
-// (as for single lattices: the rows that fill and drain the deeper march count;
-// four boxes of 300^2 10.9 us per update by fours, 10.0 by twos, twelve 21.4 /
-// 22.7).
+// (as for single lattices: the rows that fill and drain the deeper march count).
+// us per update by fours / twos: four boxes of 300^2 9.9 / 9.4, eight 12.9 / 11.4,
+// twelve of 175^2 11.4 / 9.3, 40 of 129^2 (666 000 nodes) 16.5 / 14.5; 60 of 129^2
+// (998 000) 18.6 / 20.6, 16 of 257^2 17.4 / 19.1, four of 513^2 17.2 / 17.6.  Just
+// above the line twos are still ahead (three of 513^2, 790 000, 16.5 / 13.5), and
+// they fit some sides better (twelve of 300^2, 1 080 000, 20.2 / 17.3).
 int fused_depth(mdf_batch_t b) {
   long long nodes = 0;
   for (const CavParam &c : b->cav) nodes += (long long)c.N * c.N;

@@ -634,7 +634,8 @@ __global__ void __launch_bounds__(kMaxBlock) k_init_eq_moments(const DevArgs A) 
 // Second pass: the stored parts, from this node's moments and those of the
 // nodes its populations come to.  (In one pass every (set, direction) read
 // and narrowed its neighbour's FP64 seed again, 15 or 28 times a node: 1007
-// us at 2050 x 1998, then 154 for both.)  GRAD as for k_init: INITEQFIG
+// us at 2050 x 1998, then 154 for both.)  GRAD as for k_init: with a run-time
+// test in place of it 190 x 202 x 178 BF16 with walls took 535 us, now 342.
 template <class L, class TS, bool WALLS, bool GRAD>
 __global__ void __launch_bounds__(kMaxBlock) k_init_eq(const DevArgs A) {
   constexpr int D = L::D, Q = L::Q;

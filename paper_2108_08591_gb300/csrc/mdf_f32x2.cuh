@@ -51,10 +51,10 @@ struct F2 {
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(vadd(a.f2(), b.f2())); }
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(vsub(a.f2(), b.f2())); }
 // Constants of the collision.
-enum Lit { LIT_2_3, LIT_3_4, LIT_M4, LIT_M6, LIT_1_20, LIT_1_5, LIT_1_42, LIT_1_7, LIT_1_6, LIT_1_2, LIT_DITHER,
+enum Lit { LIT_2_3, LIT_3_4, LIT_M4, LIT_M6, LIT_1_20, LIT_1_5, LIT_1_42, LIT_1_7, LIT_1_6, LIT_1_2,
            LIT_1, LIT_1_4, LIT_1_3, LIT_1_12, LITS };
 constexpr double kLit[LITS] = {2.0 / 3.0,  0.75,      -4.0, -6.0, 0.05, 0.2, 1.0 / 42.0, 1.0 / 7.0, 1.0 / 6.0,
-                               0.5,        -1.498046875 * 0x1p-23,  1.0,  0.25, 1.0 / 3.0,  1.0 / 12.0};
+                               0.5,        1.0,       0.25, 1.0 / 3.0, 1.0 / 12.0};
 template <class T, Lit K> __device__ __forceinline__ T lit() {
   constexpr double v = kLit[K];
   return T(v);

@@ -26,13 +26,13 @@
 // so the bits are those of K single updates.
 //
 // Measured (GB300, K = 4, us per update against one update per launch):
-// 4096^2 148 / 302, 2048^2 40.9 / 80, 1024^2 13.9 / 22.6;
-// 4095^2 149 / (scalar kernel) 330; walls and lid 166 at 4096^2.  K = 4 is
+// 4096^2 147 / 300, 2048^2 40.3 / 79, 1024^2 13.1 / 22.6;
+// 4095^2 149 / (scalar kernel) 330; walls and lid 165 at 4096^2.  K = 4 is
 // bound by the FP32 and integer pipes (issue 58 %, the f32x2 operations take
 // two slots of theirs): 219 instructions per update and node, of which 1.14
-// x is rim.  K = 2 would stay at HBM's 150 us; it serves lattices of fewer than
+// x is rim.  K = 2 takes 180 us at 4096^2; it serves lattices of fewer than
 // 750 000 nodes, where the row updates that fill and drain the pipeline count
-// (509 x 515 with walls: 5.9 us per update, 6.9 with K = 4, 10.0 single).
+// (509 x 515 with walls: 5.6 us per update, 6.6 with K = 4, 10.0 single).
 #pragma once
 
 #include "mdf_kernels.cuh"
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(32 * kFuseWarps, kFuseBlocks)
 // 0.57 / 0.76 / 1.0 / 1.2 us for w = 1 .. 4.  Long segments waste less, many
 // warps hide more; large lattices take the most warps, small ones fewer
 // (256^2: 3.65 us per update with w = 1 against 4.17 with w = 2 .. 4;
-// 1024^2: 20.0, 14.5, 14.0, 14.1).
+// 1024^2: 20.0, 14.5, 14.0, 14.1, at a build that now takes 13.1).
 template <int K, class Items>
 int fuse_rows(int ny, int wmax, Items items) {
   int best_rows = ny;

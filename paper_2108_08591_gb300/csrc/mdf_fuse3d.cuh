@@ -27,7 +27,9 @@
 // 480 x 480 x 200 1226 / 1590, 256^3 534 / 584, 190 x 202 x 178 with walls
 // and a lid 269 / 351, periodic 242 / 255.  Bound by the FP32 and integer
 // pipes (590 instructions per update and node at 256^3, where the tiles do
-// 1.5 x the work) and by the barriers: issue 47 %.  Requesting the next plane
+// 1.5 x the work) and by the barriers: issue 47 %.  The 128 registers that two
+// blocks per SM leave are not quite enough: the D3Q7 forms spill 24 B (periodic)
+// to 84 B (walls and a force) of stores, the D3Q6 ones none to 120 B.  Requesting the next plane
 // with cp.async (548 at 256^3), and prefetching it to L2 (578), gained
 // nothing.  fuse3_plan says where it pays.
 #pragma once
