@@ -24,6 +24,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -51,15 +52,22 @@ TG3D_U0, TG3D_RE = 0.05, 1600.0
 # viscosity (set by s1, Eq. 3-13a) unchanged.  The 2D case keeps the rule.
 TG3D_S2 = 1.0
 S2 = -1.0  # the workload's s2 (negative: the paper's rule); set in main()
-KERNEL_SOURCES = ("paper_2108_08591_gb300/csrc/mdf_kernels.cuh",
-                  "paper_2108_08591_gb300/csrc/mdf_lattice.cuh")
-# sources of the fused FP32 update
-FUSED_SOURCES = KERNEL_SOURCES + ("paper_2108_08591_gb300/csrc/mdf_fuse2d.cuh",
-                                  "paper_2108_08591_gb300/csrc/mdf_f32x2.cuh")
-# sources of the equilibrium-shifted update (its recorded traffic is keyed
-# by their hash)
-EQ_SOURCES = KERNEL_SOURCES + ("paper_2108_08591_gb300/csrc/mdf_eq.cuh",
-                               "paper_2108_08591_gb300/csrc/mdf_pack16.cuh")
+CSRC = os.path.join(ROOT, "paper_2108_08591_gb300", "csrc")
+
+
+def _sources(path: str, d: int):
+    """The headers of the kernel that plain updates run (`path` as Lattice.plan()
+    names it): its own and every one that it includes.  The recorded traffic is
+    keyed by their hash."""
+    todo, seen = [{"single": "mdf_kernels.cuh", "resident": "mdf_res2d.cuh",
+                   "fused": f"mdf_fuse{d}d.cuh"}[path]], []
+    while todo:
+        name = todo.pop()
+        if name not in seen:
+            seen.append(name)
+            with open(os.path.join(CSRC, name)) as fh:
+                todo += re.findall(r'#include "(mdf_\w+\.cuh)"', fh.read())
+    return sorted(os.path.join(CSRC, name) for name in seen)
 
 
 def _dist():
@@ -97,10 +105,10 @@ def aggregate(local_updates: float, local_ms: float, dist=None, device="cpu"):
     return total / (t_max / 1e3) / 1e6, t_max, world
 
 
-def _kernel_sha(sources=KERNEL_SOURCES) -> str:
+def _kernel_sha(sources) -> str:
     h = hashlib.sha256()
     for p in sources:
-        with open(os.path.join(ROOT, p), "rb") as fh:
+        with open(p, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
@@ -122,19 +130,15 @@ def _traffic(kernel_sha: str, leg: str = ""):
     return t.get("dram_bytes_per_launch_4096")
 
 
-def _fused_launches(n: int, shape, storage: str, single: bool = False):
-    """(updates per fused launch, launches) of a run of n plain updates on the
-    library's default launch shape: FP32 with two buffers runs 4 updates per
-    launch on 2D lattices from 750 000 nodes (then 2, then 1 for the rest) and 2
-    on the 3D workload's box; every other storage, a streaming in place and a
-    caller's own launch shape (`single`) one."""
-    nodes = math.prod(shape)
-    if storage != "f32" or single:
-        return 1, n
-    if len(shape) == 3:
-        return 2, n // 2 + n % 2
-    K = 4 if nodes >= 750000 else 2
-    return K, n // K + (n % K) // 2 + n % 2
+def _bound(path: str):
+    """What bounds the plain updates, for the roofline entry: HBM where each is a
+    pass over memory.  Fused updates share passes (their kernels' counters: issue
+    56 .. 64 %, the FP32 and integer pipes 40 .. 52 %), resident ones make none."""
+    if path == "single":
+        return {"bound": "hbm"}
+    return {"bound": "instruction issue (FP32 and integer pipes)" if path == "fused" else
+            "latency (cluster barrier and neighbours' shared memory per update)",
+            "frac_is": "bytes of each launch (one pass for updates_per_launch updates) against hbm"}
 
 
 def _peaks():
@@ -374,21 +378,23 @@ def storage_leg(shape, s1, P, u, storage, steps=5, warmup=3, q=0, oracle_check=T
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1)
     plain_ms = sum(a.elapsed_time(b) for a, b in plain) / (steps * (EPI_EVERY - 1))
+    plan = lat.plan(EPI_EVERY - 1)
     lat.close()
     del fields
     peak, kind = _peaks()
     # bytes each launch cannot do without, over all launches of the plain updates
-    per_launch, launches = _fused_launches(EPI_EVERY - 1, shape, storage)
+    per_launch, launches = plan["updates"], plan["launches"]
     achieved = info.bytes_per_update * N * launches / ((EPI_EVERY - 1) * plain_ms / 1e3) / 1e9
-    sha = _kernel_sha(EQ_SOURCES) if storage.endswith("eq") else _kernel_sha()
+    sha = _kernel_sha(_sources(plan["path"], len(shape)))
     traffic = _traffic(sha, storage) if (N_GRID == 4096 and len(shape) == 2) else None
     out = {"storage": storage, "value": steps * EPI_EVERY * N / (ms / 1e3) / 1e6, "unit": "MLUPS",
            "steps": steps, "warmup": warmup,
-           "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                        "frac": achieved / peak, "traffic": traffic, "kernel_sha": sha,
+           "roofline": {**_bound(plan["path"]), "achieved": achieved, "peak": peak,
+                        "unit": "GB/s", "frac": achieved / peak, "traffic": traffic, "kernel_sha": sha,
                         "bytes_per_node": info.bytes_per_update, "updates_per_launch": per_launch,
                         "avg_launch_ms": plain_ms * (EPI_EVERY - 1) / launches,
-                        "ms_per_update": plain_ms, "vx": info.vx, "block": info.block,
+                        "ms_per_update": plain_ms, "path": plan["path"], "block": plan["threads"],
+                        **({"vx": info.vx} if plan["path"] == "single" else {}),
                         "peak_source": f"{kind} hbm_gbs (MEASURED_PEAKS.json)"}}
     if oracle_check:
         out["fp64_oracle_error"] = sampled_oracle_error(shape, s1, P, u, storage,
@@ -414,7 +420,8 @@ def tg3d_leg(oracle_check=True):
         out["workload"] = (f"3D Taylor-Green vortex, periodic 512^3, D3Q7 x 4 sets, U0 = {TG3D_U0}, "
                            f"Re = {TG3D_RE:.0f}, s2 = {TG3D_S2:g}, FP32 rest-shifted storage, "
                            "epilogue every 200 steps")
-        out["kernel"] = "k_update_fused3d<D3Q7,2,periodic>"
+        out["kernel"] = ("k_update_fused3d<D3Q7,2,periodic>" if out["roofline"]["path"] == "fused"
+                         else "k_update<D3Q7,float,MODE_STEP,periodic>")
         return out
     finally:
         S2, EPI_EVERY = saved
@@ -446,7 +453,7 @@ def run_mdf(args):
     lat = Lattice(shape, s1=s1, s2=S2, storage=args.storage, stream=stream, vx=args.vx or 0,
                   block=args.block or 0, q=args.q, inplace=args.inplace)
     lat.init(P, u)
-    info = lat.info
+    info, plan = lat.info, lat.plan(EPI_EVERY - 1)
     fields = lat.alloc_fields(("P", "u", "G", "div", "S", "sigma", "omega"))
 
     def bench_step(ev_a=None, ev_b=None):
@@ -520,10 +527,9 @@ def run_mdf(args):
     peak, peak_kind = _peaks()
     bytes_per_launch = info.bytes_per_update * N
     # several updates share a pass over memory: bytes count per launch
-    per_launch, launches = _fused_launches(EPI_EVERY - 1, shape, args.storage,
-                                           args.inplace or bool(args.vx or args.block))
+    path, per_launch, launches = plan["path"], plan["updates"], plan["launches"]
     achieved = bytes_per_launch * launches / ((EPI_EVERY - 1) * plain_ms / 1e3) / 1e9
-    sha = _kernel_sha(FUSED_SOURCES if per_launch > 1 else KERNEL_SOURCES)
+    sha = _kernel_sha(_sources(path, d))
     default_lattice = args.q in (0, 5 if d == 2 else 7) and not args.inplace
     traffic = _traffic(sha) if (args.workload == "tg2d" and N_GRID == 4096
                                 and args.storage == "f32" and default_lattice) else None
@@ -550,7 +556,9 @@ def run_mdf(args):
                   else f"k_update_aa<{kname},{tname},even+odd,MODE_STEP,periodic>")
     elif args.storage.endswith("eq"):
         kernel = f"k_update_eq<{kname},{tname},VX={info.vx},MODE_STEP,periodic>"
-    elif per_launch > 1:
+    elif path == "resident":
+        kernel = f"k_resident2d<{kname},periodic>"
+    elif path == "fused":
         kernel = f"k_update_fused{d}d<{kname},{per_launch},periodic>"
     elif info.vx == 4 and args.storage == "f32":
         kernel = f"k_update_vec_f32x4<{kname},MODE_STEP,periodic>"
@@ -568,10 +576,10 @@ def run_mdf(args):
                   "f16eq": "f16 equilibrium-shifted storage + f32 moments / f32",
                   "bf16eq": "bf16 equilibrium-shifted storage + f32 moments / f32"}[args.storage],
         "data": "synthetic", "config": _config(world, args.storage, d, args.q, args.inplace),
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+        "roofline": {**_bound(path), "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)",
-                     "kernel": kernel, "block": info.block,
+                     "kernel": kernel, "path": path, "block": plan["threads"],
                      "algorithmic_bytes_per_launch": bytes_per_launch,
                      "updates_per_launch": per_launch,
                      "avg_launch_ms": plain_ms * (EPI_EVERY - 1) / launches,
@@ -597,7 +605,8 @@ def run_mdf(args):
 def run_cavities(args):
     """Batched lid-driven cavities (64 seeded boxes, sides from {65, 129, 257,
     513}, Re ~ U[100, 3200], lid 0.1, D2Q5 x 3 FP32): plain-step throughput of
-    the persistent kernel, then every cavity to its residual tolerance."""
+    the path that the autotuner chooses, then every cavity to its residual
+    tolerance."""
     import collections
     import numpy as np
     import torch
@@ -625,10 +634,10 @@ def run_cavities(args):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / (args.steps * 100)
 
-    sched_default = b.schedule()
+    path_default = b.path
     ms_default = timed()
     t0 = time.perf_counter()
-    sched = b.autotune(reps=60)  # untimed: chooses the persistent kernel's launch shape
+    sched = b.autotune(reps=60)  # untimed: the persistent kernel's launch shape, and the faster path
     tune_s = time.perf_counter() - t0
     ms = timed()
     mlups = nodes.sum() / (ms / 1e3) / 1e6
@@ -646,11 +655,12 @@ def run_cavities(args):
         "ms_per_step": ms, "nodes": int(nodes.sum()), "cavities": len(sides),
         "roofline": {"bound": "hbm", "achieved": mlups * 120 / 1e3, "peak": peak, "unit": "GB/s",
                      "frac": mlups * 120 / 1e3 / peak, "peak_source": f"{kind} hbm_gbs",
-                     "kernel": "k_batch_fused<D2Q5,4> and k_batch_resident<D2Q5>, or where the autotuner "
-                               f"measured it faster k_batch_chunk<D2Q5,{sched['threads']},{sched['sched']}>",
+                     "kernel": {"fused": f"k_batch_fused<{b.path['updates']}>", "resident": "k_batch_resident",
+                                "persistent": f"k_batch_chunk<D2Q5,{sched['threads']},{sched['sched']}>"
+                                }[b.path["path"]],
                      "bytes": "120 per node and update, as if every update were a pass of its own (4 updates "
                               "share a pass, boxes on chip make none between checks): above 1 means shared passes"},
-        "schedule": {"tuned": sched, "default": sched_default, "autotune_s": tune_s,
+        "schedule": {"path": b.path, "default_path": path_default, "persistent": sched, "autotune_s": tune_s,
                      "default_mlups": float(nodes.sum() / (ms_default / 1e3) / 1e6)},
         "to_steady": {"tol": 1e-8, "max_steps": args.max_steps, "seconds": run_s,
                       "aggregate_mlups": float((steps * nodes).sum()) / run_s / 1e6 if run_s > 0 else None,
