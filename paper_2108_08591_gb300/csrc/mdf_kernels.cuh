@@ -585,8 +585,17 @@ constexpr int kVecF32x4Regs = 96;
 template <class L, class TS, int VX, int MODE, bool WALLS, bool S2>
 __device__ __forceinline__ void update_vec_body(const DevArgs &A);
 
+// Blocks of kMaxBlock threads per SM that the register budget leaves room for.
+// Three (80 registers, up to 52 B spilled) for four FP16 nodes of D2Q5 per
+// thread: of its own the compiler takes 95 to 100, and the warps that this costs
+// would keep HBM busy.  us per update with 80 / without a budget: 4096^2 147.4 /
+// 159.9, with walls 249.9 / 275.2, 1500^2 24.8 / 26.8, 4096 x 2048 Scheme II 95.1 /
+// 113.6.  D2Q4 (76 to 91 of its own) loses with it: 4096^2 with walls 183.1 / 177.3.
+template <class L, class TS, int VX> constexpr int vec_min_blocks() {
+  return L::D == 2 && L::Q == 5 && VX == 4 && std::is_same<TS, __half>::value ? 3 : 1;
+}
 template <class L, class TS, int VX, int MODE, bool WALLS, bool S2>
-__global__ void __launch_bounds__(kMaxBlock) k_update_vec(const DevArgs A) {
+__global__ void __launch_bounds__(kMaxBlock, vec_min_blocks<L, TS, VX>()) k_update_vec(const DevArgs A) {
   update_vec_body<L, TS, VX, MODE, WALLS, S2>(A);
 }
 template <class L, int MODE, bool WALLS, bool S2>
