@@ -706,7 +706,7 @@ struct mdf_batch_s {
   bool own_limit = false;  // nor with a barrier limit of the caller's own
   bool fuse() const { return can_fuse && !own_shape && !own_limit; }
   BatchItems items[2] = {};  // of launches of two and of four updates
-  BatchItem *item_mem[2] = {};
+  BatchItem *item_mem = nullptr;
   int seats = 0;     // CTAs of the resident kernel's launch (0: the batch does not go that way)
   bool seat_pair = false;
   int seat_threads = 0;
@@ -842,13 +842,12 @@ cudaError_t max_grid(mdf_batch_t b, int threads, int sched, int *grid) {
   return e;
 }
 
-// The item lists of the fused kernel (see BatchItems).  On an error the batch
-// keeps to the persistent kernel.
+// Append the item lists of launches of K updates (see BatchItems) to `all`, each
+// from first[list] on.
 template <int K>
-cudaError_t build_items(mdf_batch_t b) {
+cudaError_t list_items(mdf_batch_t b, std::vector<BatchItem> &all, size_t (&first)[kItemLists]) {
   constexpr int OUT = fuse_out<K>();
   BatchItems &items = b->items[K / 4];
-  BatchItem *&mem = b->item_mem[K / 4];
   constexpr size_t smem = (size_t)kFuseWarps * fuse_slots<K, D2Q5::Q>() * sizeof(float2);
   int per = 0, nmax = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_fused<K, false>, 32 * kFuseWarps, smem);
@@ -860,12 +859,12 @@ cudaError_t build_items(mdf_batch_t b) {
     return n;
   };
   const int rows0 = fuse_rows<K>(nmax, per * kFuseWarps / 4, count);
-  std::vector<BatchItem> all;
-  size_t first[kItemLists] = {};
   for (int l = 0; l < kItemLists; ++l) {
     const int rows = std::max(2, rows0 >> l);
     first[l] = all.size();
-    if (all.size() + (size_t)count(rows) > (1u << 30)) return cudaErrorInvalidValue;
+    const size_t n = (size_t)count(rows);
+    if (all.size() + n > (1u << 30)) return cudaErrorInvalidValue;
+    if (l == 0) all.reserve(all.size() + std::min<size_t>(7 * n, 1u << 20));  // the later lists: 2, 4 times as many
     for (int c = 0; c < b->ncav; ++c) {
       const int N = b->cav[c].N;
       for (int y = 0; y < N; y += rows)
@@ -874,11 +873,22 @@ cudaError_t build_items(mdf_batch_t b) {
     items.n[l] = (int)(all.size() - first[l]);
   }
   items.wave = std::max(items.n[0], 4 * kSMs);
-  e = cudaMalloc(&mem, all.size() * sizeof(BatchItem));
+  return cudaSuccess;
+}
+
+// The item lists of the fused kernel.  On an error the batch keeps to the
+// persistent kernel.
+cudaError_t build_items(mdf_batch_t b) {
+  std::vector<BatchItem> all;
+  size_t first[2][kItemLists];
+  cudaError_t e = list_items<2>(b, all, first[0]);
+  if (e == cudaSuccess) e = list_items<4>(b, all, first[1]);
+  if (e == cudaSuccess) e = cudaMalloc(&b->item_mem, all.size() * sizeof(BatchItem));
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(mem, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(b->item_mem, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // `all` leaves scope
-  for (int l = 0; l < kItemLists; ++l) items.list[l] = mem + first[l];
+  for (int k = 0; k < 2 && e == cudaSuccess; ++k)
+    for (int l = 0; l < kItemLists; ++l) b->items[k].list[l] = b->item_mem + first[k][l];
   return e;
 }
 
@@ -1160,8 +1170,9 @@ mdf_status mdf_batch_create(mdf_batch_t *out, int d, int n, const int *side, con
   // what only the fused and the resident launches need does not fail the
   // batch: without it the next slower path takes its updates
   if (e == cudaSuccess && d == 2 && b->with_rho) {
-    b->can_fuse = build_items<2>(b) == cudaSuccess && build_items<4>(b) == cudaSuccess;
-    if (!b->can_fuse || build_seats(b) != cudaSuccess) cudaGetLastError();
+    if (build_seats(b) != cudaSuccess) cudaGetLastError();
+    b->can_fuse = b->seats || build_items(b) == cudaSuccess;
+    if (!b->can_fuse) cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
@@ -1183,8 +1194,8 @@ void mdf_batch_destroy(mdf_batch_t b) {
   cudaFree(B.f[0]); cudaFree(B.f[1]); cudaFree((void *)B.cav); cudaFree((void *)B.tile_cav);
   cudaFree(B.live); cudaFree(B.n_live); cudaFree(B.usave); cudaFree(B.part); cudaFree(B.badtile);
   cudaFree(B.status); cudaFree(B.steps); cudaFree(B.res); cudaFree(B.bar); cudaFree(B.err);
-  cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem[0]);
-  cudaFree(b->item_mem[1]); cudaFree(b->seat_mem); cudaFree(b->stage);
+  cudaFree(B.prog); cudaFree(B.clock); cudaFree(b->item_mem);
+  cudaFree(b->seat_mem); cudaFree(b->stage);
   cudaFreeHost(b->host_live);
   delete b;
 }

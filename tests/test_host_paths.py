@@ -76,23 +76,23 @@ def test_batch_falls_back_where_its_faster_path_cannot_be_set_up(fake):
     assert all("k_batch_fused" in n for n in _step_kernels(fake, b))
     lib.mdf_batch_destroy(b)
     lib.fake_fail_clusters(0)
-    side, Re = (ctypes.c_int * 2)(65, 97), (ctypes.c_double * 2)(100.0, 100.0)
-    got = []
-    for k in range(1, 40):  # the k-th allocation fails
-        lib.fake_fail_malloc(k)
-        b = ctypes.c_void_p()
-        st = lib.mdf_batch_create(ctypes.byref(b), 2, 2, side, Re, 0.1, None)
-        lib.fake_fail_malloc(0)
-        if st != _lib.OK:
-            assert st == _lib.ENOMEM
-            got.append("refused")
-            continue
-        kinds = _step_kernels(fake, b)
-        got.append(next(n for n in ("chunk", "fused", "resident") if any(n in x for x in kinds)))
-        lib.mdf_batch_destroy(b)
-    # the state's own, the lists of fused launches, the seats on chip, none
-    order = [g for k, g in enumerate(got) if k == 0 or g != got[k - 1]]
-    assert order == ["refused", "chunk", "fused", "resident"], got
+    Re = (ctypes.c_double * 2)(100.0, 100.0)
+    # the state's own allocations, then the seats on chip or the item lists, then none
+    for sides, want in (((65, 97), ["refused", "fused", "resident"]), ((300, 240), ["refused", "chunk", "fused"])):
+        got = []
+        for k in range(1, 40):  # the k-th allocation fails
+            lib.fake_fail_malloc(k)
+            b = ctypes.c_void_p()
+            st = lib.mdf_batch_create(ctypes.byref(b), 2, 2, (ctypes.c_int * 2)(*sides), Re, 0.1, None)
+            lib.fake_fail_malloc(0)
+            if st != _lib.OK:
+                assert st == _lib.ENOMEM
+                got.append("refused")
+                continue
+            kinds = _step_kernels(fake, b)
+            got.append(next(n for n in ("chunk", "fused", "resident") if any(n in x for x in kinds)))
+            lib.mdf_batch_destroy(b)
+        assert [g for k, g in enumerate(got) if k == 0 or g != got[k - 1]] == want, got
 
 
 class _Items(ctypes.Structure):  # of the fused batch kernel: lists, their lengths
