@@ -19,8 +19,12 @@ def link(out):
         _build.build(force=True)
         objs = sorted(glob.glob(os.path.join(_build.BUILD, "mdf_*.o")))
     inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build._nvcc()))), "include")
-    # -Bsymbolic: the library's calls bind to the stand-in also where a real runtime is loaded
-    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", inc,
+    # every other symbol is local: the process may hold the real library as well,
+    # whose templates' statics (kernel handles) the dynamic linker would share
+    script = str(out) + ".map"
+    with open(script, "w") as fh:
+        fh.write("{ global: mdf_*; fake_*; local: *; };\n")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", f"-Wl,--version-script={script}", "-I", inc,
                     os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", str(out)], check=True)
 
 
