@@ -585,14 +585,16 @@ constexpr int kVecF32x4Regs = 96;
 template <class L, class TS, int VX, int MODE, bool WALLS, bool S2>
 __device__ __forceinline__ void update_vec_body(const DevArgs &A);
 
-// Blocks of kMaxBlock threads per SM that the register budget leaves room for.
-// Three (80 registers, up to 52 B spilled) for four FP16 nodes of D2Q5 per
-// thread: of its own the compiler takes 95 to 100, and the warps that this costs
-// would keep HBM busy.  us per update with 80 / without a budget: 4096^2 147.4 /
-// 159.9, with walls 249.9 / 275.2, 1500^2 24.8 / 26.8, 4096 x 2048 Scheme II 95.1 /
-// 113.6.  D2Q4 (76 to 91 of its own) loses with it: 4096^2 with walls 183.1 / 177.3.
+// Blocks of kMaxBlock threads per SM that the register budget leaves room for; 0:
+// no budget (1 is one, with other code: BF16 at 4096^2 191.7 us per update with 1,
+// 151.0 with 0).  Three (80 registers, up to 52 B spilled) for four 16-bit nodes of
+// D2Q5 per thread: of its own the compiler takes up to 108, and the warps that
+// this costs would keep HBM busy.  us per update with 80 / without a budget: FP16
+// 4096^2 147.4 / 159.9, with walls 249.9 / 275.2, 4096 x 2048 Scheme II 95.1 / 113.6;
+// BF16 4096^2 151.9 / 151.0, with walls 227.6 / 287.9.  D2Q4 (76 to 91 of its own)
+// loses with it: FP16 4096^2 with walls 183.1 / 177.3.
 template <class L, class TS, int VX> constexpr int vec_min_blocks() {
-  return L::D == 2 && L::Q == 5 && VX == 4 && std::is_same<TS, __half>::value ? 3 : 1;
+  return L::D == 2 && L::Q == 5 && VX == 4 && sizeof(TS) == 2 ? 3 : 0;
 }
 template <class L, class TS, int VX, int MODE, bool WALLS, bool S2>
 __global__ void __launch_bounds__(kMaxBlock, vec_min_blocks<L, TS, VX>()) k_update_vec(const DevArgs A) {
